@@ -15,6 +15,27 @@
 
 using namespace rqa;
 
+namespace rqa {
+
+Split split_cells(uint64_t cells, int nb, int sm_count)
+{
+    const uint64_t per_unit = cells / ((uint64_t)sm_count * 2 * 6);
+    const uint64_t blocks = per_unit / ((uint64_t)nb * DB * ROW_BLOCK);
+    return Split{nb, ROW_BLOCK * (int)std::min<uint64_t>(std::max<uint64_t>(blocks, 8), 585)};
+}
+
+int64_t units_of_series(int64_t ne, const Split &sp, bool vert)
+{
+    int64_t n = 0;
+    for (int64_t r = 0; r < ne; r += sp.rc) {
+        const int64_t bands = vert ? (ne + DB - 1) / DB : (ne - 1 - r + DB - 1) / DB;
+        n += (bands + sp.nb - 1) / sp.nb;
+    }
+    return n;
+}
+
+}  // namespace rqa
+
 namespace {
 
 struct DevBuf {
@@ -52,7 +73,6 @@ struct rqa_ctx {
     cudaStream_t stream = nullptr;
     int schedule = RQA_SCHED_BATCHED;
     int select = RQA_SELECT_AUTO;
-    int band = 16;          // diagonals per band of the counting rounds
     int line_tile = 0;      // diagonals per register window of the line pass (0 = default)
     int unit_bands = 0;     // bands per line-pass work unit (0 = planned)
     int line_ctas = 0;      // persistent line-pass CTAs per SM (0 = all that fit)
@@ -65,7 +85,7 @@ struct rqa_ctx {
 
     // scratch (grow-only)
     DevBuf arena;      // uploaded plan: series, targets, items, lmin, hist offsets
-    DevBuf prefix, level, rank, below, tab_sub, tab_mid, tab_fin1, tab_fin2, tab_hash, ngroups, hist, krange,
+    DevBuf prefix, level, rank, below, tab_sub, tab_mid, tab_hash, ngroups, hist, krange,
         redo;
     DevBuf queue, status;
     DevBuf eps_tmp, le_tmp, lt_tmp, count, lmax, hshort;
@@ -111,10 +131,10 @@ struct Plan {
     int64_t total = 0;          // values in the batch buffer
     std::vector<SeriesDev> sd;
     std::vector<uint64_t> T;    // S*K (empty if no targets)
-    std::vector<Item> items_lpt;             // whole batch, largest first
-    std::vector<Item> items_ser;             // grouped by series
-    std::vector<int> ser_begin;              // S+1 into items_ser
     std::vector<int32_t> order;              // series by size, largest first
+    Split split{};                           // cell-walk units of the batch ...
+    std::vector<Split> split1;               // ... and of each series alone
+    std::vector<int64_t> cprefix, cprefix1;  // their unit-count prefixes, as uprefix / uprefix1
     std::vector<int64_t> uprefix;            // S+1 unit-count prefix along order
     int32_t chunk = 1;                       // bands per line-pass unit (batched)
     int32_t line_tile = LINE_TILE_DEFAULT;   // diagonals per register window of the line pass
@@ -127,10 +147,8 @@ struct Plan {
     // device pointers into the arena after upload
     SeriesDev *d_sd = nullptr;
     uint64_t *d_T = nullptr;
-    Item *d_lpt = nullptr;
-    Item *d_ser = nullptr;
     int32_t *d_order = nullptr, *d_ident = nullptr;
-    int64_t *d_uprefix = nullptr, *d_uprefix1 = nullptr;
+    int64_t *d_uprefix = nullptr, *d_uprefix1 = nullptr, *d_cprefix = nullptr, *d_cprefix1 = nullptr;
     int32_t *d_lmin = nullptr;
     int64_t *d_hoff = nullptr;
     uint8_t *d_dom = nullptr;
@@ -158,34 +176,6 @@ void mark(rqa_ctx *c, int i)
         // of the graph, so replays record the phase boundaries too
         cudaEventRecordWithFlags(c->ev[i], c->stream, cudaEventRecordExternal);
         if (i == 6) c->ev_recorded = true;
-    }
-}
-
-uint64_t band_cost(int64_t ne, int64_t d_lo, int64_t d_hi)
-{
-    // sum_{delta = d_lo}^{d_hi - 1} (ne - delta)
-    const int64_t n = d_hi - d_lo;
-    return (uint64_t)(n * ne - (d_lo + d_hi - 1) * n / 2);
-}
-
-void build_items(const SeriesDev &s, int sidx, int band, uint64_t target, int min_bands,
-                 std::vector<Item> &out, std::vector<uint64_t> *costs)
-{
-    Item cur{sidx, 0, 0, 0};
-    uint64_t acc = 0;
-    for (int b = 0; b < s.nbands; ++b) {
-        const int64_t d_lo = 1 + (int64_t)b * band;
-        const int64_t d_hi = std::min<int64_t>(d_lo + band, s.ne);
-        acc += band_cost(s.ne, d_lo, d_hi);
-        cur.b_hi = b + 1;
-        const bool enough = acc >= target && cur.b_hi - cur.b_lo >= min_bands &&
-                            s.nbands - cur.b_hi >= min_bands;
-        if (enough || acc >= ((uint64_t)1 << 30) || b + 1 == s.nbands) {
-            out.push_back(cur);
-            if (costs) costs->push_back(acc);
-            cur.b_lo = b + 1;
-            acc = 0;
-        }
     }
 }
 
@@ -245,8 +235,6 @@ int make_plan(rqa_ctx *c, const rqa_batch *b, const int32_t *rr_num, int32_t rr_
         d.tau = b->tau[s];
         d.ne = d.n - (d.m - 1) * d.tau;
         d.P = (uint64_t)d.ne * (uint64_t)(d.ne - 1) / 2;
-        d.nbands = (d.ne - 1 + c->band - 1) / c->band;
-        d.pad = 0;
         uniform &= (d.m == m0);
         uniform_tau &= (d.tau == t0);
         total_cells += d.P;
@@ -282,27 +270,11 @@ int make_plan(rqa_ctx *c, const rqa_batch *b, const int32_t *rr_num, int32_t rr_
                     return RQA_ERR_INVALID_ARG;
         }
     }
-    // CTA work items (counting rounds): runs of consecutive bands of one
-    // series, about three per persistent CTA and at least four bands per warp,
-    // sorted largest first.  Per series: the same rule within the series.
-    const uint64_t ctas = (uint64_t)c->sm_count * 2;
-    const uint64_t cap = (uint64_t)1 << 30;  // keeps 32-bit shared counters exact
-    uint64_t tgt = std::max<uint64_t>(total_cells / (ctas * 3), 1);
-    tgt = std::min(tgt, cap);
-    std::vector<Item> items;
-    std::vector<uint64_t> costs;
-    for (int s = 0; s < S; ++s) build_items(pl.sd[s], s, c->band, tgt, ITEM_MIN_BANDS, items, &costs);
-    std::vector<size_t> idx(items.size());
-    for (size_t i = 0; i < idx.size(); ++i) idx[i] = i;
-    std::stable_sort(idx.begin(), idx.end(), [&](size_t x, size_t y) { return costs[x] > costs[y]; });
-    pl.items_lpt.resize(items.size());
-    for (size_t i = 0; i < idx.size(); ++i) pl.items_lpt[i] = items[idx[i]];
-    pl.ser_begin.assign(S + 1, 0);
-    for (int s = 0; s < S; ++s) {
-        uint64_t t = std::min(std::max<uint64_t>(pl.sd[s].P / (ctas * 3), 1), cap);
-        build_items(pl.sd[s], s, c->band, t, ITEM_MIN_BANDS, pl.items_ser, nullptr);
-        pl.ser_begin[s + 1] = (int)pl.items_ser.size();
-    }
+    // units of the cell walk (counting rounds, grid search)
+    pl.split = split_cells(total_cells, COUNT_NB, c->sm_count);
+    pl.split1.resize(S);
+    pl.cprefix.assign(S + 1, 0);
+    pl.cprefix1.assign(2 * (size_t)S, 0);
     // warp work units (line pass): runs of `chunk` bands of LINE_BAND
     // diagonals, series largest first; about eight units per warp so the tail
     // stays short while each unit's histogram flush is spread over many cells.
@@ -327,8 +299,10 @@ int make_plan(rqa_ctx *c, const rqa_batch *b, const int32_t *rr_num, int32_t rr_
     std::stable_sort(pl.order.begin(), pl.order.end(),
                      [&](int x, int y) { return pl.sd[x].P > pl.sd[y].P; });
     pl.uprefix.assign(S + 1, 0);
-    for (int i = 0; i < S; ++i)
+    for (int i = 0; i < S; ++i) {
         pl.uprefix[i + 1] = pl.uprefix[i] + (nbl(pl.order[i]) + pl.chunk - 1) / pl.chunk;
+        pl.cprefix[i + 1] = pl.cprefix[i] + units_of_series(pl.sd[pl.order[i]].ne, pl.split, false);
+    }
     pl.ident.resize(S);
     pl.uprefix1.resize(2 * (size_t)S);
     pl.chunk1.resize(S);
@@ -337,6 +311,8 @@ int make_plan(rqa_ctx *c, const rqa_batch *b, const int32_t *rr_num, int32_t rr_
         pl.chunk1[s] = chunk_for(nbl(s));
         pl.uprefix1[2 * s] = 0;
         pl.uprefix1[2 * s + 1] = (nbl(s) + pl.chunk1[s] - 1) / pl.chunk1[s];
+        pl.split1[s] = split_cells(pl.sd[s].P, COUNT_NB, c->sm_count);
+        pl.cprefix1[2 * s + 1] = units_of_series(pl.sd[s].ne, pl.split1[s], false);
     }
     return RQA_OK;
 }
@@ -346,9 +322,9 @@ int upload_plan(rqa_ctx *c, Plan &pl, const int32_t *lmin, int n_lmin, const int
 {
     const size_t o_sd = 0;
     const size_t o_T = align16(o_sd + pl.sd.size() * sizeof(SeriesDev));
-    const size_t o_lpt = align16(o_T + pl.T.size() * sizeof(uint64_t));
-    const size_t o_ser = align16(o_lpt + pl.items_lpt.size() * sizeof(Item));
-    const size_t o_order = align16(o_ser + pl.items_ser.size() * sizeof(Item));
+    const size_t o_cpre = align16(o_T + pl.T.size() * sizeof(uint64_t));
+    const size_t o_cpre1 = align16(o_cpre + pl.cprefix.size() * sizeof(int64_t));
+    const size_t o_order = align16(o_cpre1 + pl.cprefix1.size() * sizeof(int64_t));
     const size_t o_upre = align16(o_order + pl.order.size() * sizeof(int32_t));
     const size_t o_ident = align16(o_upre + pl.uprefix.size() * sizeof(int64_t));
     const size_t o_upre1 = align16(o_ident + pl.ident.size() * sizeof(int32_t));
@@ -376,8 +352,8 @@ int upload_plan(rqa_ctx *c, Plan &pl, const int32_t *lmin, int n_lmin, const int
     char *h = static_cast<char *>(c->h_stage);
     std::memcpy(h + o_sd, pl.sd.data(), pl.sd.size() * sizeof(SeriesDev));
     if (!pl.T.empty()) std::memcpy(h + o_T, pl.T.data(), pl.T.size() * sizeof(uint64_t));
-    std::memcpy(h + o_lpt, pl.items_lpt.data(), pl.items_lpt.size() * sizeof(Item));
-    std::memcpy(h + o_ser, pl.items_ser.data(), pl.items_ser.size() * sizeof(Item));
+    std::memcpy(h + o_cpre, pl.cprefix.data(), pl.cprefix.size() * sizeof(int64_t));
+    std::memcpy(h + o_cpre1, pl.cprefix1.data(), pl.cprefix1.size() * sizeof(int64_t));
     std::memcpy(h + o_order, pl.order.data(), pl.order.size() * sizeof(int32_t));
     std::memcpy(h + o_upre, pl.uprefix.data(), pl.uprefix.size() * sizeof(int64_t));
     std::memcpy(h + o_ident, pl.ident.data(), pl.ident.size() * sizeof(int32_t));
@@ -391,8 +367,8 @@ int upload_plan(rqa_ctx *c, Plan &pl, const int32_t *lmin, int n_lmin, const int
     c->stage_pending = true;
     pl.d_sd = reinterpret_cast<SeriesDev *>(d + o_sd);
     pl.d_T = reinterpret_cast<uint64_t *>(d + o_T);
-    pl.d_lpt = reinterpret_cast<Item *>(d + o_lpt);
-    pl.d_ser = reinterpret_cast<Item *>(d + o_ser);
+    pl.d_cprefix = reinterpret_cast<int64_t *>(d + o_cpre);
+    pl.d_cprefix1 = reinterpret_cast<int64_t *>(d + o_cpre1);
     pl.d_order = reinterpret_cast<int32_t *>(d + o_order);
     pl.d_uprefix = reinterpret_cast<int64_t *>(d + o_upre);
     pl.d_ident = reinterpret_cast<int32_t *>(d + o_ident);
@@ -415,8 +391,6 @@ int ensure_select_bufs(rqa_ctx *c, int S, int K)
     if ((rc = ensure(c->below, sk * 8))) return rc;
     if ((rc = ensure(c->tab_sub, (size_t)S * NCOARSE))) return rc;
     if ((rc = ensure(c->tab_mid, (size_t)S * NCOARSE))) return rc;
-    if ((rc = ensure(c->tab_fin1, (size_t)S * NCOARSE))) return rc;
-    if ((rc = ensure(c->tab_fin2, (size_t)S * KMAX * NFINE))) return rc;
     if ((rc = ensure(c->tab_hash, (size_t)S * NHASH * 4))) return rc;
     if ((rc = ensure(c->ngroups, (size_t)S * 4 * sizeof(int32_t)))) return rc;
     if ((rc = ensure(c->krange, (size_t)S * 2 * sizeof(uint32_t)))) return rc;
@@ -438,9 +412,6 @@ SelBufs sel_bufs(rqa_ctx *c, const Plan &pl)
     sb.below = P<uint64_t>(c->below);
     sb.tab_sub = P<int8_t>(c->tab_sub);
     sb.tab_mid = P<int8_t>(c->tab_mid);
-    sb.tab_fin1 = P<int8_t>(c->tab_fin1);
-    sb.tab_fin2 = P<int8_t>(c->tab_fin2);
-    sb.fin2_stride = (int64_t)KMAX * NFINE;
     int32_t *ng = P<int32_t>(c->ngroups);
     sb.n_sub = ng;
     sb.n_mid = ng + pl.S;
@@ -470,20 +441,30 @@ int reset_queue(rqa_ctx *c, int n, unsigned **q)
     return RQA_OK;
 }
 
-// Exact selection for series [s0, s0+ns) using the given item list: three
-// counting rounds, the first one split by the learned bracket if asked.
-int run_select(rqa_ctx *c, const Plan &pl, const SelBufs &sb, const Item *items, int n_items,
-               int s0, int ns, unsigned *&q, float *eps, uint64_t *le, uint64_t *lt, bool bracket)
+// The cell-walk units of the whole batch, or of series s alone (s >= 0).
+CellArgs cell_args(rqa_ctx *c, const Plan &pl, int s)
 {
-    const int K = pl.K;
-    const int grid = persistent_grid(c, (size_t)n_items);
     CellArgs a{};
     a.y = pl.y;
     a.series = pl.d_sd;
-    a.items = items;
-    a.n_items = n_items;
-    a.band = c->band;
     a.status = P<int>(c->status);
+    const Split sp = s < 0 ? pl.split : pl.split1[s];
+    a.nb = sp.nb;
+    a.rc = sp.rc;
+    a.order = s < 0 ? pl.d_order : pl.d_ident + s;
+    a.uprefix = s < 0 ? pl.d_cprefix : pl.d_cprefix1 + 2 * (size_t)s;
+    a.n_pos = s < 0 ? pl.S : 1;
+    a.n_units = s < 0 ? pl.cprefix[pl.S] : pl.cprefix1[2 * (size_t)s + 1];
+    return a;
+}
+
+// Exact selection for series [s0, s0+ns) over the given work units: three
+// counting rounds, the first one split by the learned bracket if asked.
+int run_select(rqa_ctx *c, const Plan &pl, const SelBufs &sb, const CellArgs &cells, int s0, int ns, unsigned *&q, float *eps, uint64_t *le, uint64_t *lt, bool bracket)
+{
+    const int K = pl.K;
+    CellArgs a = cells;
+    const int grid = persistent_grid(c, (size_t)a.n_units);
     const size_t hbytes = (size_t)ns * sb.hstride * 8;
     uint64_t *hbase = sb.hist + (int64_t)s0 * sb.hstride;
     if (bracket) {
@@ -519,8 +500,7 @@ int run_select(rqa_ctx *c, const Plan &pl, const SelBufs &sb, const Item *items,
             if (int rc = launched(c, launch_count(rounds[r], a, sb, K, grid, pl.mt, c->stream)))
                 return rc;
         }
-        if (int rc = launched(c, launch_select(rounds[r], sb, pl.d_sd, s0, ns, K, eps, le, lt,
-                                               P<int>(c->status), c->stream)))
+        if (int rc = launched(c, launch_select(rounds[r], sb, s0, ns, K, eps, le, lt, P<int>(c->status), c->stream)))
             return rc;
         if (r == 0)
             if (int rc = launched(c, launch_bracket_stats(sb.level + (int64_t)s0 * K, pl.d_dom + s0, ns, K,
@@ -570,15 +550,13 @@ int select_all(rqa_ctx *c, const rqa_batch *b, Plan &pl, float *eps, uint64_t *l
     if (c->schedule == RQA_SCHED_PER_SERIES) {
         if (int rc = reset_queue(c, select_launches(pl.K) * pl.S, &q)) return rc;
         for (int s = 0; s < pl.S; ++s) {
-            const int ib = pl.ser_begin[s], ie = pl.ser_begin[s + 1];
-            if (int rc = run_select(c, pl, sb, pl.d_ser + ib, ie - ib, s, 1, q, eps, le, lt, bracket))
+            if (int rc = run_select(c, pl, sb, cell_args(c, pl, s), s, 1, q, eps, le, lt, bracket))
                 return rc;
         }
         return RQA_OK;
     }
     if (int rc = reset_queue(c, select_launches(pl.K), &q)) return rc;
-    return run_select(c, pl, sb, pl.d_lpt, (int)pl.items_lpt.size(), 0, pl.S, q, eps, le, lt,
-                      bracket);
+    return run_select(c, pl, sb, cell_args(c, pl, -1), 0, pl.S, q, eps, le, lt, bracket);
 }
 
 int ensure_line_bufs(rqa_ctx *c, int S, int K)
@@ -611,7 +589,6 @@ int run_lines(rqa_ctx *c, const Plan &pl, const float *eps, uint64_t *hist, cons
     CellArgs a{};
     a.y = pl.y;
     a.series = pl.d_sd;
-    a.band = c->band;
     a.line_tile = pl.line_tile;
     a.line_ctas = c->line_ctas;
     a.line_stage = c->line_stage;
@@ -798,7 +775,6 @@ int rqa_create(rqa_ctx **out, const rqa_config *cfg)
     c->stream = static_cast<cudaStream_t>(cfg->stream);
     c->schedule = cfg->schedule;
     c->select = cfg->select;
-    c->band = BAND;
     c->line_tile = cfg->tile;
     c->tile_fixed = cfg->tile != 0;
     c->graphs = !(cfg->flags & RQA_FLAG_NO_GRAPHS);
@@ -827,7 +803,7 @@ void rqa_destroy(rqa_ctx *c)
     cudaSetDevice(c->device);
     cudaStreamSynchronize(c->stream);
     DevBuf *bufs[] = {&c->arena, &c->prefix, &c->level, &c->rank, &c->below, &c->tab_sub,
-                      &c->tab_mid, &c->tab_fin1, &c->tab_fin2, &c->tab_hash, &c->ngroups, &c->hist,
+                      &c->tab_mid, &c->tab_hash, &c->ngroups, &c->hist,
                       &c->krange, &c->meas, &c->grid_thr, &c->grid_hist, &c->grid_rr,
                       &c->redo,
                       &c->queue,
@@ -1144,18 +1120,12 @@ int rqa_eps_approx(rqa_ctx *c, const rqa_batch *b, const int32_t *rr_num, int32_
         return rc;
     unsigned *q = nullptr;
     if (int rc = reset_queue(c, 1, &q)) return rc;
-    CellArgs a{};
-    a.y = pl.y;
-    a.series = pl.d_sd;
-    a.items = pl.d_lpt;
-    a.n_items = (int)pl.items_lpt.size();
-    a.band = c->band;
+    CellArgs a = cell_args(c, pl, -1);
     a.queue = q;
-    a.status = P<int>(c->status);
     c->launches += 2;  // grid and selection kernels
     return launched(c, launch_grid_select(a, pl.S, n_thr, P<float>(c->grid_thr), P<uint64_t>(c->grid_hist),
                                           P<int32_t>(c->grid_rr), rr_den, K, eps_out, rr_out, count_out,
-                                          persistent_grid(c, (size_t)a.n_items), pl.mt, c->stream));
+                                          persistent_grid(c, (size_t)a.n_units), pl.mt, c->stream));
 }
 
 int rqa_set_timing(rqa_ctx *c, int enable)

@@ -7,7 +7,7 @@
 // so that any implementation reproduces it: thr_i = i * ((max - min) / n),
 // i = 1..n.  A cell is recurrent at thr_i iff d <= thr_i (upper triangle).
 #include <cstdint>
-#include "rqa_common.cuh"
+#include "dense.cuh"
 
 namespace rqa {
 
@@ -47,68 +47,113 @@ k_grid_thr(const float *__restrict__ y, const SeriesDev *__restrict__ series, in
 }
 
 // Counting pass: for every cell the number of grid thresholds below its
-// distance, r = #{i : thr_i < d} in 0..n (a binary search over the grid keys
-// in shared memory), histogrammed per series: bin r holds the cells first
-// recurrent at thr_{r+1}.  Persistent CTAs over the band items of the exact
-// selection.
-template <int M, int TAU>
+// distance, r = #{i : thr_i < d} in 0..n, histogrammed per series: bin r holds
+// the cells first recurrent at thr_{r+1}.
+//
+// The grid is uniform, so r follows from one multiplication: with rho the
+// integer nearest to d / scale, every thr_i with i < rho lies below d and every
+// one with i > rho above it (the rounding of 1 / scale, of the product and of
+// thr_i moves d / scale by less than n 2^-22, far from one half), so
+// r = rho - 1 + [thr_rho < d] (0 for rho = 0): one multiply-add into the
+// integers of [2^23, 2^24), one DPX clamp, one lookup, one compare and one
+// shared reduction per cell.  A binary search took log2(n) dependent lookups
+// (grid-400's counting pass: 5.5 ms).  Grids whose step or its reciprocal
+// could be subnormal or overflow are searched (UNI false).
+template <class Src>
 __global__ void __launch_bounds__(GT)
 k_count_grid(CellArgs a, const float *__restrict__ thr, int n_thr, uint64_t *hist)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    uint32_t *h = reinterpret_cast<uint32_t *>(smem);   // n_thr + 1 bins
-    uint32_t *tk = h + n_thr + 1;                         // grid keys, padded to a power of two
-    __shared__ int slot, next_band;
-    const int lane = threadIdx.x & 31;
-    int npow = 1;
-    while (npow < n_thr) npow <<= 1;
-    for (;;) {
-        const int it = next_item(a.queue, a.n_items, &slot);
-        if (it < 0) break;
-        const Item item = a.items[it];
-        const SeriesDev sd = a.series[item.s];
-        for (int x = threadIdx.x; x <= n_thr; x += GT) h[x] = 0;
-        for (int x = threadIdx.x; x < npow; x += GT)
-            tk[x] = x < n_thr ? __float_as_uint(thr[(int64_t)item.s * n_thr + x]) : 0xffffffffu;
-        if (threadIdx.x == 0) next_band = item.b_lo;
+    __shared__ Unit unit;
+    __shared__ int next_band;
+    __shared__ uint32_t sink[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t *win = reinterpret_cast<uint32_t *>(smem) + warp * WIN_WORDS;
+    uint32_t *h = reinterpret_cast<uint32_t *>(smem) + (GT / 32) * WIN_WORDS;  // bin r + 1; bin 0 belongs to r = 0
+    uint32_t *tk = h + n_thr + 2;  // keys of thr_0 = 0, thr_1, .., thr_n
+    for (int x = threadIdx.x; x < n_thr + 2; x += GT) h[x] = 0;
+    int cur = -1;
+    uint64_t acc = 0;
+    float inv = 0.f;
+    bool uni = false;
+    auto flush = [&]() {
+        if (cur < 0) return;
         __syncthreads();
-        const float *ys = a.y + sd.off;
-        for (;;) {
-            int b = 0;
-            if (lane == 0) b = atomicAdd(&next_band, 1);
-            b = __shfl_sync(FULL, b, 0);
-            if (b >= item.b_hi) break;
-            int d_lo, d_hi;
-            band_range(b, BAND, sd.ne, d_lo, d_hi);
-            const int rows = sd.ne - d_lo;
-            for (int i0 = 0; i0 < rows; i0 += 32) {
-                const int i = i0 + lane;
-                BandTile<M, TAU, BAND> tile;
-                tile.load(ys, sd.n, i, d_lo, rows, sd.tau, sd.m);
-#pragma unroll 4
-                for (int j = 0; j < BAND; ++j) {
-                    const int dl = d_lo + j;
-                    const bool valid = i < sd.ne - dl;
-                    if (!(TAU > 0 || valid)) continue;
-                    const uint32_t key = __float_as_uint(tile.dist(ys, j, i, dl, sd.tau, sd.m));
-                    int r = 0;  // grid keys below key (non-negative floats order as their bits)
-                    for (int step = npow >> 1; step > 0; step >>= 1)
-                        if (tk[r + step - 1] < key) r += step;
-                    if (r < npow && r < n_thr && tk[r] < key) ++r;
-                    if (valid) atomicAdd(&h[min(r, n_thr)], 1u);
-                }
+        unsigned long long *gh = reinterpret_cast<unsigned long long *>(hist + (int64_t)cur * (n_thr + 1));
+        for (int x = threadIdx.x; x < n_thr + 2; x += GT)
+            if (h[x]) {
+                atomicAdd(gh + (x ? x - 1 : 0), (unsigned long long)h[x]);
+                h[x] = 0;
+            }
+        acc = 0;
+        __syncthreads();
+    };
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            const unsigned t = atomicAdd(a.queue, 1u);
+            if ((int64_t)t < a.n_units) {
+                unit = unit_of<false>(a, (int64_t)t);
+                next_band = unit.b_lo;
+            } else {
+                unit.s = -1;
             }
         }
         __syncthreads();
-        uint64_t *gh = hist + (int64_t)item.s * (n_thr + 1);
-        for (int x = threadIdx.x; x <= n_thr; x += GT)
-            if (h[x]) atomicAdd(reinterpret_cast<unsigned long long *>(gh + x), (unsigned long long)h[x]);
-        __syncthreads();
+        const Unit w = unit;
+        if (w.s < 0) break;
+        const SeriesDev sd = a.series[w.s];
+        if (w.s != cur) {
+            flush();
+            cur = w.s;
+            const float *tg = thr + (int64_t)cur * n_thr;
+            for (int x = threadIdx.x; x <= n_thr; x += GT) tk[x] = x ? __float_as_uint(tg[x - 1]) : 0u;
+            const float scale = tg[0];  // 1 * ((max - min) / n)
+            uni = scale == 0.f || (scale >= 0x1p-100f && scale <= 0x1p100f);
+            inv = scale > 0.f ? 1.f / scale : 0.f;  // a constant series: every distance is 0
+            __syncthreads();
+        }
+        const uint64_t cells = (uint64_t)(w.b_hi - w.b_lo) * DB * (uint64_t)(w.r_hi - w.r_lo);
+        if (acc + cells > 0xffffffffull) flush();
+        acc += cells;
+        const uint32_t sink_a = static_cast<uint32_t>(__cvta_generic_to_shared(&sink[lane]));
+        const uint32_t h_a = static_cast<uint32_t>(__cvta_generic_to_shared(h));
+        Src src;
+        src.init(a.y + sd.off, sd, lane, win);
+        auto bands = [&](auto &&f) {
+            for (;;) {
+                int b = 0;
+                if (lane == 0) b = atomicAdd(&next_band, 1);
+                b = __shfl_sync(FULL, b, 0);
+                if (b >= w.b_hi) break;
+                walk_keys(src, sd.ne, 1 + b * DB, w.r_lo, w.r_hi, lane, f);
+            }
+        };
+        if (uni) {
+            bands([&](uint32_t key, bool valid) {
+                const float f = fmaf(__uint_as_float(key), inv, 8388608.f);
+                const int rho = __viaddmin_s32_relu((int)__float_as_uint(f), -0x4B000000, n_thr);
+                const uint32_t r1 = (uint32_t)rho + (tk[rho] < key ? 1u : 0u);
+                red_shared(valid ? h_a + (r1 << 2) : sink_a);
+            });
+        } else {
+            bands([&](uint32_t key, bool valid) {
+                int lo = 0, hi = n_thr;  // grid keys below key (ascending)
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (tk[mid + 1] < key) lo = mid + 1;
+                    else hi = mid;
+                }
+                red_shared(valid ? h_a + ((uint32_t)(lo + 1) << 2) : sink_a);
+            });
+        }
     }
+    flush();
 }
 
 // Per series: grid counts C_j = #{d <= thr_j} (prefix sums of the bins) and,
-// for each target, the first j minimising |C_j den - rr_num P| (exact).
+// for each target, the first j minimising |C_j den - rr_num P| (exact).  One
+// warp scans the bins, then a warp per target searches.
 __global__ void __launch_bounds__(GT)
 k_select_grid(const uint64_t *hist, const float *thr, const SeriesDev *series, int n_thr,
               const int32_t *rr_num, int rr_den, int K, float *eps_out, double *rr_out,
@@ -116,22 +161,31 @@ k_select_grid(const uint64_t *hist, const float *thr, const SeriesDev *series, i
 {
     extern __shared__ __align__(16) unsigned char smem[];
     uint64_t *c = reinterpret_cast<uint64_t *>(smem);  // n_thr prefix counts
-    const int s = blockIdx.x;
+    const int s = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint64_t *h = hist + (int64_t)s * (n_thr + 1);
-    if (threadIdx.x == 0) {
-        uint64_t acc = 0;
-        for (int j = 0; j < n_thr; ++j) {
-            acc += h[j];
-            c[j] = acc;
+    for (int x = threadIdx.x; x < n_thr; x += GT) c[x] = h[x];
+    __syncthreads();
+    if (warp == 0) {
+        uint64_t base = 0;
+        for (int x0 = 0; x0 < n_thr; x0 += 32) {
+            uint64_t v = x0 + lane < n_thr ? c[x0 + lane] : 0;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint64_t u = __shfl_up_sync(FULL, v, o);
+                if (lane >= o) v += u;
+            }
+            v += base;
+            if (x0 + lane < n_thr) c[x0 + lane] = v;
+            base = __shfl_sync(FULL, v, 31);
         }
     }
     __syncthreads();
     const uint64_t P = series[s].P;
-    for (int k = threadIdx.x; k < K; k += GT) {
+    for (int k = warp; k < K; k += GT / 32) {
         const unsigned __int128 target = (unsigned __int128)(uint64_t)rr_num[k] * P;
-        int best = 0;
+        int best = 0x7fffffff;
         unsigned __int128 best_err = ~(unsigned __int128)0;
-        for (int j = 0; j < n_thr; ++j) {
+        for (int j = lane; j < n_thr; j += 32) {
             const unsigned __int128 v = (unsigned __int128)c[j] * (unsigned)rr_den;
             const unsigned __int128 err = v > target ? v - target : target - v;
             if (err < best_err) {
@@ -139,10 +193,23 @@ k_select_grid(const uint64_t *hist, const float *thr, const SeriesDev *series, i
                 best = j;
             }
         }
-        const int64_t o = (int64_t)s * K + k;
-        eps_out[o] = thr[(int64_t)s * n_thr + best];
-        if (rr_out) rr_out[o] = (double)c[best] / (double)P;
-        if (count_out) count_out[o] = c[best];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {  // the smallest error, then the smallest j
+            const uint64_t hi = __shfl_xor_sync(FULL, (uint64_t)(best_err >> 64), o);
+            const uint64_t lo = __shfl_xor_sync(FULL, (uint64_t)best_err, o);
+            const int bj = __shfl_xor_sync(FULL, best, o);
+            const unsigned __int128 err = ((unsigned __int128)hi << 64) | lo;
+            if (err < best_err || (err == best_err && bj < best)) {
+                best_err = err;
+                best = bj;
+            }
+        }
+        if (lane == 0) {
+            const int64_t o = (int64_t)s * K + k;
+            eps_out[o] = thr[(int64_t)s * n_thr + best];
+            if (rr_out) rr_out[o] = (double)c[best] / (double)P;
+            if (count_out) count_out[o] = c[best];
+        }
     }
 }
 
@@ -151,24 +218,20 @@ cudaError_t launch_grid_select(const CellArgs &a, int S, int n_thr, float *thr, 
                                double *rr_out, uint64_t *count_out, int grid, int embed,
                                cudaStream_t st)
 {
-    if (!a.y || !a.series || !a.items || !a.queue || a.n_items < 1 || a.band != BAND || S < 1 ||
-        n_thr < 1 || n_thr > 1024 || !thr || !hist || !rr_num_dev || K < 1 || K > KMAX || !eps_out ||
+    if (!a.y || !a.series || !a.order || !a.uprefix || !a.queue || a.n_units < 1 || a.n_pos < 1 ||
+        a.nb < 1 || a.rc < RB || a.rc % RB || S < 1 || n_thr < 1 || n_thr > 1024 || !thr || !hist || !rr_num_dev || K < 1 || K > KMAX || !eps_out ||
         grid < 1)
         return cudaErrorInvalidValue;
     k_grid_thr<<<S, GT, 0, st>>>(a.y, a.series, n_thr, thr);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int smem = (n_thr + 1 + 1024) * 4;
+    const int smem = ((GT / 32) * WIN_WORDS + 2 * n_thr + 3) * 4;
     void (*kern)(CellArgs, const float *, int, uint64_t *);
     switch (embed) {
-    case E_M1T1: kern = k_count_grid<1, 1>; break;
-    case E_M3T1: kern = k_count_grid<3, 1>; break;
-    case E_M3T3: kern = k_count_grid<3, 3>; break;
-    case E_M1: kern = k_count_grid<1, 0>; break;
-    case E_M2: kern = k_count_grid<2, 0>; break;
-    case E_M3: kern = k_count_grid<3, 0>; break;
-    case E_M4: kern = k_count_grid<4, 0>; break;
-    default: kern = k_count_grid<0, 0>; break;
+    case E_M1T1: kern = k_count_grid<DiagSrc<1, 1>>; break;
+    case E_M3T1: kern = k_count_grid<DiagSrc<3, 1>>; break;
+    case E_M3T3: kern = k_count_grid<DiagSrc<3, 3>>; break;
+    default: kern = k_count_grid<GenSrc>; break;
     }
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
         return e;

@@ -1,0 +1,265 @@
+// The cell walk shared by the counting rounds, the grid search and the line
+// passes: a warp owns a band of 128 consecutive diagonals (or columns) of the
+// never-materialised distance matrix and walks down it in blocks of 28 rows;
+// lane x holds the four neighbouring diagonals d0 + 4x .. d0 + 4x + 3, so the
+// cells of a lane follow each other along their diagonals.
+//
+// Why this shape: the cell loop is bound by instruction issue.  Along a
+// diagonal the coordinate difference e(s) = y[s] - y[s + d] of row s serves
+// the cells of rows s, s - tau, .., s - (m-1) tau, so a lane that walks down
+// its diagonals needs one subtraction and (m = 3) one three-input maximum per
+// cell, where a lane that holds one row needs m subtractions.  Four
+// neighbouring diagonals share their column values (row r, diagonal j reads
+// value r + j of a window), so four rows of a lane's sixteen cells take one
+// 16-byte shared load for the columns and one (broadcast) for the rows.
+#pragma once
+#include <cstdint>
+#include "rqa_common.cuh"
+
+namespace rqa {
+
+constexpr int DPL = 4;             // diagonals per lane
+constexpr int RB = ROW_BLOCK;      // 28 rows per block: a multiple of 4 and of the ring of m = tau = 3
+constexpr int COLW = DB + RB + 4;  // column window of a block, in values
+constexpr int ROWW = 32;           // row window
+constexpr int WIN_WORDS = COLW + ROWW;  // 32-bit words of a warp's windows (16-byte multiples)
+static_assert(DB == 32 * DPL && RB % 4 == 0 && COLW % 32 == 0 && WIN_WORDS % 4 == 0, "band shape");
+
+// Work unit u of a launch: bands [b_lo, b_hi) of series s over rows
+// [r_lo, r_hi).  The units of a series are its row chunks of a.rc rows, each
+// cut into groups of a.nb bands; the chunk at r_lo has the bands whose
+// longest diagonal reaches it (diagonal pass) or every band (vertical pass).
+struct Unit {
+    int s, b_lo, b_hi, r_lo, r_hi;
+};
+template <bool VERT>
+__device__ __forceinline__ Unit unit_of(const CellArgs &a, int64_t u)
+{
+    int lo = 0, hi = a.n_pos;  // last pos with uprefix[pos] <= u
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (a.uprefix[mid] <= u) lo = mid;
+        else hi = mid;
+    }
+    Unit w;
+    w.s = a.order[lo];
+    const int ne = a.series[w.s].ne;
+    int64_t rem = u - a.uprefix[lo];
+    int bands = 0;
+    w.r_lo = 0;
+    for (;;) {
+        bands = VERT ? (ne + DB - 1) / DB : (ne - 1 - w.r_lo + DB - 1) / DB;
+        const int items = (bands + a.nb - 1) / a.nb;
+        if (rem < items || w.r_lo + a.rc >= ne) break;
+        rem -= items;
+        w.r_lo += a.rc;
+    }
+    w.b_lo = (int)rem * a.nb;
+    w.b_hi = min(w.b_lo + a.nb, bands);
+    w.r_hi = min(w.r_lo + a.rc, ne);
+    return w;
+}
+
+// Distances of the compile-time embedding (M, TAU): the ring e[] holds the
+// coordinate differences of the last (M-1) TAU rows of each diagonal.
+template <int M, int TAU>
+struct DiagSrc {
+    static constexpr int H = (M - 1) * TAU, RS = H + 1;
+    float e[RS][DPL];
+    float pc[COLW / 32], pr;  // the next block's windows on their way from memory
+    float4 c0;
+    const float *ys;
+    int n, d0, lane;
+    float *cw, *rw;
+
+    __device__ __forceinline__ void init(const float *y, const SeriesDev &sd, int lane_, uint32_t *win)
+    {
+        ys = y;
+        n = sd.n;
+        lane = lane_;
+        cw = reinterpret_cast<float *>(win);
+        rw = cw + COLW;
+    }
+    __device__ __forceinline__ void fetch(int i0)
+    {
+        const int cb = i0 + H + d0 + lane, rr = i0 + H + lane;
+#pragma unroll
+        for (int x = 0; x < COLW / 32; ++x) pc[x] = cb + 32 * x < n ? __ldg(ys + cb + 32 * x) : 0.f;
+        pr = lane < RB && rr < n ? __ldg(ys + rr) : 0.f;
+    }
+    // first block of a walk: the differences of the rows above its ring
+    __device__ __forceinline__ void begin(int d, int i0)
+    {
+        d0 = d;
+#pragma unroll
+        for (int s = 0; s < H; ++s)
+#pragma unroll
+            for (int j = 0; j < DPL; ++j) {
+                const int c = i0 + s + d0 + DPL * lane + j;
+                e[s][j] = c < n ? __ldg(ys + i0 + s) - __ldg(ys + c) : 0.f;
+            }
+        fetch(i0);
+    }
+    // the windows of block i0 into shared memory, those of the next one requested
+    __device__ __forceinline__ void enter(int i0)
+    {
+        __syncwarp();
+#pragma unroll
+        for (int x = 0; x < COLW / 32; ++x) cw[lane + 32 * x] = pc[x];
+        rw[lane] = pr;
+        __syncwarp();
+        fetch(i0 + RB);
+        c0 = *reinterpret_cast<const float4 *>(cw + DPL * lane);
+    }
+    // distances of rows 4u .. 4u+3 of the block; u is a compile-time constant
+    // after unrolling (it picks the ring's registers)
+    template <bool CHECK>
+    __device__ __forceinline__ void quad(int u, int, float (&d)[4][DPL])
+    {
+        const float4 r4 = *reinterpret_cast<const float4 *>(rw + 4 * u);
+        const float4 c1 = *reinterpret_cast<const float4 *>(cw + 4 * u + 4 + DPL * lane);
+        const float rv[4] = {r4.x, r4.y, r4.z, r4.w};
+        const float cv[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int j = 0; j < DPL; ++j) {
+                const int t = 4 * u + r;
+                e[(t + H) % RS][j] = rv[r] - cv[r + j];
+                float x[M];
+#pragma unroll
+                for (int q = 0; q < M; ++q) x[q] = e[(t + q * TAU) % RS][j];
+                d[r][j] = maxnorm<M>(x);
+            }
+        c0 = c1;
+    }
+    __device__ __forceinline__ void leave()
+    {
+        constexpr int SH = RB % RS;  // the ring's phase moves on by this many rows per block
+        if constexpr (SH != 0) {
+            float t[RS][DPL];
+#pragma unroll
+            for (int s = 0; s < RS; ++s)
+#pragma unroll
+                for (int j = 0; j < DPL; ++j) t[s][j] = e[(s + SH) % RS][j];
+#pragma unroll
+            for (int s = 0; s < RS; ++s)
+#pragma unroll
+                for (int j = 0; j < DPL; ++j) e[s][j] = t[s][j];
+        }
+    }
+};
+
+// Any embedding (m and tau at run time, also unlike between the series of a
+// batch): the values are read through L1, two coordinates per step so that
+// one three-input maximum serves both.  CHECK: indexes past the series are
+// pulled back to its last value (the caller discards those cells).
+struct GenSrc {
+    const float *ys;
+    int n, d0, lane, m, tau;
+
+    __device__ __forceinline__ void init(const float *y, const SeriesDev &sd, int lane_, uint32_t *)
+    {
+        ys = y;
+        n = sd.n;
+        m = sd.m;
+        tau = sd.tau;
+        lane = lane_;
+    }
+    __device__ __forceinline__ void begin(int d, int) { d0 = d; }
+    __device__ __forceinline__ void enter(int) {}
+    template <bool CHECK>
+    __device__ __forceinline__ float at(int i) const
+    {
+        return __ldg(ys + (CHECK ? min(i, n - 1) : i));
+    }
+    template <bool CHECK>
+    __device__ __forceinline__ void diff(int ri, float (&x)[4][DPL]) const
+    {
+        const int ci = ri + d0 + DPL * lane;
+        float rv[4], cv[3 + DPL];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) rv[r] = at<CHECK>(ri + r);
+#pragma unroll
+        for (int c = 0; c < 3 + DPL; ++c) cv[c] = at<CHECK>(ci + c);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int j = 0; j < DPL; ++j) x[r][j] = rv[r] - cv[r + j];
+    }
+    template <bool CHECK>
+    __device__ __forceinline__ void quad(int u, int i0, float (&d)[4][DPL])
+    {
+        const int i = i0 + 4 * u;
+        diff<CHECK>(i, d);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int j = 0; j < DPL; ++j) d[r][j] = fabsf(d[r][j]);
+        int q = 1;
+        for (; q + 1 < m; q += 2) {
+            float a[4][DPL], b[4][DPL];
+            diff<CHECK>(i + q * tau, a);
+            diff<CHECK>(i + (q + 1) * tau, b);
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int j = 0; j < DPL; ++j) d[r][j] = fmax3(d[r][j], fabsf(a[r][j]), fabsf(b[r][j]));
+        }
+        if (q < m) {
+            float a[4][DPL];
+            diff<CHECK>(i + q * tau, a);
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int j = 0; j < DPL; ++j) d[r][j] = fmaxf(d[r][j], fabsf(a[r][j]));
+        }
+    }
+    __device__ __forceinline__ void leave() {}
+};
+
+// Walk rows [r_lo, r_hi) of the band at diagonal d0 and hand every cell's
+// distance key to f(key, valid): valid is a compile-time true inside the
+// triangle (CHECK false) and a run-time flag in blocks that reach over its
+// edge.
+template <class Src, class F>
+__device__ __forceinline__ void walk_keys(Src &src, int ne, int d0, int r_lo, int r_hi, int lane, F &&f)
+{
+    const int r_end = min(r_hi, ne - d0);           // rows of the longest diagonal
+    const int r_in = min(r_end, ne - d0 - DB + 1);  // rows where all 128 diagonals have a cell
+    if (r_lo >= r_end) return;
+    src.begin(d0, r_lo);
+    int i0 = r_lo;
+    for (; i0 + RB <= r_in; i0 += RB) {
+        src.enter(i0);
+#pragma unroll
+        for (int u = 0; u < RB / 4; ++u) {
+            float d[4][DPL];
+            src.template quad<false>(u, i0, d);
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int j = 0; j < DPL; ++j) f(__float_as_uint(d[r][j]), true);
+        }
+        src.leave();
+    }
+    const int lim = ne - d0 - DPL * lane;  // rows of the lane's first diagonal
+    for (; i0 < r_end; i0 += RB) {
+        src.enter(i0);
+#pragma unroll
+        for (int u = 0; u < RB / 4; ++u) {
+            float d[4][DPL];
+            src.template quad<true>(u, i0, d);
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int j = 0; j < DPL; ++j) {
+                    const int i = i0 + 4 * u + r;
+                    f(__float_as_uint(d[r][j]), i < lim - j && i < r_hi);
+                }
+        }
+        src.leave();
+    }
+}
+
+}  // namespace rqa

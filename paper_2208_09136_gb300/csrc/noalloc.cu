@@ -21,11 +21,6 @@ namespace rqa {
 namespace {
 
 constexpr int NA_MAX_S = RQA_NOALLOC_MAX_SERIES;
-constexpr int NA_MAX_ITEMS_PER_SERIES = 1024;
-// Cells of one work item at most: the counting kernels histogram an item in
-// 32-bit shared bins, so an item of more cells could wrap a bin that holds
-// most of its keys (a constant or heavily quantised series).
-constexpr uint64_t NA_ITEM_CELLS_MAX = (uint64_t)1 << 30;
 constexpr int NA_KMAX = RQA_NOALLOC_K_MAX;  // targets per call here (one middle-round launch)
 static_assert(NA_KMAX < MID_GROUPS && NA_KMAX >= NSUB_MAX, "fixed-scratch layout assumptions");
 
@@ -36,17 +31,17 @@ constexpr size_t O_STATUS = 0;
 constexpr size_t O_QUEUE = O_STATUS + 256;
 constexpr size_t O_SERIES = O_QUEUE + 256;
 constexpr size_t O_T = O_SERIES + al(sizeof(SeriesDev) * NA_MAX_S);
-constexpr size_t O_ITEMS = O_T + al(sizeof(uint64_t) * NA_MAX_S * NA_KMAX);
-constexpr size_t O_PREFIX = O_ITEMS + al(sizeof(Item) * NA_MAX_S * NA_MAX_ITEMS_PER_SERIES);
+constexpr size_t O_ORDER = O_T + al(sizeof(uint64_t) * NA_MAX_S * NA_KMAX);
+constexpr size_t O_UPREFIX = O_ORDER + al(sizeof(int32_t) * NA_MAX_S);
+constexpr size_t O_PREFIX = O_UPREFIX + al(sizeof(int64_t) * (NA_MAX_S + 1));
 constexpr size_t O_LEVEL = O_PREFIX + al(sizeof(uint32_t) * NA_MAX_S * NA_KMAX);
 constexpr size_t O_RANK = O_LEVEL + al(sizeof(uint8_t) * NA_MAX_S * NA_KMAX);
 constexpr size_t O_BELOW = O_RANK + al(sizeof(uint64_t) * NA_MAX_S * NA_KMAX);
 constexpr size_t O_TSUB = O_BELOW + al(sizeof(uint64_t) * NA_MAX_S * NA_KMAX);
 constexpr size_t O_TMID = O_TSUB + al((size_t)NA_MAX_S * NCOARSE);
-constexpr size_t O_TFIN1 = O_TMID + al((size_t)NA_MAX_S * NCOARSE);
-constexpr size_t O_TFIN2 = O_TFIN1 + al((size_t)NA_MAX_S * NCOARSE);
-constexpr size_t O_NGROUPS = O_TFIN2 + al((size_t)NA_MAX_S * NA_KMAX * NFINE);
-constexpr size_t O_RANGE = O_NGROUPS + al(sizeof(int32_t) * 3 * NA_MAX_S);
+constexpr size_t O_THASH = O_TMID + al((size_t)NA_MAX_S * NCOARSE);
+constexpr size_t O_NGROUPS = O_THASH + al(sizeof(uint32_t) * (size_t)NA_MAX_S * NHASH);
+constexpr size_t O_RANGE = O_NGROUPS + al(sizeof(int32_t) * 4 * NA_MAX_S);
 constexpr size_t O_REDO = O_RANGE + al(sizeof(uint32_t) * 2 * NA_MAX_S);
 constexpr size_t O_HIST = O_REDO + 256;
 constexpr size_t NA_BYTES = O_HIST + al(sizeof(uint64_t) * NA_HSTRIDE * NA_MAX_S);
@@ -61,8 +56,7 @@ struct NaPlan {
     int S, K;
     SeriesDev sd[NA_MAX_S];
     uint64_t T[NA_MAX_S][NA_KMAX];
-    int chunk[NA_MAX_S];       // bands per work item
-    int item_begin[NA_MAX_S + 1];
+    int64_t uprefix[NA_MAX_S + 1];  // work units per series
 };
 
 // Per-device set-up: the device address of g_scratch and the SM count.
@@ -117,25 +111,19 @@ __global__ void k_na_setup(NaPlan pl, unsigned char *scr)
 {
     SeriesDev *sd = reinterpret_cast<SeriesDev *>(scr + O_SERIES);
     uint64_t *T = reinterpret_cast<uint64_t *>(scr + O_T);
-    Item *items = reinterpret_cast<Item *>(scr + O_ITEMS);
+    int32_t *order = reinterpret_cast<int32_t *>(scr + O_ORDER);
+    int64_t *uprefix = reinterpret_cast<int64_t *>(scr + O_UPREFIX);
     const int t = threadIdx.x;
     if (t == 0) *reinterpret_cast<int *>(scr + O_STATUS) = 0;
     if (t < 64) reinterpret_cast<unsigned *>(scr + O_QUEUE)[t] = 0u;
-    if (t < 3 * NA_MAX_S) reinterpret_cast<int32_t *>(scr + O_NGROUPS)[t] = 0;
+    if (t < 4 * NA_MAX_S) reinterpret_cast<int32_t *>(scr + O_NGROUPS)[t] = 0;
     if (t < NA_MAX_S) scr[O_REDO + t] = 1;  // the plain coarse round for every series
     for (int s = 0; s < pl.S; ++s) {
         if (t == 0) sd[s] = pl.sd[s];
         if (t < pl.K) T[s * pl.K + t] = pl.T[s][t];
-        const int n_it = pl.item_begin[s + 1] - pl.item_begin[s];
-        for (int i = t; i < n_it; i += blockDim.x) {
-            Item it;
-            it.s = s;
-            it.b_lo = i * pl.chunk[s];
-            it.b_hi = min((i + 1) * pl.chunk[s], pl.sd[s].nbands);
-            it.pad = 0;
-            items[pl.item_begin[s] + i] = it;
-        }
     }
+    if (t < pl.S) order[t] = t;
+    if (t <= pl.S) uprefix[t] = pl.uprefix[t];
 }
 
 __global__ void k_na_status(const unsigned char *scr, int *status_out)
@@ -165,7 +153,7 @@ extern "C" int rqa_eps_for_rr_noalloc(const rqa_batch *b, const int32_t *rr_num,
     std::memset(&pl, 0, sizeof(pl));
     pl.S = b->n_series;
     pl.K = K;
-    int n_items = 0;
+    uint64_t total = 0;
     for (int s = 0; s < pl.S; ++s) {
         const int64_t n = b->offsets[s + 1] - b->offsets[s];
         if (n < 0 || b->m[s] < 1 || b->m[s] > RQA_M_MAX || b->tau[s] < 1) return RQA_ERR_INVALID_ARG;
@@ -180,21 +168,9 @@ extern "C" int rqa_eps_for_rr_noalloc(const rqa_batch *b, const int32_t *rr_num,
         d.tau = b->tau[s];
         d.ne = (int32_t)ne;
         d.P = (uint64_t)ne * (uint64_t)(ne - 1) / 2;
-        d.nbands = (int32_t)((ne - 1 + BAND - 1) / BAND);
         if (rqa_target_counts(d.P, rr_num, rr_den, K, pl.T[s]) != RQA_OK) return RQA_ERR_INVALID_ARG;
-        // at least ITEM_MIN_BANDS bands (1024 diagonals) per item, at most
-        // NA_MAX_ITEMS_PER_SERIES items
-        int chunk = ITEM_MIN_BANDS;
-        while ((d.nbands + chunk - 1) / chunk > NA_MAX_ITEMS_PER_SERIES) chunk *= 2;
-        // the largest item is the first (the longest diagonals 1..chunk*BAND);
-        // every Ne up to RQA_NOALLOC_NE_MAX passes, this guards the invariant
-        const int64_t dl = std::min<int64_t>((int64_t)chunk * BAND, ne - 1);
-        if ((uint64_t)(dl * ne - dl * (dl + 1) / 2) > NA_ITEM_CELLS_MAX) return RQA_ERR_CAPACITY;
-        pl.chunk[s] = chunk;
-        pl.item_begin[s] = n_items;
-        n_items += (d.nbands + chunk - 1) / chunk;
+        total += d.P;
     }
-    pl.item_begin[pl.S] = n_items;
 
     int device = 0;
     if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= NA_MAX_DEVICES) {
@@ -209,6 +185,9 @@ extern "C" int rqa_eps_for_rr_noalloc(const rqa_batch *b, const int32_t *rr_num,
     if (int rc = na_setup(device, dv)) return rc;
     unsigned char *scr = dv.scratch;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const Split split = split_cells(total, COUNT_NB, dv.sm_count);
+    pl.uprefix[0] = 0;
+    for (int s = 0; s < pl.S; ++s) pl.uprefix[s + 1] = pl.uprefix[s] + units_of_series(pl.sd[s].ne, split, false);
 
     // ---- the selection, as rqa_eps_for_rr runs it, on the fixed scratch
     int embed = E_GENERIC;
@@ -229,7 +208,7 @@ extern "C" int rqa_eps_for_rr_noalloc(const rqa_batch *b, const int32_t *rr_num,
     int *status = reinterpret_cast<int *>(scr + O_STATUS);
     if (launch_check_finite(b->y, b->offsets[pl.S], status, st) != cudaSuccess) return RQA_ERR_CUDA;
 
-    SelBufs sb{};  // no hashed final-round table here: tab_hash = hash_mul = null
+    SelBufs sb{};
     sb.T = reinterpret_cast<const uint64_t *>(scr + O_T);
     sb.prefix = reinterpret_cast<uint32_t *>(scr + O_PREFIX);
     sb.level = reinterpret_cast<uint8_t *>(scr + O_LEVEL);
@@ -237,13 +216,12 @@ extern "C" int rqa_eps_for_rr_noalloc(const rqa_batch *b, const int32_t *rr_num,
     sb.below = reinterpret_cast<uint64_t *>(scr + O_BELOW);
     sb.tab_sub = reinterpret_cast<int8_t *>(scr + O_TSUB);
     sb.tab_mid = reinterpret_cast<int8_t *>(scr + O_TMID);
-    sb.tab_fin1 = reinterpret_cast<int8_t *>(scr + O_TFIN1);
-    sb.tab_fin2 = reinterpret_cast<int8_t *>(scr + O_TFIN2);
-    sb.fin2_stride = (int64_t)NA_KMAX * NFINE;
+    sb.tab_hash = reinterpret_cast<uint32_t *>(scr + O_THASH);
     int32_t *ng = reinterpret_cast<int32_t *>(scr + O_NGROUPS);
     sb.n_sub = ng;
     sb.n_mid = ng + pl.S;
     sb.n_fin = ng + 2 * pl.S;
+    sb.hash_mul = reinterpret_cast<uint32_t *>(ng + 3 * pl.S);
     sb.range = reinterpret_cast<uint32_t *>(scr + O_RANGE);
     sb.redo = scr + O_REDO;
     sb.hist = reinterpret_cast<uint64_t *>(scr + O_HIST);
@@ -252,13 +230,16 @@ extern "C" int rqa_eps_for_rr_noalloc(const rqa_batch *b, const int32_t *rr_num,
     CellArgs a{};
     a.y = b->y;
     a.series = reinterpret_cast<const SeriesDev *>(scr + O_SERIES);
-    a.items = reinterpret_cast<const Item *>(scr + O_ITEMS);
-    a.n_items = n_items;
-    a.band = BAND;
+    a.order = reinterpret_cast<const int32_t *>(scr + O_ORDER);
+    a.uprefix = reinterpret_cast<const int64_t *>(scr + O_UPREFIX);
+    a.n_pos = pl.S;
+    a.nb = split.nb;
+    a.rc = split.rc;
+    a.n_units = pl.uprefix[pl.S];
     a.g0 = 0;
     a.gn = MID_GROUPS;  // K <= NA_KMAX < MID_GROUPS: one middle-round launch
     a.status = status;
-    const int grid = (int)(n_items < dv.sm_count * 2 ? n_items : dv.sm_count * 2);
+    const int grid = (int)std::min<int64_t>(a.n_units, (int64_t)dv.sm_count * 8);
     const int rounds[3] = {R_COARSE, R_MID, R_FINAL};
     unsigned *queue = reinterpret_cast<unsigned *>(scr + O_QUEUE);
     for (int r = 0; r < 3; ++r) {
@@ -267,9 +248,9 @@ extern "C" int rqa_eps_for_rr_noalloc(const rqa_batch *b, const int32_t *rr_num,
             return RQA_ERR_CUDA;
         }
         a.queue = queue + 16 * r;
-        if (launch_count(rounds[r], a, sb, K, grid < 1 ? 1 : grid, embed, st) != cudaSuccess)
+        if (launch_count(rounds[r], a, sb, K, grid, embed, st) != cudaSuccess)
             return RQA_ERR_CUDA;
-        if (launch_select(rounds[r], sb, a.series, 0, pl.S, K, eps_out, count_le, count_lt, status,
+        if (launch_select(rounds[r], sb, 0, pl.S, K, eps_out, count_le, count_lt, status,
                           st) != cudaSuccess)
             return RQA_ERR_CUDA;
     }

@@ -228,27 +228,4 @@ inline int persistent_cap(const void *kern, int smem, int grid, int threads = TH
     return grid < cap ? grid : (cap > 0 ? cap : 1);
 }
 
-// Threads per CTA of a counting round: rounds whose shared histogram allows
-// only two CTAs per SM run twice as many warps per CTA.
-__host__ __device__ constexpr int count_threads(int round) { return (round == 1 || round == 2) ? 512 : THREADS; }
-
-// Fetch the next work item for this CTA (one atomic per CTA), -1 when done.
-__device__ __forceinline__ int next_item(unsigned int *queue, int n_items, int *sh_slot)
-{
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned t = atomicAdd(queue, 1u);
-        *sh_slot = (t < (unsigned)n_items) ? (int)t : -1;
-    }
-    __syncthreads();
-    return *sh_slot;
-}
-
-// Diagonals of band b: [d_lo, d_hi), d_hi <= Ne.
-__device__ __forceinline__ void band_range(int b, int band, int ne, int &d_lo, int &d_hi)
-{
-    d_lo = 1 + b * band;
-    d_hi = min(d_lo + band, ne);
-}
-
 }  // namespace rqa

@@ -22,13 +22,10 @@ constexpr int NSUB_MAX = 24;       // bracket-subdivided coarse buckets per seri
 constexpr int LSH = 64;            // line lengths 1..LSH counted in shared memory
 constexpr int LMIN_MAX = 8;        // entries of an lmin list
 constexpr int THREADS = 256;       // threads per CTA of the cell kernels
-constexpr int BAND = 32;           // diagonals per warp band of the counting rounds
-constexpr int ITEM_MIN_BANDS = 4 * 16 * 16 / BAND;  // bands of a work item (1024 diagonals) at least
+constexpr int DB = 128;            // diagonals (columns) per warp band of the cell walk
 constexpr int LINE_TILE_DEFAULT = 16;  // diagonals per register window of the line pass's cell phase
 constexpr int LINE_NE_MAX = (1 << 26) - 1;  // vectors per series the line pass counts exactly
-// vectors per series the counting rounds take: a work item holds under 2^30
-// cells plus one band (BAND x Ne), so its 32-bit shared bins cannot overflow
-constexpr int64_t COUNT_NE_MAX = ((int64_t)3 << 30) / BAND;
+constexpr int64_t COUNT_NE_MAX = (int64_t)3 << 25;  // vectors per series the counting rounds take
 constexpr int WARPS = THREADS / 32;
 
 // Counting rounds of the selection.
@@ -45,12 +42,6 @@ struct SeriesDev {
     int32_t ne;       // Ne = N - (m-1) tau
     int32_t m, tau;
     uint64_t P;       // Ne (Ne - 1) / 2
-    int32_t nbands;   // ceil((Ne - 1) / band)
-    int32_t pad;
-};
-
-struct Item {         // bands [b_lo, b_hi) of series s: one CTA's unit of work
-    int32_t s, b_lo, b_hi, pad;
 };
 
 // Device buffers of the selection state; [s*K + k] unless stated.
@@ -62,12 +53,9 @@ struct SelBufs {
     uint64_t *below;       // keys below the current key interval
     int8_t *tab_sub;       // [s][NCOARSE] bracket split buckets -> group, -1
     int8_t *tab_mid;       // [s][NCOARSE] coarse bucket -> middle group, -1
-    int8_t *tab_fin1;      // [s][NCOARSE] coarse bucket -> final super group, -1
-    int8_t *tab_fin2;      // [s][fin2_stride] = [s][targets][NFINE] (super group, middle digit) -> group
-    int64_t fin2_stride;   // entries of tab_fin2 per series (>= K * NFINE)
-    uint32_t *tab_hash;    // [s][NHASH] prefix | group << 21 at slot (prefix * mul) >> 20,
-                           // 0x1fffff empty; may be null (two-level tables only)
-    uint32_t *hash_mul;    // [s]: the slot multiplier, 0 = no collision-free one (or no table)
+    uint32_t *tab_hash;    // [s][NHASH] final round: prefix | group << 21 at slot (prefix * mul) >> 20,
+                           // 0x1fffff empty
+    uint32_t *hash_mul;    // [s]: the slot multiplier, 0 = no collision-free one
     int32_t *n_sub, *n_mid, *n_fin;   // [s]
     uint32_t *range;       // [s][2]: keys the next filtered round can count, inclusive
     uint8_t *redo;         // [s]: 1 = the plain coarse round runs for this series
@@ -78,17 +66,13 @@ struct SelBufs {
 struct CellArgs {
     const float *y;
     const SeriesDev *series;
-    // CTA-level work (counting rounds): items of bands
-    const Item *items;
-    int32_t n_items;
-    int32_t band;
     int32_t g0, gn;          // middle round: the groups [g0, g0 + gn) this launch counts
-    // warp-level work (line pass): units of `chunk` consecutive bands of the
-    // series order[0..n_pos)
+    // work units along the series order[0..n_pos)
     const int32_t *order;    // series, largest first
     const int64_t *uprefix;  // n_pos + 1 prefix of unit counts along order
     int32_t n_pos;
-    int32_t chunk;           // bands per unit
+    int32_t nb, rc;          // cell walk: bands per unit and rows per unit (a multiple of RB)
+    int32_t chunk;           // line pass: bands per unit
     int32_t line_tile;       // diagonals per register window of the line pass (8, 16 or 32)
     int32_t line_ctas;       // persistent CTAs of the line pass per SM (0: as many as fit)
     int32_t line_stage;      // line pass: stage the series windows by bulk copies (where supported)
@@ -98,14 +82,27 @@ struct CellArgs {
     int *status;
 };
 
+// How a launch of the cell walk cuts its work: units of `nb` bands of DB
+// diagonals over `rc` rows.
+struct Split {
+    int nb, rc;
+};
+constexpr int ROW_BLOCK = 28;  // rows per block of the cell walk (units start on block boundaries)
+constexpr int COUNT_NB = 8;  // bands per unit of the counting rounds: one per warp of a CTA
+// About six units per CTA (two CTAs per SM) over the whole launch, and rows
+// per unit between 8 and 585 blocks: shorter chunks pay their first window
+// loads over too few cells, longer ones leave a tail.
+Split split_cells(uint64_t cells, int nb, int sm_count);
+// Units of a series of ne vectors (vert: the vertical pass, every column over every row).
+int64_t units_of_series(int64_t ne, const Split &sp, bool vert);
+
 // Kernels (launch wrappers return cudaGetLastError()).
 cudaError_t launch_check_finite(const float *y, int64_t n, int *status, cudaStream_t st);
 // embed: the Embed code of the batch (rqa_common.cuh), picks the distance kernel variant.
 cudaError_t launch_count(int round, const CellArgs &a, const SelBufs &sb, int K, int grid,
                          int embed, cudaStream_t st);
-cudaError_t launch_select(int round, const SelBufs &sb, const SeriesDev *series, int s_begin,
-                          int n_series, int K, float *eps_out, uint64_t *le_out,
-                          uint64_t *lt_out, int *status, cudaStream_t st);
+cudaError_t launch_select(int round, const SelBufs &sb, int s_begin, int n_series, int K, float *eps_out,
+                          uint64_t *le_out, uint64_t *lt_out, int *status, cudaStream_t st);
 
 struct LineBufs {
     const float *eps;      // [s*kstride + k], ascending per series

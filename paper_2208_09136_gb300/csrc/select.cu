@@ -15,7 +15,7 @@
 // #{d < eps_k} = below, #{d <= eps_k} = below + (keys equal to eps_k).
 #include <cstdint>
 #include <type_traits>
-#include "rqa_common.cuh"
+#include "dense.cuh"
 
 namespace rqa {
 
@@ -39,243 +39,289 @@ cudaError_t launch_check_finite(const float *y, int64_t n, int *status, cudaStre
 }
 
 // ------------------------------------------------------------ counting
-int count_smem_bytes(int round, int K)
+// Dynamic shared memory of a counting CTA: the warps' windows, the bins
+// (32-bit) and the lookup table of its round.
+constexpr int CT = 256;        // threads per CTA
+constexpr int CW = CT / 32;
+constexpr int SUB_WIN = 512;   // coarse buckets of a sparse bracket round counted in shared memory
+constexpr int DENSE_FINAL = 48 * NFINE;  // prefixes the final round's byte table can span
+
+static int count_bins(int round, int K)
 {
     switch (round) {
-    case R_COARSE: return NCOARSE * 4;
-    case R_COARSE_SUB: return (NCOARSE + NSUB_MAX * NFINE) * 4 + NCOARSE;
-    case R_MID: return (K < MID_GROUPS ? K : MID_GROUPS) * NFINE * 4 + NCOARSE;
-    default: {  // tables only (final-round keys are rare): the hash or the two levels
-        const int two = NCOARSE + 1 + K * NFINE;
-        return two > NHASH * 4 ? two : NHASH * 4;
+    case R_COARSE: return NCOARSE;
+    case R_COARSE_SUB: return SUB_WIN + NSUB_MAX * NFINE;
+    case R_MID: {
+        const int g = K < MID_GROUPS ? K : MID_GROUPS;
+        return (g > NSUB_MAX ? g : NSUB_MAX) * NFINE + 4;  // dense: a bin below and one above the range
     }
+    default: return 0;
     }
 }
 
-__device__ __forceinline__ uint32_t smem_addr(const uint32_t *p)
+int count_smem_bytes(int round, int K)
 {
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+    const int win = CW * WIN_WORDS * 4;
+    switch (round) {
+    case R_COARSE: return win + NCOARSE * 4;
+    case R_COARSE_SUB: case R_MID: return win + count_bins(round, K) * 4 + NCOARSE;
+    default: return win + (DENSE_FINAL + 16 > NHASH * 4 ? DENSE_FINAL + 16 : NHASH * 4);
+    }
 }
 
-// Resident CTAs per SM the compiler must leave room for (0: no bound): the
-// final round of the compile-time embeddings with tau > 1 fits four in 64
-// registers without spills instead of three in 80; the others keep the
-// compiler's own choice.
-__host__ __device__ constexpr int count_min_ctas(int round, int tau)
-{
-    return round == R_FINAL && tau > 1 ? 4 : 0;
-}
-
-// One persistent launch over the work items; each CTA histograms the keys of
-// its item's bands in shared memory and adds the non-zero bins to the
-// series' 64-bit global histogram at the end of the item.
+// One persistent launch over the work units.  A CTA keeps the bins of one
+// series in shared memory over all the units of it that it takes and adds
+// the non-zero ones to the series' 64-bit global histogram when the series
+// changes (or before a 32-bit bin could overflow).
 //
-// R_COARSE counts every key.  The bracket round counts only the keys of its
-// split range and keeps the keys below it as one register count; the middle
-// and final rounds look each key up in their group tables (the final round's
-// rare hits go straight to the global bins, so it needs no shared histogram).
-template <int ROUND, int M, int TAU>
-__global__ void __launch_bounds__(count_threads(ROUND), count_min_ctas(ROUND, TAU)) k_count(CellArgs a, SelBufs sb, int K)
+// Bins of a cell:
+//   R_COARSE      key >> 20.
+//   split ranges  (bracket round; middle round when the targets' coarse
+//                 buckets span at most NSUB_MAX) the 21-bit prefix relative to
+//                 the range, clamped to one bin below and one above it: a
+//                 shift, one DPX clamp and one unconditional reduction per
+//                 cell.  The hardware merges the lanes that meet in a bin, so
+//                 the crowded outer bins cost nothing (measured: 2.1 cycles
+//                 per SM and warp reduction with 80 % of the lanes in one
+//                 bin, 2.5 with all lanes spread; a predicated reduction of
+//                 20 % of the lanes 4.2).
+//   other ranges  through the group table of the coarse buckets.
+//   R_FINAL       keys of a target's 21-bit prefix are rare and go straight
+//                 to the global bins: the prefix relative to the range is
+//                 looked up in a byte table (spans up to DENSE_FINAL), else
+//                 in a hashed table (slot = prefix x multiplier >> 20; the
+//                 slot holds the only target prefix that can map there), else
+//                 by binary search.
+//
+// Bound by shared-memory reductions and issue: one reduction and 5 to 9
+// instructions per cell (32 cells: per warp).  Units are row chunks of a few
+// bands (dense.cuh), so a batch of four 10^4-value series fills the chip.
+template <int ROUND, class Src>
+__global__ void __launch_bounds__(CT) k_count(CellArgs a, SelBufs sb, int K, int nbins)
 {
-    constexpr int NT = count_threads(ROUND);
-    constexpr bool FILTERED = ROUND != R_COARSE;
-    constexpr bool GLOBAL_BINS = ROUND == R_FINAL;  // final-round keys are rare: count in HBM
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int slot;
-    __shared__ int nb_used_sh;
-    __shared__ uint32_t hmul_sh;
+    __shared__ Unit unit;
     __shared__ int next_band;
-    __shared__ uint32_t key_lo, key_hi;
-    __shared__ unsigned long long below_sh;
     __shared__ uint32_t sink[32];  // lane x's reductions of cells that count nowhere (never read)
-    const int nbins_max = (ROUND == R_COARSE) ? NCOARSE
-                        : (ROUND == R_COARSE_SUB) ? NCOARSE + NSUB_MAX * NFINE
-                        : (ROUND == R_MID) ? (K < MID_GROUPS ? K : MID_GROUPS) * NFINE : 0;
-    uint32_t *h = reinterpret_cast<uint32_t *>(smem);
-    int8_t *t1 = reinterpret_cast<int8_t *>(h + nbins_max);
-    int8_t *t2 = t1 + NCOARSE;
-    uint32_t *th = reinterpret_cast<uint32_t *>(smem);  // final round, hashed: instead of t1/t2
-    const int lane = threadIdx.x & 31;
+    __shared__ uint32_t pfx[KMAX + 1];  // final round: the distinct target prefixes, ascending
+    __shared__ int n_pfx;
+    __shared__ unsigned fbits[4];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t *win = reinterpret_cast<uint32_t *>(smem) + warp * WIN_WORDS;
+    uint32_t *h = reinterpret_cast<uint32_t *>(smem) + CW * WIN_WORDS;
+    int8_t *t1 = reinterpret_cast<int8_t *>(h + nbins);                   // sparse ranges
+    unsigned char *t8 = reinterpret_cast<unsigned char *>(h);             // final round, byte table
+    uint32_t *th = h;                                                     // final round, hashed table
 
-    for (int x = threadIdx.x; x < nbins_max; x += NT) h[x] = 0;
+    for (int x = threadIdx.x; x < nbins; x += CT) h[x] = 0;
 
-    for (;;) {
-        const int it = next_item(a.queue, a.n_items, &slot);
-        if (it < 0) break;
-        const Item item = a.items[it];
-        const SeriesDev sd = a.series[item.s];
-        if (threadIdx.x == 0) {
-            int nb;
-            if (ROUND == R_COARSE) nb = sb.redo[item.s] ? NCOARSE : 0;
-            else if (ROUND == R_COARSE_SUB) nb = sb.n_sub[item.s] ? NCOARSE + sb.n_sub[item.s] * NFINE : 0;
-            else if (ROUND == R_MID) nb = max(0, min(sb.n_mid[item.s] - a.g0, a.gn)) * NFINE;
-            else nb = sb.n_fin[item.s] * NFINE;
-            nb_used_sh = nb;
-            next_band = item.b_lo;
-            key_lo = 0u;
-            key_hi = 0xffffffffu;
-            if (FILTERED) {
-                key_lo = sb.range[2 * (int64_t)item.s];
-                key_hi = sb.range[2 * (int64_t)item.s + 1];
-            }
-            below_sh = 0ull;
-            hmul_sh = (ROUND == R_FINAL && sb.hash_mul) ? sb.hash_mul[item.s] : 0u;
-        }
+    int cur = -1;
+    bool busy = false;              // the current series has work in this round
+    uint64_t acc = 0;               // cells counted since the last flush
+    uint32_t klo = 0, kspan = 0;    // key range of the filtered rounds: key - klo <= kspan
+    int nfine = 0;                  // bins of the series' groups in this launch
+    bool dense = false;
+    uint32_t hmul = 0;
+    uint64_t below = 0;             // sparse bracket round: this lane's keys under the range
+    int32_t qoff = 0, qtop = 0;     // dense: clamp of the relative prefix
+
+    auto flush = [&]() {
+        if (cur < 0 || !busy || ROUND == R_FINAL) return;
         __syncthreads();
-        const int nb_used = nb_used_sh;
-        const uint32_t hmul = hmul_sh;
-        if (nb_used == 0) continue;  // no target of this series needs this round
-        if (ROUND == R_FINAL && hmul) {
-            const uint4 *src = reinterpret_cast<const uint4 *>(sb.tab_hash + (int64_t)item.s * NHASH);
-            for (int x = threadIdx.x; x < NHASH / 4; x += NT) reinterpret_cast<uint4 *>(th)[x] = src[x];
-            __syncthreads();
-        } else if (ROUND != R_COARSE) {
-            const int8_t *src = (ROUND == R_COARSE_SUB) ? sb.tab_sub
-                              : (ROUND == R_MID) ? sb.tab_mid : sb.tab_fin1;
-            src += (int64_t)item.s * NCOARSE;
-            for (int x = threadIdx.x; x < NCOARSE; x += NT) t1[x] = src[x];
-            if (ROUND == R_FINAL) {
-                const int8_t *s2 = sb.tab_fin2 + (int64_t)item.s * sb.fin2_stride;
-                for (int x = threadIdx.x; x < K * NFINE; x += NT) t2[1 + x] = s2[x];
-                if (threadIdx.x == 0) t2[0] = -1;
-            }
-            __syncthreads();
-        }
-
-        const float *ys = a.y + sd.off;
-        const uint32_t klo = key_lo, kspan = key_hi - key_lo;  // inside: key - klo <= kspan
-        unsigned long long *gbins =
-            reinterpret_cast<unsigned long long *>(sb.hist + (int64_t)item.s * sb.hstride + NCOARSE);
-        uint32_t below = 0;  // bracket round: keys under its range
-        // bracket round with every bucket from the first to the last split
-        // one split (the usual case): split group g is bucket first + g, so
-        // the bin is (key - klo) >> 10 past the coarse bins, no table
-        const bool dense = ROUND == R_COARSE_SUB && ((kspan >> COARSE_SHIFT) + 1u) * NFINE + NCOARSE ==
-                                                        (uint32_t)nb_used;
-        const uint32_t hsub = static_cast<uint32_t>(__cvta_generic_to_shared(h + NCOARSE));
-        const uint32_t sink_a = smem_addr(&sink[lane]);
-        // the item's bands; FAST: dense bracket round, or final round with the
-        // hashed prefix table
-        auto item_bands = [&](auto fast) {
-        constexpr bool FAST = decltype(fast)::value;
-        for (;;) {
-            // bands are handed to warps one at a time, so no warp idles while
-            // another still has several bands of the item left
-            int b = 0;
-            if (lane == 0) b = atomicAdd(&next_band, 1);
-            b = __shfl_sync(FULL, b, 0);
-            if (b >= item.b_hi) break;
-            int d_lo, d_hi;
-            band_range(b, BAND, sd.ne, d_lo, d_hi);
-            const int rows = sd.ne - d_lo;
-            int last = -1;
-            uint32_t run = 0;
-            // plain coarse round: every key counts and neighbouring cells of
-            // a lane often share a coarse bin, so equal bins are aggregated
-            auto count_coarse = [&](uint32_t key) {
-                const int bin = (int)(key >> COARSE_SHIFT);
-                if (bin == last) {
-                    ++run;
-                } else {
-                    if (run) atomicAdd(&h[last], run);
-                    last = bin;
-                    run = 1;
-                }
-            };
-            // the BAND cells of a lane in one row block; valid = inside the
-            // triangle.  The filtered rounds compute the bin of every cell
-            // (keys of finite or NaN distances have bit 31 clear, so key >> 20
-            // indexes the 2048-entry table).  The bracket round, where many
-            // cells fall in the range, adds one for every cell with an
-            // unconditional reduction (into the lane's sink word for a cell
-            // outside the range); a conditional one would make the compiler
-            // wrap each cell in a branch region.  The middle round, where few
-            // cells count, uses a predicated reduction, and the final round
-            // branches around its rare global atomics.
-            auto row_block = [&](const BandTile<M, TAU, BAND> &tile, int i, bool interior) {
-#pragma unroll
-                for (int j = 0; j < BAND; ++j) {
-                    const int dl = d_lo + j;
-                    const bool valid = interior || i < sd.ne - dl;
-                    const uint32_t key = __float_as_uint(tile.dist(ys, j, i, dl, sd.tau, sd.m));
-                    const int c = (int)(key >> COARSE_SHIFT);
-                    const int fine = (int)((key >> 10) & (NFINE - 1));
-                    if (ROUND == R_COARSE) {
-                        if (valid) count_coarse(key);
-                    } else if (ROUND == R_COARSE_SUB && FAST) {
-                        // keys under klo wrap to rel >= 2^31 (keys are < 2^31)
-                        const uint32_t rel = key - klo;
-                        below += valid ? rel >> 31 : 0u;
-                        red_shared(valid && rel <= kspan ? hsub + ((rel >> 10) << 2) : sink_a);
-                    } else if (ROUND == R_COARSE_SUB) {
-                        below += (valid && key < klo) ? 1u : 0u;
-                        const int g = t1[c];
-                        const int bin = g < 0 ? c : NCOARSE + g * NFINE + fine;
-                        red_shared(valid && key - klo <= kspan ? smem_addr(&h[bin]) : sink_a);
-                    } else if (ROUND == R_MID) {
-                        // groups outside this launch's window [g0, g0 + gn) wait for another
-                        const uint32_t gw = (uint32_t)((int)t1[c] - a.g0);
-                        red_shared_if_le(smem_addr(&h[min(gw, (uint32_t)(nbins_max / NFINE - 1)) * NFINE + fine]),
-                                         valid ? gw : ~0u, (uint32_t)a.gn - 1u);
-                    } else if (FAST) {
-                        // one probe: the slot holds the only target prefix
-                        // that can map there.  Empty slots hold group 0 with
-                        // prefix 0x1fffff, which only a NaN key (already an
-                        // error) can match, inside group 0's bins.
-                        const uint32_t pfx = key >> 10;
-                        const uint32_t e = th[(pfx * hmul) >> (32 - NHASH_BITS)];
-                        if (valid && ((e ^ pfx) & 0x1FFFFFu) == 0u)  // rare
-                            atomicAdd(gbins + (e >> 21) * NFINE + (key & (NFINE - 1)), 1ull);
-                    } else {
-                        // t2[0] is a -1 sentinel: no branch on the first lookup
-                        const int g1 = t1[c];
-                        const int g = t2[g1 < 0 ? 0 : 1 + g1 * NFINE + fine];
-                        if (valid && g >= 0)  // rare: a key of a target's 21-bit prefix
-                            atomicAdd(gbins + g * NFINE + (int)(key & (NFINE - 1)), 1ull);
-                    }
-                }
-            };
-            int i0 = 0;
-            // interior row blocks: every lane's cells on all BAND diagonals exist
-            for (; i0 + 32 <= rows - (BAND - 1); i0 += 32) {
-                BandTile<M, TAU, BAND> tile;
-                tile.load_fast(ys, i0 + lane, d_lo, sd.tau);
-                row_block(tile, i0 + lane, true);
-            }
-            for (; i0 < rows; i0 += 32) {
-                BandTile<M, TAU, BAND> tile;
-                tile.load(ys, sd.n, i0 + lane, d_lo, rows, sd.tau, sd.m);
-                row_block(tile, i0 + lane, false);
-            }
-            if (run) atomicAdd(&h[last], run);
-        }
-        };
-        if ((ROUND == R_FINAL && hmul) || dense) item_bands(std::true_type{});
-        else item_bands(std::false_type{});
-        if (ROUND == R_COARSE_SUB) {
-            // keys under the bracket: one count, kept in the coarse bucket
-            // just below it (every bucket under it is empty in this round)
-            unsigned long long bw = below;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) bw += __shfl_xor_sync(FULL, bw, o);
-            if (lane == 0 && bw) atomicAdd(&below_sh, bw);
-        }
-        __syncthreads();
-        if (ROUND == R_COARSE_SUB && threadIdx.x == 0 && below_sh) {
-            const int cb = (int)(klo >> COARSE_SHIFT) - 1;  // >= 0 whenever keys lie below
-            atomicAdd(reinterpret_cast<unsigned long long *>(sb.hist + (int64_t)item.s * sb.hstride + cb),
-                      below_sh);
-        }
-        uint64_t *gh = sb.hist + (int64_t)item.s * sb.hstride + (ROUND >= R_MID ? NCOARSE : 0) +
-                       (ROUND == R_MID ? (int64_t)a.g0 * NFINE : 0);
-        for (int x = threadIdx.x; x < (GLOBAL_BINS ? 0 : nb_used); x += NT) {
+        unsigned long long *gh =
+            reinterpret_cast<unsigned long long *>(sb.hist + (int64_t)cur * sb.hstride);
+        auto add = [&](unsigned long long *dst, int x) {
             const uint32_t v = h[x];
             if (v) {
-                atomicAdd(reinterpret_cast<unsigned long long *>(gh + x), (unsigned long long)v);
+                if (dst) atomicAdd(dst, (unsigned long long)v);
                 h[x] = 0;
             }
+        };
+        const int clo = (int)(klo >> COARSE_SHIFT);
+        if (ROUND == R_COARSE) {
+            for (int x = threadIdx.x; x < NCOARSE; x += CT) add(gh + x, x);
+        } else if (dense) {
+            // bin 0: keys under the range; they only count in the bracket
+            // round, kept in the coarse bucket just below it
+            for (int x = threadIdx.x; x < nfine + 2; x += CT) {
+                unsigned long long *dst = gh + NCOARSE + x - 1;
+                if (x == 0) dst = ROUND == R_COARSE_SUB && clo > 0 ? gh + clo - 1 : nullptr;
+                if (x == nfine + 1) dst = nullptr;
+                add(dst, x);
+            }
+        } else if (ROUND == R_COARSE_SUB) {
+            for (int x = threadIdx.x; x < SUB_WIN; x += CT) add(clo + x < NCOARSE ? gh + clo + x : nullptr, x);
+            for (int x = threadIdx.x; x < nfine; x += CT) add(gh + NCOARSE + x, SUB_WIN + x);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) below += __shfl_xor_sync(FULL, below, o);
+            if (lane == 0 && below && clo > 0) atomicAdd(gh + clo - 1, (unsigned long long)below);
+            below = 0;
+        } else {
+            for (int x = threadIdx.x; x < nfine; x += CT) add(gh + NCOARSE + (int64_t)a.g0 * NFINE + x, x);
+        }
+        acc = 0;
+        __syncthreads();
+    };
+
+    for (;;) {
+        __syncthreads();  // every warp done with the unit before
+        if (threadIdx.x == 0) {
+            const unsigned t = atomicAdd(a.queue, 1u);
+            if ((int64_t)t < a.n_units) {
+                unit = unit_of<false>(a, (int64_t)t);
+                next_band = unit.b_lo;
+            } else {
+                unit.s = -1;
+            }
+        }
+        __syncthreads();
+        const Unit w = unit;
+        if (w.s < 0) break;
+        const SeriesDev sd = a.series[w.s];
+        if (w.s != cur) {
+            flush();
+            cur = w.s;
+            if (ROUND == R_COARSE) {
+                busy = sb.redo[cur] != 0;
+            } else {
+                klo = sb.range[2 * (int64_t)cur];
+                kspan = sb.range[2 * (int64_t)cur + 1] - klo;
+                const int ng = ROUND == R_COARSE_SUB ? sb.n_sub[cur]
+                             : ROUND == R_MID ? max(0, min(sb.n_mid[cur] - a.g0, a.gn)) : sb.n_fin[cur];
+                nfine = ng * NFINE;
+                busy = ng > 0;
+                // every coarse bucket of the range is a group of its own, in order
+                dense = (kspan >> COARSE_SHIFT) + 1u == (uint32_t)ng && ng <= NSUB_MAX && a.g0 == 0;
+                if (ROUND == R_FINAL) {
+                    nfine = (int)(kspan >> 10) + 1;
+                    dense = kspan < (uint32_t)DENSE_FINAL << 10;
+                }
+                qoff = 1 - (int32_t)(klo >> 10);
+                qtop = nfine + 1;
+            }
+            if (busy && ROUND == R_FINAL) {
+                // the targets' prefixes ascend: one entry per run of equal ones
+                const int k = threadIdx.x;
+                uint32_t p = 0;
+                bool first = false;
+                if (k < K) {
+                    const uint32_t *pk = sb.prefix + (int64_t)cur * K + k;
+                    p = pk[0];
+                    first = k == 0 || pk[-1] != p;
+                }
+                const unsigned fb = __ballot_sync(FULL, first);
+                if (lane == 0 && warp < 4) fbits[warp] = fb;
+                __syncthreads();
+                if (k < 128) {
+                    int g = __popc(fb & ((1u << lane) - 1u));
+                    for (int x = 0; x < warp; ++x) g += __popc(fbits[x]);
+                    if (first) pfx[g] = p;
+                    if (k == 127) n_pfx = g + (first ? 1 : 0);
+                }
+                hmul = !dense && sb.hash_mul ? sb.hash_mul[cur] : 0u;
+                if (dense) {
+                    for (int x = threadIdx.x; x < (nfine + 2 + 3) / 4; x += CT) h[x] = 0;
+                } else if (hmul) {
+                    const uint4 *src = reinterpret_cast<const uint4 *>(sb.tab_hash + (int64_t)cur * NHASH);
+                    for (int x = threadIdx.x; x < NHASH / 4; x += CT) reinterpret_cast<uint4 *>(th)[x] = src[x];
+                }
+                __syncthreads();
+                if (dense && (int)threadIdx.x < n_pfx)
+                    t8[(int32_t)pfx[threadIdx.x] + qoff] = (unsigned char)(threadIdx.x + 1);
+                __syncthreads();
+            } else if (busy && ROUND != R_COARSE && !dense) {
+                const int8_t *src = (ROUND == R_COARSE_SUB ? sb.tab_sub : sb.tab_mid) + (int64_t)cur * NCOARSE;
+                for (int x = threadIdx.x; x < NCOARSE; x += CT) t1[x] = src[x];
+                __syncthreads();
+            }
+        }
+        if (!busy) continue;  // no target of this series needs this round
+        const uint64_t cells = (uint64_t)(w.b_hi - w.b_lo) * DB * (uint64_t)(w.r_hi - w.r_lo);
+        if (acc + cells > 0xffffffffull) flush();  // 32-bit bins stay exact
+        acc += cells;
+
+        unsigned long long *gbins =
+            reinterpret_cast<unsigned long long *>(sb.hist + (int64_t)cur * sb.hstride + NCOARSE);
+        const uint32_t sink_a = static_cast<uint32_t>(__cvta_generic_to_shared(&sink[lane]));
+        const uint32_t h_a = static_cast<uint32_t>(__cvta_generic_to_shared(h));
+        Src src;
+        src.init(a.y + sd.off, sd, lane, win);
+        auto bands = [&](auto &&f) {
+            for (;;) {
+                // bands are handed to warps one at a time, so no warp idles
+                // while another still has several bands of the unit left
+                int b = 0;
+                if (lane == 0) b = atomicAdd(&next_band, 1);
+                b = __shfl_sync(FULL, b, 0);
+                if (b >= w.b_hi) break;
+                walk_keys(src, sd.ne, 1 + b * DB, w.r_lo, w.r_hi, lane, f);
+            }
+        };
+        // keys of finite or NaN distances have bit 31 clear, so key >> 20
+        // indexes the 2048-entry tables
+        if (ROUND == R_COARSE) {
+            bands([&](uint32_t key, bool valid) {
+                red_shared(valid ? h_a + ((key >> COARSE_SHIFT) << 2) : sink_a);
+            });
+        } else if (dense && ROUND != R_FINAL) {
+            bands([&](uint32_t key, bool valid) {
+                const int q = __viaddmin_s32_relu((int)(key >> 10), qoff, qtop);
+                red_shared(valid ? h_a + ((uint32_t)q << 2) : sink_a);
+            });
+        } else if (ROUND == R_COARSE_SUB) {
+            const uint32_t clo = klo >> COARSE_SHIFT;
+            bands([&](uint32_t key, bool valid) {
+                below += (valid && key < klo) ? 1u : 0u;
+                const uint32_t c = key >> COARSE_SHIFT;
+                const int g = t1[c];
+                const uint32_t fine = (key >> 10) & (NFINE - 1);
+                const bool in = valid && key - klo <= kspan;
+                const uint32_t bin = g < 0 ? c - clo : SUB_WIN + (uint32_t)g * NFINE + fine;
+                if (in && g < 0 && bin >= (uint32_t)SUB_WIN)  // a range of over 64 octaves: never seen
+                    atomicAdd(gbins - NCOARSE + c, 1ull);
+                else
+                    red_shared(in ? h_a + (bin << 2) : sink_a);
+            });
+        } else if (ROUND == R_MID) {
+            const uint32_t top = (uint32_t)nfine / NFINE - 1u;
+            bands([&](uint32_t key, bool valid) {
+                // groups outside this launch's window [g0, g0 + gn) wait for another
+                const uint32_t gw = (uint32_t)((int)t1[key >> COARSE_SHIFT] - a.g0);
+                const uint32_t fine = (key >> 10) & (NFINE - 1);
+                red_shared(valid && gw <= top ? h_a + ((gw * NFINE + fine) << 2) : sink_a);
+            });
+        } else if (dense) {
+            bands([&](uint32_t key, bool valid) {
+                const int q = __viaddmin_s32_relu((int)(key >> 10), qoff, qtop);
+                const uint32_t g = t8[q];
+                if (valid && g)  // rare
+                    atomicAdd(gbins + (int64_t)(g - 1) * NFINE + (key & (NFINE - 1)), 1ull);
+            });
+        } else if (hmul) {
+            bands([&](uint32_t key, bool valid) {
+                // empty slots hold group 0 with prefix 0x1fffff, which only a
+                // NaN key (already an error) can match, inside group 0's bins
+                const uint32_t p = key >> 10;
+                const uint32_t e = th[(p * hmul) >> (32 - NHASH_BITS)];
+                if (valid && ((e ^ p) & 0x1FFFFFu) == 0u)  // rare
+                    atomicAdd(gbins + (int64_t)(e >> 21) * NFINE + (key & (NFINE - 1)), 1ull);
+            });
+        } else {
+            const int np = n_pfx;
+            bands([&](uint32_t key, bool valid) {
+                const uint32_t p = key >> 10;
+                int lo = 0, hi = np;  // first prefix >= p
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (pfx[mid] < p) lo = mid + 1;
+                    else hi = mid;
+                }
+                if (valid && lo < np && pfx[lo] == p)
+                    atomicAdd(gbins + (int64_t)lo * NFINE + (key & (NFINE - 1)), 1ull);
+            });
         }
     }
+    flush();
 }
 
 template <int ROUND>
@@ -283,29 +329,26 @@ static cudaError_t launch_count_m(const CellArgs &a, const SelBufs &sb, int K, i
                                   int embed, cudaStream_t st)
 {
     const int smem = count_smem_bytes(ROUND, K);
-    void (*kern)(CellArgs, SelBufs, int);
+    void (*kern)(CellArgs, SelBufs, int, int);
     switch (embed) {
-    case E_M1T1: kern = k_count<ROUND, 1, 1>; break;
-    case E_M3T1: kern = k_count<ROUND, 3, 1>; break;
-    case E_M3T3: kern = k_count<ROUND, 3, 3>; break;
-    case E_M1: kern = k_count<ROUND, 1, 0>; break;
-    case E_M2: kern = k_count<ROUND, 2, 0>; break;
-    case E_M3: kern = k_count<ROUND, 3, 0>; break;
-    case E_M4: kern = k_count<ROUND, 4, 0>; break;
-    default: kern = k_count<ROUND, 0, 0>; break;
+    case E_M1T1: kern = k_count<ROUND, DiagSrc<1, 1>>; break;
+    case E_M3T1: kern = k_count<ROUND, DiagSrc<3, 1>>; break;
+    case E_M3T3: kern = k_count<ROUND, DiagSrc<3, 3>>; break;
+    default: kern = k_count<ROUND, GenSrc>; break;
     }
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    grid = persistent_cap(reinterpret_cast<const void *>(kern), smem, grid, count_threads(ROUND));
-    kern<<<grid, count_threads(ROUND), smem, st>>>(a, sb, K);
+    grid = persistent_cap(reinterpret_cast<const void *>(kern), smem, grid, CT);
+    kern<<<grid, CT, smem, st>>>(a, sb, K, count_bins(ROUND, K));
     return cudaGetLastError();
 }
 
 cudaError_t launch_count(int round, const CellArgs &a, const SelBufs &sb, int K, int grid,
                          int embed, cudaStream_t st)
 {
-    if (!a.y || !a.series || !a.items || !a.queue || !a.status || !sb.hist || K < 1 || K > KMAX ||
-        grid < 1 || a.n_items < 1 || a.band != BAND)
+    if (!a.y || !a.series || !a.order || !a.uprefix || !a.queue || !a.status || !sb.hist || K < 1 ||
+        K > KMAX || grid < 1 || a.n_units < 1 || a.n_units > 0x7fffffff || a.n_pos < 1 || a.nb < 1 ||
+        a.rc < RB || a.rc % RB)
         return cudaErrorInvalidValue;
     if (round == R_MID && (a.g0 < 0 || a.gn < 1 || a.gn > MID_GROUPS)) return cudaErrorInvalidValue;
     switch (round) {
@@ -317,11 +360,14 @@ cudaError_t launch_count(int round, const CellArgs &a, const SelBufs &sb, int K,
 }
 
 // ------------------------------------------------------------ selection
+constexpr int ST = 512;  // threads per series
+constexpr int SW = ST / 32;
+
 // In-place inclusive scan of n 64-bit values in shared memory (n a multiple
-// of THREADS).
+// of ST).
 __device__ void block_scan_u64(uint64_t *v, int n, uint64_t *warp_tot)
 {
-    const int per = n / THREADS;
+    const int per = n / ST;
     const int t = threadIdx.x;
     uint64_t s = 0;
     for (int x = 0; x < per; ++x) {
@@ -355,66 +401,134 @@ __device__ __forceinline__ int lower_bound_u64(const uint64_t *a, int n, uint64_
     return lo;
 }
 
-// Load the NFINE bins of fine group g of series s and scan them.
-__device__ void load_scan_group(const uint64_t *gh_fine, int g, uint64_t *cum, uint64_t *wt)
+__device__ __forceinline__ uint64_t warp_scan_u64(uint64_t v, int lane)
 {
-    const uint64_t *src = gh_fine + (int64_t)g * NFINE;
-    for (int x = threadIdx.x; x < NFINE; x += THREADS) cum[x] = src[x];
-    __syncthreads();
-    block_scan_u64(cum, NFINE, wt);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t u = __shfl_up_sync(FULL, v, o);
+        if (lane >= o) v += u;
+    }
+    return v;
 }
 
-// One CTA per series.  ROUND is the counting round whose histogram is read.
-template <int ROUND>
-__global__ void __launch_bounds__(THREADS)
-k_select(SelBufs sb, const SeriesDev *series, int s_begin, int K, float *eps_out,
-         uint64_t *le_out, uint64_t *lt_out, int *status)
+// One warp: the bin x of the NFINE bins at src whose cumulative count first
+// reaches R (NFINE if none), the counts below it and in it.  Two levels of 32,
+// so a target costs two scans and no barrier (a scan of the whole group by
+// the CTA per target took 3 us and four barriers each).
+__device__ __forceinline__ int warp_search(const uint64_t *src, uint64_t R, int lane, uint64_t &below,
+                                           uint64_t &in)
 {
-    __shared__ uint64_t cum[NCOARSE];
-    __shared__ uint64_t wt[WARPS];
-    __shared__ uint32_t pre[KMAX];
-    __shared__ uint8_t lev[KMAX];
-    __shared__ uint64_t rnk[KMAX], blw[KMAX];
-    __shared__ int grp[KMAX];
-    const int s = s_begin + blockIdx.x;
+    static_assert(NFINE == 32 * 32, "two levels of 32");
+    uint64_t seg = 0;  // lane: bins 32 lane .. 32 lane + 31
+    const ulonglong2 *p = reinterpret_cast<const ulonglong2 *>(src) + lane * 16;
+#pragma unroll
+    for (int x = 0; x < 16; ++x) {
+        const ulonglong2 v = p[x];
+        seg += v.x + v.y;
+    }
+    const uint64_t cs = warp_scan_u64(seg, lane);
+    const unsigned hit = __ballot_sync(FULL, cs >= R);
+    below = 0;
+    in = 0;
+    if (!hit) return NFINE;
+    const int sl = __ffs(hit) - 1;
+    const uint64_t base = __shfl_sync(FULL, cs - seg, sl);
+    const uint64_t v = src[32 * sl + lane];
+    const uint64_t cv = base + warp_scan_u64(v, lane);
+    const int bl = __ffs(__ballot_sync(FULL, cv >= R)) - 1;
+    below = __shfl_sync(FULL, cv - v, bl);
+    in = __shfl_sync(FULL, v, bl);
+    return 32 * sl + bl;
+}
+
+// Number of distinct values up to each of the K ascending values v (threads
+// t < K; K <= 128): grp = index of v[t] among them; returns their count.
+__device__ int distinct_groups(const uint32_t *v, int K, int *grp, unsigned *bits)
+{
     const int t = threadIdx.x;
+    if (t < 128) {
+        const bool first = t < K && (t == 0 || v[t] != v[t - 1]);
+        const unsigned b = __ballot_sync(FULL, first);
+        if ((t & 31) == 0) bits[t >> 5] = b;
+    }
+    __syncthreads();
+    int n = 0;
+    for (int w = 0; w < 4; ++w) n += __popc(bits[w]);
+    if (t < K) {
+        int g = __popc(bits[t >> 5] & (0xffffffffu >> (31 - (t & 31)))) - 1;
+        for (int w = 0; w < (t >> 5); ++w) g += __popc(bits[w]);
+        grp[t] = g;
+    }
+    __syncthreads();
+    return n;
+}
+
+// One CTA per series, a warp per target.  ROUND is the counting round whose
+// histogram is read.
+template <int ROUND>
+__global__ void __launch_bounds__(ST)
+k_select(SelBufs sb, int s_begin, int K, float *eps_out, uint64_t *le_out, uint64_t *lt_out, int *status)
+{
+    __shared__ uint64_t cum[ROUND == R_COARSE || ROUND == R_COARSE_SUB ? NCOARSE : 1];
+    __shared__ uint64_t wt[SW];
+    __shared__ uint32_t pre[KMAX + 1];
+    __shared__ uint8_t lev[KMAX + 1];
+    __shared__ uint64_t rnk[KMAX + 1], blw[KMAX + 1];
+    __shared__ int grp[KMAX + 1];
+    __shared__ unsigned bits[4];
+    const int s = s_begin + blockIdx.x;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int64_t sk = (int64_t)s * K;
     const uint64_t *gh = sb.hist + (int64_t)s * sb.hstride;
     const uint64_t *gfine = gh + NCOARSE;
-    (void)series;
+
+    // targets of group grp[k] (>= 0): the middle digit, one warp each
+    auto middle_digit = [&]() {
+        for (int k = warp; k < K; k += SW) {
+            if (grp[k] < 0) continue;
+            uint64_t below, in;
+            const int x = warp_search(gfine + (int64_t)grp[k] * NFINE, rnk[k], lane, below, in);
+            __syncwarp();
+            if (lane == 0) {
+                if (x >= NFINE) {
+                    set_status(status, 10 /*INTERNAL*/);
+                } else {
+                    pre[k] = (pre[k] << 10) | (uint32_t)x;
+                    lev[k] = 2;
+                    rnk[k] -= below;
+                    blw[k] += below;
+                }
+            }
+        }
+        __syncthreads();
+    };
 
     if (ROUND == R_COARSE && !sb.redo[s]) return;  // the bracket settled this series
     if (ROUND == R_COARSE || ROUND == R_COARSE_SUB) {
         __shared__ int hard;  // bracket round: some target outside the bracket
         if (t == 0) hard = 0;
         // bucket totals; a split bucket's keys sit in its fine group
-        for (int x = t; x < NCOARSE; x += THREADS) cum[x] = gh[x];
+        for (int x = t; x < NCOARSE; x += ST) cum[x] = gh[x];
         __syncthreads();
+        const int8_t *tab = ROUND == R_COARSE_SUB ? sb.tab_sub + (int64_t)s * NCOARSE : nullptr;
+        const int nsub = ROUND == R_COARSE_SUB ? sb.n_sub[s] : 0;
         if (ROUND == R_COARSE_SUB) {
             __shared__ int inv[NSUB_MAX];
-            const int nsub = sb.n_sub[s];
-            const int8_t *tab = sb.tab_sub + (int64_t)s * NCOARSE;
             if (t < NSUB_MAX) inv[t] = -1;
             __syncthreads();
-            for (int c = t; c < NCOARSE; c += THREADS) {
+            for (int c = t; c < NCOARSE; c += ST) {
                 const int g = tab[c];
                 if (g >= 0 && g < NSUB_MAX) inv[g] = c;
             }
             __syncthreads();
-            for (int g = 0; g < nsub; ++g) {
+            for (int g = warp; g < nsub; g += SW) {
                 uint64_t part = 0;
-                for (int x = t; x < NFINE; x += THREADS) part += gfine[(int64_t)g * NFINE + x];
+                for (int x = lane; x < NFINE; x += 32) part += gfine[(int64_t)g * NFINE + x];
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(FULL, part, o);
-                if ((t & 31) == 0) wt[t >> 5] = part;
-                __syncthreads();
-                if (t == 0 && inv[g] >= 0) {
-                    uint64_t tot = 0;
-                    for (int w = 0; w < WARPS; ++w) tot += wt[w];
-                    cum[inv[g]] += tot;
-                }
-                __syncthreads();
+                if (lane == 0 && inv[g] >= 0) cum[inv[g]] += part;
             }
+            __syncthreads();
         }
         block_scan_u64(cum, NCOARSE, wt);
         // bracket round: only the bracket's buckets were counted (keys under it
@@ -424,8 +538,7 @@ k_select(SelBufs sb, const SeriesDev *series, int s_begin, int K, float *eps_out
         if (t < K) {
             const uint64_t R = sb.T[sk + t];
             const int c = lower_bound_u64(cum, NCOARSE, R);
-            if (ROUND == R_COARSE_SUB &&
-                (sb.n_sub[s] == 0 || c >= NCOARSE || c < sub_lo || c > sub_hi)) {
+            if (ROUND == R_COARSE_SUB && (nsub == 0 || c >= NCOARSE || c < sub_lo || c > sub_hi)) {
                 pre[t] = 0; lev[t] = 0; rnk[t] = R; blw[t] = 0;  // outside: full selection
                 hard = 1;
             } else if (c >= NCOARSE || R == 0) {
@@ -438,35 +551,11 @@ k_select(SelBufs sb, const SeriesDev *series, int s_begin, int K, float *eps_out
                 rnk[t] = R - below;
                 blw[t] = below;
             }
-            grp[t] = -1;
+            grp[t] = ROUND == R_COARSE_SUB && lev[t] == 1 ? tab[pre[t]] : -1;
         }
         __syncthreads();
         if (ROUND == R_COARSE_SUB) {
-            const int8_t *tab = sb.tab_sub + (int64_t)s * NCOARSE;
-            if (t < K) grp[t] = (lev[t] == 1) ? tab[pre[t]] : -1;
-            __syncthreads();
-            const int nsub = sb.n_sub[s];
-            for (int g = 0; g < nsub; ++g) {
-                bool any = false;
-                for (int k = 0; k < K; ++k) any |= (grp[k] == g);
-                if (!any) continue;
-                load_scan_group(gfine, g, cum, wt);
-                if (t < K && grp[t] == g) {
-                    const int x = lower_bound_u64(cum, NFINE, rnk[t]);
-                    if (x >= NFINE) {
-                        set_status(status, 10);
-                    } else {
-                        const uint64_t below = x ? cum[x - 1] : 0;
-                        pre[t] = (pre[t] << 10) | (uint32_t)x;
-                        lev[t] = 2;
-                        rnk[t] -= below;
-                        blw[t] += below;
-                    }
-                }
-                __syncthreads();
-            }
-        }
-        if (ROUND == R_COARSE_SUB) {
+            middle_digit();
             if (t == 0) sb.redo[s] = (uint8_t)hard;
             if (hard) {  // the plain rounds redo this series; levels kept for the statistics
                 if (t < K) sb.level[sk + t] = lev[t];
@@ -474,21 +563,39 @@ k_select(SelBufs sb, const SeriesDev *series, int s_begin, int K, float *eps_out
             }
         }
         // middle-round table: coarse bucket -> group, for targets at level 1
+        // (ascending buckets).  Buckets that span at most NSUB_MAX make every
+        // bucket of the span a group, so the counting kernel needs no table.
+        __shared__ int n_mid, c_lo, c_hi;
         int8_t *tm = sb.tab_mid + (int64_t)s * NCOARSE;
-        for (int x = t; x < NCOARSE; x += THREADS) tm[x] = -1;
-        __syncthreads();
+        for (int x = t; x < NCOARSE / 4; x += ST) reinterpret_cast<uint32_t *>(tm)[x] = 0xffffffffu;
         if (t == 0) {
-            int g = 0;
-            uint32_t lo = 0xffffffffu, hi = 0u;
-            for (int k = 0; k < K; ++k) {
-                if (lev[k] != 1) continue;
-                if (tm[pre[k]] < 0) tm[pre[k]] = (int8_t)g++;
-                lo = min(lo, pre[k] << COARSE_SHIFT);
-                hi = max(hi, ((pre[k] + 1u) << COARSE_SHIFT) - 1u);
+            int lo = NCOARSE, hi = -1;
+            for (int k = 0; k < K; ++k)
+                if (lev[k] == 1) {
+                    lo = min(lo, (int)pre[k]);
+                    hi = max(hi, (int)pre[k]);
+                }
+            c_lo = lo;
+            c_hi = hi;
+            n_mid = hi < lo ? 0 : hi - lo + 1;
+        }
+        __syncthreads();
+        if (n_mid > 0 && n_mid <= NSUB_MAX) {
+            if (t < n_mid) tm[c_lo + t] = (int8_t)t;
+        } else if (n_mid > 0) {
+            __syncthreads();  // every thread has read n_mid
+            if (t == 0) {
+                int g = 0;
+                for (int k = 0; k < K; ++k)
+                    if (lev[k] == 1 && tm[pre[k]] < 0) tm[pre[k]] = (int8_t)g++;
+                n_mid = g;
             }
-            sb.n_mid[s] = g;
-            sb.range[2 * (int64_t)s] = lo;
-            sb.range[2 * (int64_t)s + 1] = hi;
+            __syncthreads();
+        }
+        if (t == 0) {
+            sb.n_mid[s] = n_mid;
+            sb.range[2 * (int64_t)s] = n_mid ? (uint32_t)c_lo << COARSE_SHIFT : 0xffffffffu;
+            sb.range[2 * (int64_t)s + 1] = n_mid ? (((uint32_t)c_hi + 1u) << COARSE_SHIFT) - 1u : 0u;
         }
         if (t < K) {
             sb.prefix[sk + t] = pre[t];
@@ -512,67 +619,15 @@ k_select(SelBufs sb, const SeriesDev *series, int s_begin, int K, float *eps_out
         const int8_t *tm = sb.tab_mid + (int64_t)s * NCOARSE;
         if (t < K) grp[t] = (lev[t] == 1) ? tm[pre[t]] : -1;
         __syncthreads();
-        const int nmid = sb.n_mid[s];
-        for (int g = 0; g < nmid; ++g) {
-            load_scan_group(gfine, g, cum, wt);
-            if (t < K && grp[t] == g) {
-                const int x = lower_bound_u64(cum, NFINE, rnk[t]);
-                if (x >= NFINE) {
-                    set_status(status, 10);
-                } else {
-                    const uint64_t below = x ? cum[x - 1] : 0;
-                    pre[t] = (pre[t] << 10) | (uint32_t)x;
-                    lev[t] = 2;
-                    rnk[t] -= below;
-                    blw[t] += below;
-                }
-            }
-            __syncthreads();
-        }
-        // final-round tables for all targets (every target is at level 2 now)
-        int8_t *f1 = sb.tab_fin1 + (int64_t)s * NCOARSE;
-        int8_t *f2 = sb.tab_fin2 + (int64_t)s * sb.fin2_stride;
-        uint32_t *fh = sb.tab_hash ? sb.tab_hash + (int64_t)s * NHASH : nullptr;
-        for (int x = t; x < NCOARSE; x += THREADS) f1[x] = -1;
-        for (int x = t; x < K * NFINE; x += THREADS) f2[x] = -1;
-        for (int x = t; fh && x < NHASH; x += THREADS) fh[x] = 0x1fffffu;  // group 0, no finite key
-        __syncthreads();
+        middle_digit();
+        // final round: the distinct prefixes (every target is at level 2 now,
+        // ascending) are its groups, in order
+        const int nfin = distinct_groups(pre, K, grp, bits);
+        const uint32_t lo = pre[0] << 10, hi = ((pre[K - 1] + 1u) << 10) - 1u;
         if (t == 0) {
-            int g1 = 0, g = 0;
-            uint32_t lo = 0xffffffffu, hi = 0u;
-            for (int k = 0; k < K; ++k) {
-                const uint32_t c = pre[k] >> 10, mid = pre[k] & (NFINE - 1);
-                if (f1[c] < 0) f1[c] = (int8_t)g1++;
-                int8_t *e = f2 + f1[c] * NFINE + mid;
-                if (*e < 0) *e = (int8_t)g++;
-                lo = min(lo, pre[k] << 10);
-                hi = max(hi, ((pre[k] + 1u) << 10) - 1u);
-            }
-            sb.n_fin[s] = g;
+            sb.n_fin[s] = nfin;
             sb.range[2 * (int64_t)s] = lo;
             sb.range[2 * (int64_t)s + 1] = hi;
-            // hashed table of the distinct prefixes (group order): the first
-            // odd multiplier of a fixed sequence that puts them in distinct
-            // slots; none among 64 (never seen) keeps the two-level tables
-            if (fh) {
-                uint32_t pg[KMAX];
-                for (int k = 0; k < K; ++k) {
-                    const int gk = f2[f1[pre[k] >> 10] * NFINE + (pre[k] & (NFINE - 1))];
-                    pg[gk] = pre[k];
-                }
-                uint32_t mul = 0;
-                for (int a = 0; a < 64 && !mul; ++a) {
-                    const uint32_t m = (0x9E3779B1u + 0x6A09E668u * (uint32_t)a) | 1u;
-                    bool ok = true;
-                    for (int i = 1; i < g && ok; ++i)
-                        for (int j = 0; j < i && ok; ++j)
-                            ok = ((pg[i] * m) >> (32 - NHASH_BITS)) != ((pg[j] * m) >> (32 - NHASH_BITS));
-                    if (ok) mul = m;
-                }
-                if (mul)
-                    for (int i = 0; i < g; ++i) fh[(pg[i] * mul) >> (32 - NHASH_BITS)] = pg[i] | ((uint32_t)i << 21);
-                sb.hash_mul[s] = mul;
-            }
         }
         if (t < K) {
             sb.prefix[sk + t] = pre[t];
@@ -580,61 +635,66 @@ k_select(SelBufs sb, const SeriesDev *series, int s_begin, int K, float *eps_out
             sb.rank[sk + t] = rnk[t];
             sb.below[sk + t] = blw[t];
         }
+        // hashed table of the prefixes, read when their span exceeds the
+        // counting kernel's byte table: the first odd multiplier of a fixed
+        // sequence that puts them in distinct slots (none among 64: the
+        // kernel searches)
+        if (sb.tab_hash && hi - lo >= (uint32_t)DENSE_FINAL << 10) {
+            uint32_t *fh = sb.tab_hash + (int64_t)s * NHASH;
+            __shared__ uint32_t pg[KMAX + 1];
+            if (t < K) pg[grp[t]] = pre[t];
+            for (int x = t; x < NHASH; x += ST) fh[x] = 0x1fffffu;  // group 0, no finite key
+            __syncthreads();
+            uint32_t mul = 0;
+            for (int at = 0; at < 64 && !mul; ++at) {
+                const uint32_t m = (0x9E3779B1u + 0x6A09E668u * (uint32_t)at) | 1u;
+                bool clash = false;
+                for (int x = t; x < nfin * nfin; x += ST) {
+                    const int i = x / nfin, j = x - i * nfin;
+                    clash |= j < i && ((pg[i] * m) >> (32 - NHASH_BITS)) == ((pg[j] * m) >> (32 - NHASH_BITS));
+                }
+                if (!__syncthreads_or(clash)) mul = m;
+            }
+            if (mul && t < nfin) fh[(pg[t] * mul) >> (32 - NHASH_BITS)] = pg[t] | ((uint32_t)t << 21);
+            if (t == 0) sb.hash_mul[s] = mul;
+        }
         return;
     }
 
     // R_FINAL: the low digit completes the key
-    {
-        const int8_t *f1 = sb.tab_fin1 + (int64_t)s * NCOARSE;
-        const int8_t *f2 = sb.tab_fin2 + (int64_t)s * sb.fin2_stride;
-        if (t < K) {
-            const int g1 = f1[pre[t] >> 10];
-            grp[t] = (g1 < 0) ? -1 : f2[g1 * NFINE + (pre[t] & (NFINE - 1))];
-            if (grp[t] < 0) set_status(status, 10);
-        }
-        __syncthreads();
-        const int nfin = sb.n_fin[s];
-        for (int g = 0; g < nfin; ++g) {
-            load_scan_group(gfine, g, cum, wt);
-            if (t < K && grp[t] == g) {
-                const int x = lower_bound_u64(cum, NFINE, rnk[t]);
-                if (x >= NFINE) {
-                    set_status(status, 10);
-                } else {
-                    const uint64_t lt = blw[t] + (x ? cum[x - 1] : 0);
-                    const uint64_t le = blw[t] + cum[x];
-                    const uint32_t key = (pre[t] << 10) | (uint32_t)x;
-                    eps_out[sk + t] = __uint_as_float(key);
-                    if (le_out) le_out[sk + t] = le;
-                    if (lt_out) lt_out[sk + t] = lt;
-                }
+    distinct_groups(pre, K, grp, bits);
+    for (int k = warp; k < K; k += SW) {
+        uint64_t below, in;
+        const int x = warp_search(gfine + (int64_t)grp[k] * NFINE, rnk[k], lane, below, in);
+        if (lane == 0) {
+            if (x >= NFINE) {
+                set_status(status, 10);
+            } else {
+                const uint64_t lt = blw[k] + below;
+                eps_out[sk + k] = __uint_as_float((pre[k] << 10) | (uint32_t)x);
+                if (le_out) le_out[sk + k] = lt + in;
+                if (lt_out) lt_out[sk + k] = lt;
             }
-            __syncthreads();
         }
     }
 }
 
-cudaError_t launch_select(int round, const SelBufs &sb, const SeriesDev *series, int s_begin,
-                          int n_series, int K, float *eps_out, uint64_t *le_out,
-                          uint64_t *lt_out, int *status, cudaStream_t st)
+cudaError_t launch_select(int round, const SelBufs &sb, int s_begin, int n_series, int K, float *eps_out,
+                          uint64_t *le_out, uint64_t *lt_out, int *status, cudaStream_t st)
 {
     if (n_series <= 0) return cudaSuccess;
     switch (round) {
     case R_COARSE:
-        k_select<R_COARSE><<<n_series, THREADS, 0, st>>>(sb, series, s_begin, K, eps_out, le_out,
-                                                          lt_out, status);
+        k_select<R_COARSE><<<n_series, ST, 0, st>>>(sb, s_begin, K, eps_out, le_out, lt_out, status);
         break;
     case R_COARSE_SUB:
-        k_select<R_COARSE_SUB><<<n_series, THREADS, 0, st>>>(sb, series, s_begin, K, eps_out,
-                                                              le_out, lt_out, status);
+        k_select<R_COARSE_SUB><<<n_series, ST, 0, st>>>(sb, s_begin, K, eps_out, le_out, lt_out, status);
         break;
     case R_MID:
-        k_select<R_MID><<<n_series, THREADS, 0, st>>>(sb, series, s_begin, K, eps_out, le_out,
-                                                       lt_out, status);
+        k_select<R_MID><<<n_series, ST, 0, st>>>(sb, s_begin, K, eps_out, le_out, lt_out, status);
         break;
     default:
-        k_select<R_FINAL><<<n_series, THREADS, 0, st>>>(sb, series, s_begin, K, eps_out, le_out,
-                                                         lt_out, status);
+        k_select<R_FINAL><<<n_series, ST, 0, st>>>(sb, s_begin, K, eps_out, le_out, lt_out, status);
         break;
     }
     return cudaGetLastError();
