@@ -129,22 +129,34 @@ k_count_grid(CellArgs a, const float *__restrict__ thr, int n_thr, uint64_t *his
                 walk_keys(src, sd.ne, 1 + b * DB, w.r_lo, w.r_hi, lane, f);
             }
         };
+        auto count = [&](auto &&bin) {  // bin(key): r + 1
+            bands([&](const float (&d)[4][DPL], auto valid) {
+                uint32_t r1[4][DPL];
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int j = 0; j < DPL; ++j) r1[r][j] = bin(__float_as_uint(d[r][j]));
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int j = 0; j < DPL; ++j) red_shared(valid(r, j) ? h_a + (r1[r][j] << 2) : sink_a);
+            });
+        };
         if (uni) {
-            bands([&](uint32_t key, bool valid) {
+            count([&](uint32_t key) -> uint32_t {
                 const float f = fmaf(__uint_as_float(key), inv, 8388608.f);
                 const int rho = __viaddmin_s32_relu((int)__float_as_uint(f), -0x4B000000, n_thr);
-                const uint32_t r1 = (uint32_t)rho + (tk[rho] < key ? 1u : 0u);
-                red_shared(valid ? h_a + (r1 << 2) : sink_a);
+                return (uint32_t)rho + (tk[rho] < key ? 1u : 0u);
             });
         } else {
-            bands([&](uint32_t key, bool valid) {
+            count([&](uint32_t key) -> uint32_t {
                 int lo = 0, hi = n_thr;  // grid keys below key (ascending)
                 while (lo < hi) {
                     const int mid = (lo + hi) >> 1;
                     if (tk[mid + 1] < key) lo = mid + 1;
                     else hi = mid;
                 }
-                red_shared(valid ? h_a + ((uint32_t)(lo + 1) << 2) : sink_a);
+                return (uint32_t)lo + 1u;
             });
         }
     }

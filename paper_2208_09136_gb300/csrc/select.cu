@@ -97,7 +97,7 @@ int count_smem_bytes(int round, int K)
 // instructions per cell (32 cells: per warp).  Units are row chunks of a few
 // bands (dense.cuh), so a batch of four 10^4-value series fills the chip.
 template <int ROUND, class Src>
-__global__ void __launch_bounds__(CT) k_count(CellArgs a, SelBufs sb, int K, int nbins)
+__global__ void __launch_bounds__(CT, 2) k_count(CellArgs a, SelBufs sb, int K, int nbins)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ Unit unit;
@@ -257,20 +257,29 @@ __global__ void __launch_bounds__(CT) k_count(CellArgs a, SelBufs sb, int K, int
                 walk_keys(src, sd.ne, 1 + b * DB, w.r_lo, w.r_hi, lane, f);
             }
         };
+        // f(key, ok) for the sixteen cells of a step, one after the other
+        auto each = [&](auto &&f) {
+            bands([&](const float (&d)[4][DPL], auto valid) {
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int j = 0; j < DPL; ++j) f(__float_as_uint(d[r][j]), valid(r, j));
+            });
+        };
         // keys of finite or NaN distances have bit 31 clear, so key >> 20
         // indexes the 2048-entry tables
         if (ROUND == R_COARSE) {
-            bands([&](uint32_t key, bool valid) {
+            each([&](uint32_t key, bool valid) {
                 red_shared(valid ? h_a + ((key >> COARSE_SHIFT) << 2) : sink_a);
             });
         } else if (dense && ROUND != R_FINAL) {
-            bands([&](uint32_t key, bool valid) {
+            each([&](uint32_t key, bool valid) {
                 const int q = __viaddmin_s32_relu((int)(key >> 10), qoff, qtop);
                 red_shared(valid ? h_a + ((uint32_t)q << 2) : sink_a);
             });
         } else if (ROUND == R_COARSE_SUB) {
             const uint32_t clo = klo >> COARSE_SHIFT;
-            bands([&](uint32_t key, bool valid) {
+            each([&](uint32_t key, bool valid) {
                 below += (valid && key < klo) ? 1u : 0u;
                 const uint32_t c = key >> COARSE_SHIFT;
                 const int g = t1[c];
@@ -284,41 +293,71 @@ __global__ void __launch_bounds__(CT) k_count(CellArgs a, SelBufs sb, int K, int
             });
         } else if (ROUND == R_MID) {
             const uint32_t top = (uint32_t)nfine / NFINE - 1u;
-            bands([&](uint32_t key, bool valid) {
+            bands([&](const float (&d)[4][DPL], auto valid) {
                 // groups outside this launch's window [g0, g0 + gn) wait for another
-                const uint32_t gw = (uint32_t)((int)t1[key >> COARSE_SHIFT] - a.g0);
-                const uint32_t fine = (key >> 10) & (NFINE - 1);
-                red_shared(valid && gw <= top ? h_a + ((gw * NFINE + fine) << 2) : sink_a);
-            });
-        } else if (dense) {
-            bands([&](uint32_t key, bool valid) {
-                const int q = __viaddmin_s32_relu((int)(key >> 10), qoff, qtop);
-                const uint32_t g = t8[q];
-                if (valid && g)  // rare
-                    atomicAdd(gbins + (int64_t)(g - 1) * NFINE + (key & (NFINE - 1)), 1ull);
-            });
-        } else if (hmul) {
-            bands([&](uint32_t key, bool valid) {
-                // empty slots hold group 0 with prefix 0x1fffff, which only a
-                // NaN key (already an error) can match, inside group 0's bins
-                const uint32_t p = key >> 10;
-                const uint32_t e = th[(p * hmul) >> (32 - NHASH_BITS)];
-                if (valid && ((e ^ p) & 0x1FFFFFu) == 0u)  // rare
-                    atomicAdd(gbins + (int64_t)(e >> 21) * NFINE + (key & (NFINE - 1)), 1ull);
+                uint32_t gw[4][DPL];
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int j = 0; j < DPL; ++j)
+                        gw[r][j] = (uint32_t)((int)t1[__float_as_uint(d[r][j]) >> COARSE_SHIFT] - a.g0);
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int j = 0; j < DPL; ++j) {
+                        const uint32_t fine = (__float_as_uint(d[r][j]) >> 10) & (NFINE - 1);
+                        red_shared(valid(r, j) && gw[r][j] <= top ? h_a + ((gw[r][j] * NFINE + fine) << 2) : sink_a);
+                    }
             });
         } else {
-            const int np = n_pfx;
-            bands([&](uint32_t key, bool valid) {
-                const uint32_t p = key >> 10;
-                int lo = 0, hi = np;  // first prefix >= p
-                while (lo < hi) {
-                    const int mid = (lo + hi) >> 1;
-                    if (pfx[mid] < p) lo = mid + 1;
-                    else hi = mid;
-                }
-                if (valid && lo < np && pfx[lo] == p)
-                    atomicAdd(gbins + (int64_t)lo * NFINE + (key & (NFINE - 1)), 1ull);
-            });
+            // final round: hit[r][j] = group + 1 of a target's key, 0 for all
+            // others; one branch per sixteen cells around the rare hits
+            auto finals = [&](auto &&look) {
+                bands([&](const float (&d)[4][DPL], auto valid) {
+                    uint32_t hit[4][DPL], any = 0;
+#pragma unroll
+                    for (int r = 0; r < 4; ++r)
+#pragma unroll
+                        for (int j = 0; j < DPL; ++j) hit[r][j] = look(__float_as_uint(d[r][j]));
+#pragma unroll
+                    for (int r = 0; r < 4; ++r)
+#pragma unroll
+                        for (int j = 0; j < DPL; ++j) any |= hit[r][j];
+                    if (any == 0u) return;
+#pragma unroll
+                    for (int r = 0; r < 4; ++r)
+#pragma unroll
+                        for (int j = 0; j < DPL; ++j)
+                            if (valid(r, j) && hit[r][j])
+                                atomicAdd(gbins + (int64_t)(hit[r][j] - 1) * NFINE +
+                                              (__float_as_uint(d[r][j]) & (NFINE - 1)), 1ull);
+                });
+            };
+            if (dense) {
+                finals([&](uint32_t key) -> uint32_t {
+                    return t8[__viaddmin_s32_relu((int)(key >> 10), qoff, qtop)];
+                });
+            } else if (hmul) {
+                finals([&](uint32_t key) -> uint32_t {
+                    // empty slots hold group 0 with prefix 0x1fffff, which only a
+                    // NaN key (already an error) can match, inside group 0's bins
+                    const uint32_t p = key >> 10;
+                    const uint32_t e = th[(p * hmul) >> (32 - NHASH_BITS)];
+                    return ((e ^ p) & 0x1FFFFFu) == 0u ? (e >> 21) + 1u : 0u;
+                });
+            } else {
+                const int np = n_pfx;
+                finals([&](uint32_t key) -> uint32_t {
+                    const uint32_t p = key >> 10;
+                    int lo = 0, hi = np;  // first prefix >= p
+                    while (lo < hi) {
+                        const int mid = (lo + hi) >> 1;
+                        if (pfx[mid] < p) lo = mid + 1;
+                        else hi = mid;
+                    }
+                    return lo < np && pfx[lo] == p ? (uint32_t)lo + 1u : 0u;
+                });
+            }
         }
     }
     flush();
