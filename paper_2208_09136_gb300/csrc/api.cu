@@ -24,11 +24,30 @@ Split split_cells(uint64_t cells, int nb, int sm_count)
     return Split{nb, ROW_BLOCK * (int)std::min<uint64_t>(std::max<uint64_t>(blocks, 8), 585)};
 }
 
-int64_t units_of_series(int64_t ne, const Split &sp, bool vert)
+Split split_lines(uint64_t cells, int64_t bands, int32_t ne_max, int unit_bands, int sm_count)
+{
+    const int64_t warps = (int64_t)sm_count * 16;
+    const int64_t cap = std::max<int64_t>(1, ((int64_t)1 << 28) / std::max(ne_max, 1));
+    const int32_t whole = (std::max(ne_max, 1) + 31) / 32 * 32;  // rows of the longest band
+    Split sp{};
+    if (bands >= 8 * warps) {
+        sp.nb = (int)std::min<int64_t>(64, bands / (8 * warps));
+        sp.rc = whole;
+    } else {
+        sp.nb = 1;
+        const uint64_t blocks = cells / ((uint64_t)LINE_BAND * 32 * (uint64_t)warps * 4);
+        sp.rc = (int)std::min<uint64_t>(32 * std::max<uint64_t>(blocks, 8), (uint64_t)whole);
+    }
+    if (unit_bands > 0) sp.nb = unit_bands;  // a tuned size
+    sp.nb = (int)std::min<int64_t>(sp.nb, cap);
+    return sp;
+}
+
+int64_t units_of_series(int64_t ne, const Split &sp, bool vert, int w)
 {
     int64_t n = 0;
     for (int64_t r = 0; r < ne; r += sp.rc) {
-        const int64_t bands = vert ? (ne + DB - 1) / DB : (ne - 1 - r + DB - 1) / DB;
+        const int64_t bands = vert ? (ne + w - 1) / w : (ne - 1 - r + w - 1) / w;
         n += (bands + sp.nb - 1) / sp.nb;
     }
     return n;
@@ -88,7 +107,7 @@ struct rqa_ctx {
     DevBuf prefix, level, rank, below, tab_sub, tab_mid, tab_hash, ngroups, hist, krange,
         redo;
     DevBuf queue, status;
-    DevBuf eps_tmp, le_tmp, lt_tmp, count, lmax, hshort;
+    DevBuf eps_tmp, le_tmp, lt_tmp, count, lmax, hshort, edges;
     DevBuf meas;  // per-target L / ENTR when only their averages are asked for
     DevBuf grid_thr, grid_hist, grid_rr;  // the approximate grid search
 
@@ -135,13 +154,13 @@ struct Plan {
     Split split{};                           // cell-walk units of the batch ...
     std::vector<Split> split1;               // ... and of each series alone
     std::vector<int64_t> cprefix, cprefix1;  // their unit-count prefixes, as uprefix / uprefix1
+    Split lsplit{};                          // line-pass units of the batch ...
+    std::vector<Split> lsplit1;              // ... and of each series alone
     std::vector<int64_t> uprefix;            // S+1 unit-count prefix along order
-    int32_t chunk = 1;                       // bands per line-pass unit (batched)
     int32_t line_tile = LINE_TILE_DEFAULT;   // diagonals per register window of the line pass
     int32_t ne_max = 0;                      // largest Ne of the batch
     std::vector<int32_t> ident;              // 0..S-1
     std::vector<int64_t> uprefix1;           // [2s], [2s+1] = 0, units of s alone
-    std::vector<int32_t> chunk1;             // bands per unit of s alone
     std::vector<uint8_t> dom;                // 1: the series may be bracketed
     bool any_dom = false;
     // device pointers into the arena after upload
@@ -216,8 +235,9 @@ int persistent_grid(rqa_ctx *c, size_t n_items)
     return (int)std::max<size_t>(1, std::min(g, n_items));
 }
 
+// vert: the line-pass units are those of the vertical pass.
 int make_plan(rqa_ctx *c, const rqa_batch *b, const int32_t *rr_num, int32_t rr_den, int K,
-              Plan &pl)
+              Plan &pl, bool vert = false)
 {
     const int S = b->n_series;
     pl.y = b->y;
@@ -275,42 +295,32 @@ int make_plan(rqa_ctx *c, const rqa_batch *b, const int32_t *rr_num, int32_t rr_
     pl.split1.resize(S);
     pl.cprefix.assign(S + 1, 0);
     pl.cprefix1.assign(2 * (size_t)S, 0);
-    // warp work units (line pass): runs of `chunk` bands of LINE_BAND
-    // diagonals, series largest first; about eight units per warp so the tail
-    // stays short while each unit's histogram flush is spread over many cells.
-    // A unit covers at most 2^33 cells, so the warp's 32-bit counts of lines of
-    // length >= 4 (each line and the cell after it: >= 5 cells) stay exact.
-    const int64_t n_warps = (int64_t)c->sm_count * 16;  // resident warps of the line pass
     for (int s = 0; s < S; ++s) pl.ne_max = std::max(pl.ne_max, pl.sd[s].ne);
-    const int64_t chunk_cap = std::max<int64_t>(1, ((int64_t)1 << 28) / std::max(pl.ne_max, 1));
-    auto chunk_for = [&](int64_t bands) {
-        int64_t ch = std::max<int64_t>(1, std::min<int64_t>(64, bands / (n_warps * 8)));
-        if (c->unit_bands > 0) ch = c->unit_bands;  // a tuned size
-        return (int32_t)std::min(ch, chunk_cap);
-    };
     pl.line_tile = c->line_tile ? c->line_tile : LINE_TILE_DEFAULT;
     if (!lines_tile_ok(pl.mt, pl.line_tile)) pl.line_tile = LINE_TILE_DEFAULT;
-    auto nbl = [&](int s) { return (int64_t)(pl.sd[s].ne - 1 + LINE_BAND - 1) / LINE_BAND; };
+    // warp work units of the line pass
+    auto nbl = [&](int s) { return ((int64_t)pl.sd[s].ne - (vert ? 0 : 1) + LINE_BAND - 1) / LINE_BAND; };
+    auto cells_of = [&](uint64_t P) { return vert ? 2 * P : P; };
     int64_t total_bands = 0;
     for (int s = 0; s < S; ++s) total_bands += nbl(s);
-    pl.chunk = chunk_for(total_bands);
+    pl.lsplit = split_lines(cells_of(total_cells), total_bands, pl.ne_max, c->unit_bands, c->sm_count);
+    pl.lsplit1.resize(S);
     pl.order.resize(S);
     for (int s = 0; s < S; ++s) pl.order[s] = s;
     std::stable_sort(pl.order.begin(), pl.order.end(),
                      [&](int x, int y) { return pl.sd[x].P > pl.sd[y].P; });
     pl.uprefix.assign(S + 1, 0);
     for (int i = 0; i < S; ++i) {
-        pl.uprefix[i + 1] = pl.uprefix[i] + (nbl(pl.order[i]) + pl.chunk - 1) / pl.chunk;
+        pl.uprefix[i + 1] = pl.uprefix[i] + units_of_series(pl.sd[pl.order[i]].ne, pl.lsplit, vert, LINE_BAND);
         pl.cprefix[i + 1] = pl.cprefix[i] + units_of_series(pl.sd[pl.order[i]].ne, pl.split, false);
     }
     pl.ident.resize(S);
     pl.uprefix1.resize(2 * (size_t)S);
-    pl.chunk1.resize(S);
     for (int s = 0; s < S; ++s) {
         pl.ident[s] = s;
-        pl.chunk1[s] = chunk_for(nbl(s));
+        pl.lsplit1[s] = split_lines(cells_of(pl.sd[s].P), nbl(s), pl.sd[s].ne, c->unit_bands, c->sm_count);
         pl.uprefix1[2 * s] = 0;
-        pl.uprefix1[2 * s + 1] = (nbl(s) + pl.chunk1[s] - 1) / pl.chunk1[s];
+        pl.uprefix1[2 * s + 1] = units_of_series(pl.sd[s].ne, pl.lsplit1[s], vert, LINE_BAND);
         pl.split1[s] = split_cells(pl.sd[s].P, COUNT_NB, c->sm_count);
         pl.cprefix1[2 * s + 1] = units_of_series(pl.sd[s].ne, pl.split1[s], false);
     }
@@ -441,20 +451,30 @@ int reset_queue(rqa_ctx *c, int n, unsigned **q)
     return RQA_OK;
 }
 
-// The cell-walk units of the whole batch, or of series s alone (s >= 0).
-CellArgs cell_args(rqa_ctx *c, const Plan &pl, int s)
+// The cell-walk units of the whole batch, or of series s alone (s >= 0);
+// lines: those of the line pass.
+CellArgs cell_args(rqa_ctx *c, const Plan &pl, int s, bool lines = false)
 {
     CellArgs a{};
     a.y = pl.y;
     a.series = pl.d_sd;
     a.status = P<int>(c->status);
-    const Split sp = s < 0 ? pl.split : pl.split1[s];
+    const Split sp = lines ? (s < 0 ? pl.lsplit : pl.lsplit1[s]) : (s < 0 ? pl.split : pl.split1[s]);
     a.nb = sp.nb;
     a.rc = sp.rc;
     a.order = s < 0 ? pl.d_order : pl.d_ident + s;
-    a.uprefix = s < 0 ? pl.d_cprefix : pl.d_cprefix1 + 2 * (size_t)s;
     a.n_pos = s < 0 ? pl.S : 1;
-    a.n_units = s < 0 ? pl.cprefix[pl.S] : pl.cprefix1[2 * (size_t)s + 1];
+    if (s < 0) {
+        a.uprefix = lines ? pl.d_uprefix : pl.d_cprefix;
+        a.n_units = (lines ? pl.uprefix : pl.cprefix)[pl.S];
+    } else {
+        a.uprefix = (lines ? pl.d_uprefix1 : pl.d_cprefix1) + 2 * (size_t)s;
+        a.n_units = (lines ? pl.uprefix1 : pl.cprefix1)[2 * (size_t)s + 1];
+    }
+    a.line_tile = pl.line_tile;
+    a.line_ctas = c->line_ctas;
+    a.line_stage = c->line_stage;
+    a.y_len = pl.total;
     return a;
 }
 
@@ -559,10 +579,21 @@ int select_all(rqa_ctx *c, const rqa_batch *b, Plan &pl, float *eps, uint64_t *l
     return run_select(c, pl, sb, cell_args(c, pl, -1), 0, pl.S, q, eps, le, lt, bracket);
 }
 
-int ensure_line_bufs(rqa_ctx *c, int S, int K)
+int ensure_line_bufs(rqa_ctx *c, const Plan &pl)
 {
-    const size_t sk = (size_t)S * K;
+    const int K = pl.K;
+    const size_t sk = (size_t)pl.S * K;
     int rc = RQA_OK;
+    // lines at row-chunk boundaries: a slot per unit and band of one launch
+    int64_t slots = 0;
+    if (c->schedule != RQA_SCHED_PER_SERIES) {
+        if (pl.lsplit.rc < pl.ne_max) slots = pl.uprefix[pl.S] * pl.lsplit.nb;
+    } else {
+        for (int s = 0; s < pl.S; ++s)
+            if (pl.lsplit1[s].rc < pl.sd[s].ne)
+                slots = std::max(slots, pl.uprefix1[2 * (size_t)s + 1] * pl.lsplit1[s].nb);
+    }
+    if ((rc = ensure(c->edges, (size_t)slots * LINE_EDGE_BYTES))) return rc;
     if ((rc = ensure(c->count, sk * 8))) return rc;
     if ((rc = ensure(c->lmax, sk * 4))) return rc;
     if ((rc = ensure(c->hshort, sk * LSH * 8))) return rc;
@@ -586,14 +617,6 @@ int run_lines(rqa_ctx *c, const Plan &pl, const float *eps, uint64_t *hist, cons
     if (int rc = check_cuda(cudaMemsetAsync(lb.count, 0, sk * 8, c->stream))) return rc;
     if (int rc = check_cuda(cudaMemsetAsync(lb.lmax, 0, sk * 4, c->stream))) return rc;
     if (int rc = check_cuda(cudaMemsetAsync(lb.hshort, 0, sk * LSH * 8, c->stream))) return rc;
-    CellArgs a{};
-    a.y = pl.y;
-    a.series = pl.d_sd;
-    a.line_tile = pl.line_tile;
-    a.line_ctas = c->line_ctas;
-    a.line_stage = c->line_stage;
-    a.y_len = pl.total;
-    a.status = P<int>(c->status);
     unsigned *q = nullptr;
     const int full_grid = persistent_grid(c, (size_t)1 << 30);
     auto grid_for = [&](int64_t units) {
@@ -601,38 +624,28 @@ int run_lines(rqa_ctx *c, const Plan &pl, const float *eps, uint64_t *hist, cons
     };
     // targets in groups of at most LINE_KMAX (one lane each), one pass per group
     const int ng = line_groups(K), gsz = (K + ng - 1) / ng;
-    auto launch_groups = [&]() -> int {
+    auto launch_groups = [&](CellArgs a, bool chunks) -> int {
         for (int g = 0; g < ng; ++g) {
             lb.k0 = g * gsz;
             a.queue = q;
             q += 16;
             const int kg = std::min(gsz, K - lb.k0);
             const int grid = grid_for(a.n_units);
-            if (int rc = launched(c, vert ? launch_vlines(a, lb, kg, grid, pl.mt, c->stream)
-                                          : launch_lines(a, lb, kg, grid, pl.mt, c->stream)))
+            if (int rc = launched(c, launch_lines(a, lb, kg, grid, pl.mt, vert, chunks,
+                                                  P<uint32_t>(c->edges), c->stream)))
                 return rc;
+            c->launches += chunks ? 1 : 0;
         }
         return RQA_OK;
     };
     int rc = RQA_OK;
     if (c->schedule == RQA_SCHED_PER_SERIES) {
         if ((rc = reset_queue(c, S * ng, &q))) return rc;
-        for (int s = 0; s < S && rc == RQA_OK; ++s) {
-            a.order = pl.d_ident + s;
-            a.uprefix = pl.d_uprefix1 + 2 * (size_t)s;
-            a.n_pos = 1;
-            a.chunk = pl.chunk1[s];
-            a.n_units = pl.uprefix1[2 * (size_t)s + 1];
-            rc = launch_groups();
-        }
+        for (int s = 0; s < S && rc == RQA_OK; ++s)
+            rc = launch_groups(cell_args(c, pl, s, true), pl.lsplit1[s].rc < pl.sd[s].ne);
     } else {
         if ((rc = reset_queue(c, ng, &q))) return rc;
-        a.order = pl.d_order;
-        a.uprefix = pl.d_uprefix;
-        a.n_pos = S;
-        a.chunk = pl.chunk;
-        a.n_units = pl.uprefix[S];
-        rc = launch_groups();
+        rc = launch_groups(cell_args(c, pl, -1, true), pl.lsplit.rc < pl.ne_max);
     }
     lb.k0 = 0;  // the finalisation kernels read all K targets
     return rc;
@@ -808,7 +821,7 @@ void rqa_destroy(rqa_ctx *c)
                       &c->redo,
                       &c->queue,
                       &c->status, &c->eps_tmp, &c->le_tmp, &c->lt_tmp, &c->count, &c->lmax,
-                      &c->hshort, &c->mlp, &c->feats, &c->centre, &c->ymlp, &c->acts,
+                      &c->hshort, &c->edges, &c->mlp, &c->feats, &c->centre, &c->ymlp, &c->acts,
                       &c->bstats, &c->learn_scratch};
     for (DevBuf *b : bufs)
         if (b->p) cudaFree(b->p);
@@ -881,7 +894,7 @@ int rqa_det_avg(rqa_ctx *c, const rqa_batch *b, const int32_t *rr_num, int32_t r
     if (pl.ne_max > LINE_NE_MAX) return RQA_ERR_CAPACITY;
     bracket = bracket && pl.any_dom;
     // every scratch buffer sized before anything is enqueued (and captured)
-    if (int rc = ensure_line_bufs(c, pl.S, K)) return rc;
+    if (int rc = ensure_line_bufs(c, pl)) return rc;
     if (!eps)
         if (int rc = ensure_select_bufs(c, pl.S, K)) return rc;
     if (bracket)
@@ -990,7 +1003,7 @@ int rqa_line_hist(rqa_ctx *c, const rqa_batch *b, const float *eps, int32_t K, u
     Plan pl;
     if (int rc = make_plan(c, b, nullptr, 0, K, pl)) return rc;
     if (pl.ne_max > LINE_NE_MAX) return RQA_ERR_CAPACITY;
-    if (int rc = ensure_line_bufs(c, pl.S, K)) return rc;
+    if (int rc = ensure_line_bufs(c, pl)) return rc;
     if (int rc = upload_plan(c, pl, nullptr, 0, hist ? hist_offsets : nullptr)) return rc;
     mark(c, 0);
     if (int rc = launched(c, launch_check_finite(b->y, pl.total, P<int>(c->status), c->stream)))
@@ -1041,11 +1054,11 @@ int rqa_vline_hist(rqa_ctx *c, const rqa_batch *b, const float *eps, int32_t K, 
     const int saved = c->line_tile;
     c->line_tile = LINE_TILE_DEFAULT;
     Plan pl;
-    const int rcp = make_plan(c, b, nullptr, 0, K, pl);
+    const int rcp = make_plan(c, b, nullptr, 0, K, pl, true);
     c->line_tile = saved;
     if (rcp) return rcp;
     if (pl.ne_max > LINE_NE_MAX) return RQA_ERR_CAPACITY;
-    if (int rc = ensure_line_bufs(c, pl.S, K)) return rc;
+    if (int rc = ensure_line_bufs(c, pl)) return rc;
     if (int rc = upload_plan(c, pl, nullptr, 0, vhist ? vhist_offsets : nullptr)) return rc;
     if (int rc = launched(c, launch_check_finite(b->y, pl.total, P<int>(c->status), c->stream)))
         return rc;
@@ -1258,7 +1271,7 @@ int rqa_autotune(rqa_ctx *c, const rqa_batch *b, const int32_t *rr_num, int32_t 
     if (best_ms == 3.4e38f && rc == RQA_OK) time_lines(&best_ms);
     // 2. bands per work unit: half and twice the planned size
     int best_units = 0;
-    const int planned = probe.chunk;
+    const int planned = probe.lsplit.nb;
     const int ucand[2] = {std::max(1, planned / 2), std::min(64, planned * 2)};
     for (int ci = 0; ci < 2 && rc == RQA_OK; ++ci) {
         if (ucand[ci] == planned) continue;

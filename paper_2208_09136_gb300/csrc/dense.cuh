@@ -33,7 +33,8 @@ static_assert(DB == 32 * DPL && RB % 4 == 0 && COLW % 32 == 0 && WIN_WORDS % 4 =
 struct Unit {
     int s, b_lo, b_hi, r_lo, r_hi;
 };
-template <bool VERT>
+// W: diagonals (columns) per band.
+template <bool VERT, int W = DB>
 __device__ __forceinline__ Unit unit_of(const CellArgs &a, int64_t u)
 {
     int lo = 0, hi = a.n_pos;  // last pos with uprefix[pos] <= u
@@ -49,7 +50,7 @@ __device__ __forceinline__ Unit unit_of(const CellArgs &a, int64_t u)
     int bands = 0;
     w.r_lo = 0;
     for (;;) {
-        bands = VERT ? (ne + DB - 1) / DB : (ne - 1 - w.r_lo + DB - 1) / DB;
+        bands = VERT ? (ne + W - 1) / W : (ne - 1 - w.r_lo + W - 1) / W;
         const int items = (bands + a.nb - 1) / a.nb;
         if (rem < items || w.r_lo + a.rc >= ne) break;
         rem -= items;

@@ -38,16 +38,80 @@ static LinesKernel lines_kernel(int embed, int tile, bool vert, bool stage, bool
     }
 }
 
+// Join the lines that meet at the chunk boundaries of a band: a thread per
+// diagonal and threshold walks down the band's chunks.  Where the last row of
+// one chunk and the first row of the next are both recurrent, the two counted
+// pieces x and y are one line of length x + y; a piece as long as its chunk
+// goes on to the next boundary.  The cells of the lines stay the same, so C_k
+// does.  One CTA per band, so that the loads of all bands are in flight.
+template <bool VERT>
+__global__ void __launch_bounds__(LD * KT) k_merge(CellArgs a, LineBufs lb, int K, const uint32_t *edges)
+{
+    __shared__ uint32_t net[LSH][KT];  // changes of P_k(1..LSH)
+    __shared__ uint32_t lmx[KT];
+    const int t = threadIdx.x, lane = t % LD, k = t / LD;
+    for (int i = t; i < LSH * KT; i += LD * KT) (&net[0][0])[i] = 0;
+    if (t < KT) lmx[t] = 0;
+    for (int64_t item = blockIdx.x; item < a.n_units * a.nb; item += gridDim.x) {
+        const int64_t u = item / a.nb;
+        const Unit w = unit_of<VERT, LD>(a, u);
+        const int ne = a.series[w.s].ne, b = w.b_lo + (int)(item - u * a.nb);
+        const int rows = VERT ? ne : ne - 1 - b * LD;
+        if (w.r_lo != 0 || b >= w.b_hi || w.r_hi >= rows) continue;  // a band of one chunk has no boundary
+        const int64_t o = (int64_t)w.s * lb.kstride + lb.k0;
+        const int64_t hrow = ne - 1 + (VERT && lb.loi ? 1 : 0);
+        uint64_t *hb = lb.hist && k < K ? lb.hist + lb.hist_off[w.s] + (int64_t)(lb.k0 + k) * hrow : nullptr;
+        __syncthreads();
+        auto add = [&](uint32_t len, bool more) {
+            if (len <= (uint32_t)LSH) atomicAdd(&net[len - 1][k], more ? 1u : ~0u);
+            else if (hb) atomicAdd(reinterpret_cast<unsigned long long *>(hb + (len - 1)), more ? 1ull : ~0ull);
+        };
+        if (k < K) {
+            int64_t base = u - (w.b_lo / a.nb);  // first unit of the chunk
+            uint32_t open = 0;                   // length up to the boundary of the line that touches it
+            for (int r0 = 0; r0 < rows; r0 += a.rc) {
+                const uint32_t *e = edges + ((base + b / a.nb) * a.nb + b % a.nb) * (2 * KT * LD) + k * LD + lane;
+                const uint32_t y = r0 ? e[0] : 0u;
+                uint32_t z = r0 + a.rc < rows ? e[KT * LD] : 0u;
+                if (open && y) {
+                    add(open, false);
+                    add(y, false);
+                    add(open + y, true);
+                    atomicMax(&lmx[k], open + y);
+                    if (z == (uint32_t)a.rc) z += open;  // the whole chunk
+                }
+                open = z;
+                const int bands = VERT ? (ne + LD - 1) / LD : (ne - 1 - r0 + LD - 1) / LD;
+                base += (bands + a.nb - 1) / a.nb;
+            }
+        }
+        __syncthreads();
+        for (int i = t; i < LSH * KT; i += LD * KT) {
+            const int l = i / KT, q = i - l * KT;
+            const int32_t v = (int32_t)net[l][q];
+            if (v) {
+                atomicAdd(reinterpret_cast<unsigned long long *>(lb.hshort + (o + q) * LSH + l),
+                          (unsigned long long)(long long)v);
+                net[l][q] = 0;
+            }
+        }
+        if (t < KT && lmx[t]) {
+            atomicMax(lb.lmax + o + t, lmx[t]);
+            lmx[t] = 0;
+        }
+    }
+}
+
 template <bool VERT>
 static cudaError_t launch_lines_v(const CellArgs &a, const LineBufs &lb, int K, int grid, int embed,
-                                  cudaStream_t st)
+                                  bool chunks, uint32_t *edges, cudaStream_t st)
 {
     if ((!VERT && !lines_tile_ok(embed, a.line_tile)) || (VERT && a.line_tile != LINE_TILE_DEFAULT))
         return cudaErrorInvalidValue;
     if (!a.y || !a.series || !a.order || !a.uprefix || !a.queue || !a.status || !lb.eps ||
         !lb.count || !lb.lmax || !lb.hshort || (lb.hist && !lb.hist_off) || K < 1 ||
         K > LINE_KMAX || lb.k0 < 0 || lb.k0 + K > lb.kstride || grid < 1 || a.n_units < 1 ||
-        a.n_pos < 1 || a.chunk < 1)
+        a.n_pos < 1 || a.nb < 1 || a.rc < 32 || a.rc % 32 || (chunks && !edges))
         return cudaErrorInvalidValue;
     // staging where the variant exists; elsewhere the flag is ignored
     const bool stage = !VERT && a.line_stage && lines_stage_ok(embed, a.line_tile);
@@ -59,20 +123,18 @@ static cudaError_t launch_lines_v(const CellArgs &a, const LineBufs &lb, int K, 
     grid *= WARPS / LWARPS;  // the caller counts CTAs of WARPS warps
     grid = persistent_cap(reinterpret_cast<const void *>(kern), smem, grid, LTHREADS);
     if (a.line_ctas > 0) grid = std::min(grid, sm_count_current() * a.line_ctas);
-    kern<<<grid, LTHREADS, smem, st>>>(a, lb, K);
+    kern<<<grid, LTHREADS, smem, st>>>(a, lb, K, edges);
+    if ((e = cudaGetLastError()) != cudaSuccess || !chunks) return e;
+    const int mg = (int)std::min<int64_t>(a.n_units * a.nb, (int64_t)sm_count_current() * 3);
+    k_merge<VERT><<<mg, LD * KT, 0, st>>>(a, lb, K, edges);
     return cudaGetLastError();
 }
 
-cudaError_t launch_lines(const CellArgs &a, const LineBufs &lb, int K, int grid, int embed,
-                         cudaStream_t st)
+cudaError_t launch_lines(const CellArgs &a, const LineBufs &lb, int K, int grid, int embed, bool vert,
+                         bool chunks, uint32_t *edges, cudaStream_t st)
 {
-    return launch_lines_v<false>(a, lb, K, grid, embed, st);
-}
-
-cudaError_t launch_vlines(const CellArgs &a, const LineBufs &lb, int K, int grid, int embed,
-                          cudaStream_t st)
-{
-    return launch_lines_v<true>(a, lb, K, grid, embed, st);
+    return vert ? launch_lines_v<true>(a, lb, K, grid, embed, chunks, edges, st)
+                : launch_lines_v<false>(a, lb, K, grid, embed, chunks, edges, st);
 }
 
 }  // namespace rqa

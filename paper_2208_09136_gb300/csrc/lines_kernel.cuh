@@ -38,13 +38,20 @@
 // caller's full histogram), L_max, and C_k = sum of l P_k(l), the recurrent
 // cells.
 //
+// A batch with too few bands to fill the chip is cut into row chunks
+// (CellArgs::rc).  A chunk counts its rows as if the matrix ended at them and
+// keeps, per diagonal and threshold, the lengths of the lines that touch its
+// first and its last row (Edges); k_merge (lines.cu) then joins the lines that
+// meet at a chunk boundary.  The four 10^4-value series of lorenz-n1e4 have
+// 1252 bands for 2432 resident warps, each 10^4 rows long.
+//
 // The vertical pass (VERT) is the same kernel over bands of 32 consecutive
 // columns walked over every row of the matrix: the word of column c is the
 // ballot over 32 consecutive rows, so its runs are vertical lines.
 #pragma once
 #include <cstdint>
 #include <type_traits>
-#include "rqa_common.cuh"
+#include "dense.cuh"
 
 namespace rqa {
 
@@ -178,28 +185,6 @@ __device__ __forceinline__ uint32_t rank_le_word_lane(uint32_t b0, uint32_t b1, 
     return lop3<0x8E>(b4, kbm[4], w);
 }
 
-// Series s and bands [b_lo, b_hi) of work unit u: a unit is a.chunk
-// consecutive bands of one series; units run over the series in a.order
-// (largest first), band 0 (longest diagonals) first.  The vertical pass uses
-// the same units over bands of columns; a series has ceil(Ne / LD) of them,
-// at most one more than of diagonals, which its last unit takes on.
-template <bool VERT>
-__device__ __forceinline__ void unit_of(const CellArgs &a, int64_t u, int &s, int &b_lo,
-                                        int &b_hi, const SeriesDev *series)
-{
-    int lo = 0, hi = a.n_pos;  // last pos with uprefix[pos] <= u
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (a.uprefix[mid] <= u) lo = mid;
-        else hi = mid;
-    }
-    s = a.order[lo];
-    b_lo = (int)(u - a.uprefix[lo]) * a.chunk;
-    const int nbd = (series[s].ne - 1 + LD - 1) / LD;
-    b_hi = min(b_lo + a.chunk, nbd);
-    if (VERT && b_lo + a.chunk >= nbd) b_hi = (series[s].ne + LD - 1) / LD;
-}
-
 // Warp-centric: every warp pulls units from one global queue and keeps its
 // own histogram in shared memory, flushed after each unit.  No CTA-wide
 // barrier, so no warp waits for another.
@@ -227,7 +212,7 @@ __device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane)
 // FK: a full sweep, K = KT thresholds known at compile time (the per-threshold
 // code then runs without a test of k against K); the argument is ignored.
 template <int M, int TAU, int JC, bool VERT, bool STAGE = false, bool FK = false>
-__global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, int K_arg)
+__global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, int K_arg, uint32_t *edges)
 {
     const int K = FK ? KT : K_arg;
     static_assert(LD % JC == 0 && JC % 4 == 0, "windows of whole plane-4 groups");
@@ -376,8 +361,8 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
         if (lane == 0) u = (int64_t)atomicAdd(reinterpret_cast<unsigned long long *>(a.queue), 1ull);
         u = __shfl_sync(FULL, u, 0);
         if (u >= a.n_units) break;
-        int s, ub_lo, ub_hi;
-        unit_of<VERT>(a, u, s, ub_lo, ub_hi, a.series);
+        const Unit un = unit_of<VERT, LD>(a, u);
+        const int s = un.s, ub_lo = un.b_lo, ub_hi = un.b_hi;
         if (s != cur) {
             flush();
             cur = s;
@@ -567,6 +552,13 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                 const int d_lo = 1 + b * LD;                 // diagonal pass: first diagonal
                 const int c_lo = b * LD;                     // vertical pass: first column
                 const int rows = VERT ? sd.ne : sd.ne - d_lo;  // rows of the band's longest line
+                const bool last = un.r_hi >= rows;             // the band's last row chunk
+                const int r_end = last ? rows : un.r_hi;
+                // lengths of the lines at the chunk's first and last row, [k][lane]
+                uint32_t *const edge = edges + (u * a.nb + (b - ub_lo)) * (2 * KT * LD) + lane;
+                // thresholds whose line from the chunk's first row has not ended: k >= mr
+                int mr = un.r_lo > 0 ? 0 : K;
+                bool at_top = un.r_lo > 0;  // some lane has one
                 uint32_t st[KT];
 #pragma unroll
                 for (int k = 0; k < KT; ++k) st[k] = 0;
@@ -623,7 +615,7 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                 };
 
                 // run phase of the same 32 rows: lane j takes diagonal j
-                auto run_phase = [&]() {
+                auto run_phase = [&](int i0) {
                     __syncwarp();
                     const uint4 ra = *reinterpret_cast<const uint4 *>(rkm + lane * 32);
                     const uint4 rb = *reinterpret_cast<const uint4 *>(rkm + lane * 32 + 16);
@@ -661,6 +653,25 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                     *reinterpret_cast<uint4 *>(pl + lane * 4) = make_uint4(B[0], B[1], B[2], B[3]);
                     pl4[lane] = B[4];
                     __syncwarp();  // rank rows read before slots overwrite them
+                    if (at_top) {
+                        // the chunk's first blocks: where the lines that touch its
+                        // first row end (thresholds nest, so those still open are
+                        // the ones from some rank on)
+                        int still = K;
+#pragma unroll 1
+                        for (int k = 0; k < K; ++k) {
+                            uint32_t km[5];
+#pragma unroll
+                            for (int p = 0; p < 5; ++p) km[p] = (((k + 1) >> p) & 1) ? FULL : 0u;
+                            const uint32_t w = rank_le_word_lane(B[0], B[1], B[2], B[3], B[4], km);
+                            if (k >= mr) {
+                                if (w != FULL) edge[k * LD] = (uint32_t)(i0 - un.r_lo) + (uint32_t)__ffs(~w) - 1u;
+                                else still = min(still, k);
+                            }
+                        }
+                        mr = still;
+                        at_top = __any_sync(FULL, mr < K);
+                    }
                     uint32_t lmask = 0;  // thresholds whose word ends lines of length >= 4
 #pragma unroll
                     for (int k = 0; k < KT; ++k) {
@@ -700,22 +711,23 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                 };
 
                 // the packed tallies take SETTLE row blocks before a field could overflow
-                int i0 = 0;
+                int i0 = un.r_lo;
                 // interior row blocks: every cell of the block inside the matrix
-                const int i_end = VERT ? (c_lo + LD <= sd.ne ? rows - 31 : 0) : rows - (LD - 1) - 31;
-                if (STAGE && son && i_end > 0) staged = stage_issue(0, d_lo);
+                const int i_end = min(r_end, VERT ? (c_lo + LD <= sd.ne ? rows - 31 : 0) : rows - (LD - 1) - 31);
+                if (STAGE && son && i0 < i_end) staged = stage_issue(i0, d_lo);
                 for (; i0 < i_end; i0 += 32) {
                     cell_phase(i0, std::true_type{}, i0 + 32 < i_end);
-                    run_phase();
+                    run_phase(i0);
                     if (++nrb == SETTLE) settle();
                 }
-                for (; i0 < rows; i0 += 32) {
+                for (; i0 < r_end; i0 += 32) {
                     cell_phase(i0, std::false_type{}, false);
-                    run_phase();
+                    run_phase(i0);
                     if (++nrb == SETTLE) settle();
                 }
-                // lines that reach the end of a diagonal exactly at a block's last
-                // row: a line of length c ending just above a word (end bit 0)
+                // lines that reach the end of a diagonal, or of the chunk, exactly at
+                // a block's last row: a line of length c ending just above a word
+                // (end bit 0)
                 uint32_t bmask = 0;
 #pragma unroll
                 for (int k = 0; k < KT; ++k) {
@@ -726,6 +738,8 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                             lq[k * LD] = make_uint2(1u, c);
                             bmask |= 1u << k;
                         }
+                        if (!last) edge[(KT + k) * LD] = c;
+                        if (k >= mr) edge[k * LD] = c;  // from the chunk's first row to its last
                     }
                 }
                 long_lines(bmask);
@@ -749,7 +763,7 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
 }  // namespace rqa
 
 namespace rqa {
-using LinesKernel = void (*)(CellArgs, LineBufs, int);
+using LinesKernel = void (*)(CellArgs, LineBufs, int, uint32_t *);
 // Instantiations, one group per translation unit (they compile in parallel).
 // full: the diagonal pass's variant for a sweep of exactly LINE_KMAX thresholds
 LinesKernel lines_kernel_m3t3(int tile, bool vert, bool full);

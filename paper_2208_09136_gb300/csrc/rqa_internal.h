@@ -71,8 +71,7 @@ struct CellArgs {
     const int32_t *order;    // series, largest first
     const int64_t *uprefix;  // n_pos + 1 prefix of unit counts along order
     int32_t n_pos;
-    int32_t nb, rc;          // cell walk: bands per unit and rows per unit (a multiple of RB)
-    int32_t chunk;           // line pass: bands per unit
+    int32_t nb, rc;          // bands per unit and rows per unit (a multiple of the kernel's row block)
     int32_t line_tile;       // diagonals per register window of the line pass (8, 16 or 32)
     int32_t line_ctas;       // persistent CTAs of the line pass per SM (0: as many as fit)
     int32_t line_stage;      // line pass: stage the series windows by bulk copies (where supported)
@@ -93,8 +92,18 @@ constexpr int COUNT_NB = 8;  // bands per unit of the counting rounds: one per w
 // per unit between 8 and 585 blocks: shorter chunks pay their first window
 // loads over too few cells, longer ones leave a tail.
 Split split_cells(uint64_t cells, int nb, int sm_count);
-// Units of a series of ne vectors (vert: the vertical pass, every column over every row).
-int64_t units_of_series(int64_t ne, const Split &sp, bool vert);
+// Units of the line pass over series with these cells and bands of LINE_BAND
+// diagonals, one warp each: runs of whole bands, about eight units per resident
+// warp (16 per SM), so the tail stays short while each unit's histogram flush is
+// spread over many cells; below that, single bands cut into row chunks for
+// about four units per warp, of at least 256 rows (a chunk's first window and
+// its edges cost under a twentieth of that).  A unit covers at most 2^33 cells,
+// so the warp's 32-bit counts of lines of length >= 4 (each line and the cell
+// after it: >= 5 cells) stay exact.
+Split split_lines(uint64_t cells, int64_t bands, int32_t ne_max, int unit_bands, int sm_count);
+// Units of a series of ne vectors with bands of w diagonals (vert: the vertical
+// pass, every column over every row).
+int64_t units_of_series(int64_t ne, const Split &sp, bool vert, int w = DB);
 
 // Kernels (launch wrappers return cudaGetLastError()).
 cudaError_t launch_check_finite(const float *y, int64_t n, int *status, cudaStream_t st);
@@ -115,12 +124,14 @@ struct LineBufs {
     int32_t kstride;       // targets per series in all arrays above (the call's K)
     int32_t loi;           // vertical pass: the cells (j, j) are recurrent
 };
-cudaError_t launch_lines(const CellArgs &a, const LineBufs &lb, int K, int grid, int embed,
-                         cudaStream_t st);
-// Vertical lines of the whole matrix: the same warp pass over bands of
-// LINE_BAND columns (every row of each), reusing the diagonal pass's work plan.
-cudaError_t launch_vlines(const CellArgs &a, const LineBufs &lb, int K, int grid, int embed,
-                          cudaStream_t st);
+// vert: vertical lines of the whole matrix, over columns instead of diagonals.
+// chunks: the units are row chunks, so a second kernel joins the lines at their
+// boundaries; edges then holds LINE_EDGE_BYTES per unit and band of it: per
+// threshold and diagonal the length of the line that touches the chunk's first
+// and its last row.
+constexpr size_t LINE_EDGE_BYTES = 2 * LINE_KMAX * LINE_BAND * 4;
+cudaError_t launch_lines(const CellArgs &a, const LineBufs &lb, int K, int grid, int embed, bool vert,
+                         bool chunks, uint32_t *edges, cudaStream_t st);
 bool lines_tile_ok(int embed, int tile);
 // The diagonal pass of this embedding and window has a staged variant.
 bool lines_stage_ok(int embed, int tile);
