@@ -52,22 +52,21 @@ __global__ void __launch_bounds__(LD * KT) k_merge(CellArgs a, LineBufs lb, int 
     const int t = threadIdx.x, lane = t % LD, k = t / LD;
     for (int i = t; i < LSH * KT; i += LD * KT) (&net[0][0])[i] = 0;
     if (t < KT) lmx[t] = 0;
-    for (int64_t item = blockIdx.x; item < a.n_units * a.nb; item += gridDim.x) {
-        const int64_t u = item / a.nb;
-        const Unit w = unit_of<VERT, LD>(a, u);
-        const int ne = a.series[w.s].ne, b = w.b_lo + (int)(item - u * a.nb);
+    for (int pos = blockIdx.y; pos < a.n_pos; pos += gridDim.y)
+    for (int b = blockIdx.x;; b += gridDim.x) {
+        const int s = a.order[pos], ne = a.series[s].ne;
         const int rows = VERT ? ne : ne - 1 - b * LD;
-        if (w.r_lo != 0 || b >= w.b_hi || w.r_hi >= rows) continue;  // a band of one chunk has no boundary
-        const int64_t o = (int64_t)w.s * lb.kstride + lb.k0;
+        if ((VERT ? b * LD >= ne : rows <= 0) || a.rc >= rows) break;  // bands of one chunk have no boundary
+        const int64_t o = (int64_t)s * lb.kstride + lb.k0;
         const int64_t hrow = ne - 1 + (VERT && lb.loi ? 1 : 0);
-        uint64_t *hb = lb.hist && k < K ? lb.hist + lb.hist_off[w.s] + (int64_t)(lb.k0 + k) * hrow : nullptr;
+        uint64_t *hb = lb.hist && k < K ? lb.hist + lb.hist_off[s] + (int64_t)(lb.k0 + k) * hrow : nullptr;
         __syncthreads();
         auto add = [&](uint32_t len, bool more) {
             if (len <= (uint32_t)LSH) atomicAdd(&net[len - 1][k], more ? 1u : ~0u);
             else if (hb) atomicAdd(reinterpret_cast<unsigned long long *>(hb + (len - 1)), more ? 1ull : ~0ull);
         };
         if (k < K) {
-            int64_t base = u - (w.b_lo / a.nb);  // first unit of the chunk
+            int64_t base = a.uprefix[pos];       // first unit of the chunk
             uint32_t open = 0;                   // length up to the boundary of the line that touches it
             for (int r0 = 0; r0 < rows; r0 += a.rc) {
                 const uint32_t *e = edges + ((base + b / a.nb) * a.nb + b % a.nb) * (2 * KT * LD) + k * LD + lane;
@@ -125,7 +124,9 @@ static cudaError_t launch_lines_v(const CellArgs &a, const LineBufs &lb, int K, 
     if (a.line_ctas > 0) grid = std::min(grid, sm_count_current() * a.line_ctas);
     kern<<<grid, LTHREADS, smem, st>>>(a, lb, K, edges);
     if ((e = cudaGetLastError()) != cudaSuccess || !chunks) return e;
-    const int mg = (int)std::min<int64_t>(a.n_units * a.nb, (int64_t)sm_count_current() * 3);
+    // a column of CTAs per series, about six CTAs per SM in all
+    const int gy = std::min(a.n_pos, 4096);
+    const dim3 mg(std::max(1, sm_count_current() * 6 / gy), gy);
     k_merge<VERT><<<mg, LD * KT, 0, st>>>(a, lb, K, edges);
     return cudaGetLastError();
 }

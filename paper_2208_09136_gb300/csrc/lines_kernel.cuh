@@ -264,6 +264,7 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
     uint32_t lmx = 0;    // the longest of them
 
     int cur = -1;
+    uint64_t acc = 0;  // cells since the last flush
     bool bad = false;
     SeriesDev sd{};
     int tshift = 0, tbm1 = 0, tnb = 0;
@@ -363,6 +364,12 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
         if (u >= a.n_units) break;
         const Unit un = unit_of<VERT, LD>(a, u);
         const int s = un.s, ub_lo = un.b_lo, ub_hi = un.b_hi;
+        // counts are kept while a warp's units are of one series and stay under
+        // 2^33 cells together
+        const uint64_t cells = (uint64_t)(ub_hi - ub_lo) * LD * (uint64_t)(un.r_hi - un.r_lo);
+        const bool full = acc + cells > (1ull << 33);
+        if (s == cur && full) flush();
+        acc = (s == cur && !full ? acc : 0ull) + cells;
         if (s != cur) {
             flush();
             cur = s;
@@ -747,9 +754,6 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
         };
         if (use_tab) bands(std::true_type{});
         else bands(std::false_type{});
-        // flush after each unit: a warp's next unit is usually another series
-        flush();
-        cur = -1;
     }
     flush();
     // a copy left in flight by a time-out: wait for it (bounded) before the
