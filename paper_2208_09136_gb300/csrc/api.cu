@@ -1356,7 +1356,7 @@ int rqa_mlp_backward(rqa_ctx *c, const float *params, const float *X, const floa
     if (!(tau_lo > 0.f && tau_lo < 1.f && tau_hi > 0.f && tau_hi < 1.f)) return RQA_ERR_INVALID_ARG;
     cudaSetDevice(c->device);
     if (int rc = ensure(c->learn_scratch, (size_t)B * (MLP_OUT + 2 * HIDDEN) * 4)) return rc;
-    c->launches += 10;
+    c->launches += 6;
     return check_cuda(mlp_backward(params, X, acts, Y, T, B, tau_lo, tau_hi, grads, loss,
                                    P<float>(c->learn_scratch), c->stream));
 }

@@ -5,7 +5,7 @@
 // passes the exact selection needs.
 //
 // The network is three dense layers on at most a few thousand rows, so the
-// contractions are hand-tiled FP32 FFMA (64 x 64 output tiles, 4 x 4 per
+// contractions are hand-tiled FP32 FFMA (32 x 32 output tiles, 4 x 4 per
 // thread); at this size the tensor cores would not change the step time.
 #include <cstdint>
 #include "rqa_common.cuh"
@@ -94,53 +94,99 @@ cudaError_t launch_sketch(const float *y, const SeriesDev *series, int s_base, i
 // ------------------------------------------------------------ GEMM
 // C[M x N] = op(A) op(B) (+ bias[N]) (ReLU) (* [mask > 0]), row-major.
 // op(A) is A [M x K] or, TA, A stored [K x M]; op(B) is B [K x N] or, TB,
-// B stored [N x K].
-constexpr int GT = 64, GK = 16;
+// B stored [N x K].  rowsum (optional): the sums over K of op(A)'s rows (a
+// bias gradient, whose operand the weight gradient reads anyway).
+//
+// The layers are far too small to fill the chip (256 x 256 x 256 is 0.5 us at
+// the FP32 rate), so a GEMM is bound by the latency of its chain of loads: a
+// 32 x 32 tile per CTA (64 CTAs at 256 x 256), panels of 128 values of K with
+// all their loads in flight at once, and the K of a panel divided among four
+// groups of 64 threads whose partial tiles are added at the end.  At 256 rows
+// the eight GEMMs of a training step take 8 to 17 us each (cold caches), where
+// 64 x 64 tiles with sixteen values of K per step took 12 to 48 us and the
+// bias gradients three more launches of 16 us.
+constexpr int GT = 32, GK = 128, GG = 4;  // tile, panel of K, groups of threads along K
 
 template <bool TA, bool TB>
 __global__ void __launch_bounds__(256)
 k_gemm(const float *__restrict__ A, const float *__restrict__ B, float *__restrict__ C, int M,
-       int N, int K, const float *__restrict__ bias, bool relu, const float *__restrict__ mask)
+       int N, int K, const float *__restrict__ bias, bool relu, const float *__restrict__ mask,
+       float *__restrict__ rowsum)
 {
     __shared__ float As[GK][GT + 1];
     __shared__ float Bs[GK][GT + 1];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const int t = threadIdx.x, g = t >> 6, tx = t & 7, ty = (t >> 3) & 7;
     const int m0 = blockIdx.y * GT, n0 = blockIdx.x * GT;
-    float acc[4][4] = {};
+    float acc[4][4] = {}, rs[4] = {};
     for (int k0 = 0; k0 < K; k0 += GK) {
-        for (int e = threadIdx.x; e < GK * GT; e += 256) {
-            const int kk = e / GT, mm = e % GT;
-            const int gm = m0 + mm, gk = k0 + kk;
-            float va = 0.f;
-            if (gm < M && gk < K) va = TA ? A[(int64_t)gk * M + gm] : A[(int64_t)gm * K + gk];
-            As[kk][mm] = va;
-            const int gn = n0 + mm;
-            float vb = 0.f;
-            if (gn < N && gk < K) vb = TB ? B[(int64_t)gn * K + gk] : B[(int64_t)gk * N + gn];
-            Bs[kk][mm] = vb;
+        float va[GK * GT / 256], vb[GK * GT / 256];
+#pragma unroll
+        for (int i = 0; i < GK * GT / 256; ++i) {
+            const int e = t + 256 * i;
+            // consecutive threads along the operand's contiguous direction
+            const int ka = TA ? e / GT : e % GK, ma = TA ? e % GT : e / GK;
+            const int kb = TB ? e % GK : e / GT, nb = TB ? e / GK : e % GT;
+            va[i] = m0 + ma < M && k0 + ka < K
+                        ? __ldg(A + (TA ? (int64_t)(k0 + ka) * M + m0 + ma : (int64_t)(m0 + ma) * K + k0 + ka)) : 0.f;
+            vb[i] = n0 + nb < N && k0 + kb < K
+                        ? __ldg(B + (TB ? (int64_t)(n0 + nb) * K + k0 + kb : (int64_t)(k0 + kb) * N + n0 + nb)) : 0.f;
+        }
+        __syncthreads();  // the panel before is used up
+#pragma unroll
+        for (int i = 0; i < GK * GT / 256; ++i) {
+            const int e = t + 256 * i;
+            As[TA ? e / GT : e % GK][TA ? e % GT : e / GK] = va[i];
+            Bs[TB ? e % GK : e / GT][TB ? e / GK : e % GT] = vb[i];
         }
         __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < GK; ++kk) {
+        const int kn = min(GK, K - k0);
+#pragma unroll 4
+        for (int kk = g; kk < kn; kk += GG) {
             float a[4], b[4];
 #pragma unroll
-            for (int r = 0; r < 4; ++r) a[r] = As[kk][ty + 16 * r];
+            for (int r = 0; r < 4; ++r) a[r] = As[kk][ty + 8 * r];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) b[q] = Bs[kk][tx + 16 * q];
+            for (int q = 0; q < 4; ++q) b[q] = Bs[kk][tx + 8 * q];
 #pragma unroll
-            for (int r = 0; r < 4; ++r)
+            for (int r = 0; r < 4; ++r) {
+                rs[r] += a[r];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) acc[r][q] = fmaf(a[r], b[q], acc[r][q]);
+            }
         }
-        __syncthreads();
+    }
+    // the four groups' partial tiles, one after the other through shared memory
+    __shared__ float part[GG - 1][64][20];
+    __syncthreads();
+    if (g > 0) {
+        float *p = part[g - 1][t & 63];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            p[16 + r] = rs[r];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) p[4 * r + q] = acc[r][q];
+        }
+    }
+    __syncthreads();
+    if (g > 0) return;
+#pragma unroll
+    for (int h = 0; h < GG - 1; ++h) {
+        const float *p = part[h][t];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            rs[r] += p[16 + r];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[r][q] += p[4 * r + q];
+        }
     }
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
-        const int gm = m0 + ty + 16 * r;
+        const int gm = m0 + ty + 8 * r;
         if (gm >= M) continue;
+        if (rowsum && blockIdx.x == 0 && tx == 0) rowsum[gm] = rs[r];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const int gn = n0 + tx + 16 * q;
+            const int gn = n0 + tx + 8 * q;
             if (gn >= N) continue;
             float v = acc[r][q];
             if (bias) v += bias[gn];
@@ -152,24 +198,13 @@ k_gemm(const float *__restrict__ A, const float *__restrict__ B, float *__restri
 }
 
 static cudaError_t gemm(bool ta, bool tb, const float *A, const float *B, float *C, int M, int N,
-                        int K, const float *bias, bool relu, const float *mask, cudaStream_t st)
+                        int K, const float *bias, bool relu, const float *mask, float *rowsum, cudaStream_t st)
 {
     dim3 grid((N + GT - 1) / GT, (M + GT - 1) / GT);
-    if (!ta && !tb) k_gemm<false, false><<<grid, 256, 0, st>>>(A, B, C, M, N, K, bias, relu, mask);
-    else if (!ta && tb) k_gemm<false, true><<<grid, 256, 0, st>>>(A, B, C, M, N, K, bias, relu, mask);
-    else if (ta && !tb) k_gemm<true, false><<<grid, 256, 0, st>>>(A, B, C, M, N, K, bias, relu, mask);
-    else k_gemm<true, true><<<grid, 256, 0, st>>>(A, B, C, M, N, K, bias, relu, mask);
+    if (!ta && !tb) k_gemm<false, false><<<grid, 256, 0, st>>>(A, B, C, M, N, K, bias, relu, mask, rowsum);
+    else if (!ta && tb) k_gemm<false, true><<<grid, 256, 0, st>>>(A, B, C, M, N, K, bias, relu, mask, rowsum);
+    else k_gemm<true, false><<<grid, 256, 0, st>>>(A, B, C, M, N, K, bias, relu, mask, rowsum);
     return cudaGetLastError();
-}
-
-// Column sums of G [M x N] into out[N].
-__global__ void k_colsum(const float *__restrict__ G, int M, int N, float *out)
-{
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    float acc = 0.f;
-    for (int m = 0; m < M; ++m) acc += G[(int64_t)m * N + n];
-    out[n] = acc;
 }
 
 // Mean pinball loss of Y [B x 2K] against T [B x K] and its gradient.
@@ -231,9 +266,9 @@ cudaError_t mlp_forward(const float *params, const float *X, int B, float *Y, fl
     const MlpView v = mlp_view(params);
     float *H1 = acts, *H2 = acts + (int64_t)B * HIDDEN;
     cudaError_t e;
-    if ((e = gemm(false, true, X, v.W1, H1, B, HIDDEN, FEATURES, v.b1, true, nullptr, st))) return e;
-    if ((e = gemm(false, true, H1, v.W2, H2, B, HIDDEN, HIDDEN, v.b2, true, nullptr, st))) return e;
-    return gemm(false, true, H2, v.W3, Y, B, MLP_OUT, HIDDEN, v.b3, false, nullptr, st);
+    if ((e = gemm(false, true, X, v.W1, H1, B, HIDDEN, FEATURES, v.b1, true, nullptr, nullptr, st))) return e;
+    if ((e = gemm(false, true, H1, v.W2, H2, B, HIDDEN, HIDDEN, v.b2, true, nullptr, nullptr, st))) return e;
+    return gemm(false, true, H2, v.W3, Y, B, MLP_OUT, HIDDEN, v.b3, false, nullptr, nullptr, st);
 }
 
 cudaError_t mlp_backward(const float *params, const float *X, const float *acts, const float *Y,
@@ -251,17 +286,13 @@ cudaError_t mlp_backward(const float *params, const float *X, const float *acts,
     k_pinball<<<(int)std::min<int64_t>((n + 255) / 256, 1024), 256, 0, st>>>(
         Y, T, B, MLP_OUT / 2, tau_lo, tau_hi, dY, loss);
     if ((e = cudaGetLastError())) return e;
-    // layer 3
-    if ((e = gemm(true, false, dY, H2, gW3, MLP_OUT, HIDDEN, B, nullptr, false, nullptr, st))) return e;
-    k_colsum<<<1, 64, 0, st>>>(dY, B, MLP_OUT, gb3);
-    if ((e = gemm(false, false, dY, v.W3, dZ2, B, HIDDEN, MLP_OUT, nullptr, false, H2, st))) return e;
-    // layer 2
-    if ((e = gemm(true, false, dZ2, H1, gW2, HIDDEN, HIDDEN, B, nullptr, false, nullptr, st))) return e;
-    k_colsum<<<1, HIDDEN, 0, st>>>(dZ2, B, HIDDEN, gb2);
-    if ((e = gemm(false, false, dZ2, v.W2, dZ1, B, HIDDEN, HIDDEN, nullptr, false, H1, st))) return e;
-    // layer 1
-    if ((e = gemm(true, false, dZ1, X, gW1, HIDDEN, FEATURES, B, nullptr, false, nullptr, st))) return e;
-    k_colsum<<<1, HIDDEN, 0, st>>>(dZ1, B, HIDDEN, gb1);
+    // each layer: weight and bias gradients in one launch, then the gradient
+    // of its input
+    if ((e = gemm(true, false, dY, H2, gW3, MLP_OUT, HIDDEN, B, nullptr, false, nullptr, gb3, st))) return e;
+    if ((e = gemm(false, false, dY, v.W3, dZ2, B, HIDDEN, MLP_OUT, nullptr, false, H2, nullptr, st))) return e;
+    if ((e = gemm(true, false, dZ2, H1, gW2, HIDDEN, HIDDEN, B, nullptr, false, nullptr, gb2, st))) return e;
+    if ((e = gemm(false, false, dZ2, v.W2, dZ1, B, HIDDEN, HIDDEN, nullptr, false, H1, nullptr, st))) return e;
+    if ((e = gemm(true, false, dZ1, X, gW1, HIDDEN, FEATURES, B, nullptr, false, nullptr, gb1, st))) return e;
     return cudaGetLastError();
 }
 
