@@ -35,8 +35,8 @@ Split split_lines(uint64_t cells, int64_t bands, int32_t ne_max, int unit_bands,
         sp.rc = whole;
     } else {
         sp.nb = 1;
-        const uint64_t blocks = cells / ((uint64_t)LINE_BAND * 32 * (uint64_t)warps * 4);
-        sp.rc = (int)std::min<uint64_t>(32 * std::max<uint64_t>(blocks, 8), (uint64_t)whole);
+        const uint64_t blocks = cells / ((uint64_t)LINE_BAND * 32 * (uint64_t)warps * 2);
+        sp.rc = (int)std::min<uint64_t>(32 * std::max<uint64_t>(blocks, 8), (uint64_t)std::min(whole, LINE_CHUNK_MAX));
     }
     if (unit_bands > 0) sp.nb = unit_bands;  // a tuned size
     sp.nb = (int)std::min<int64_t>(sp.nb, cap);
@@ -632,7 +632,7 @@ int run_lines(rqa_ctx *c, const Plan &pl, const float *eps, uint64_t *hist, cons
             const int kg = std::min(gsz, K - lb.k0);
             const int grid = grid_for(a.n_units);
             if (int rc = launched(c, launch_lines(a, lb, kg, grid, pl.mt, vert, chunks,
-                                                  P<uint32_t>(c->edges), c->stream)))
+                                                  P<uint16_t>(c->edges), c->stream)))
                 return rc;
             c->launches += chunks ? 1 : 0;
         }

@@ -45,7 +45,7 @@ static LinesKernel lines_kernel(int embed, int tile, bool vert, bool stage, bool
 // goes on to the next boundary.  The cells of the lines stay the same, so C_k
 // does.  One CTA per band, so that the loads of all bands are in flight.
 template <bool VERT>
-__global__ void __launch_bounds__(LD * KT) k_merge(CellArgs a, LineBufs lb, int K, const uint32_t *edges)
+__global__ void __launch_bounds__(LD * KT) k_merge(CellArgs a, LineBufs lb, int K, const uint16_t *edges)
 {
     __shared__ uint32_t net[LSH][KT];  // changes of P_k(1..LSH)
     __shared__ uint32_t lmx[KT];
@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(LD * KT) k_merge(CellArgs a, LineBufs lb, int 
             int64_t base = a.uprefix[pos];       // first unit of the chunk
             uint32_t open = 0;                   // length up to the boundary of the line that touches it
             for (int r0 = 0; r0 < rows; r0 += a.rc) {
-                const uint32_t *e = edges + ((base + b / a.nb) * a.nb + b % a.nb) * (2 * KT * LD) + k * LD + lane;
+                const uint16_t *e = edges + ((base + b / a.nb) * a.nb + b % a.nb) * (2 * KT * LD) + k * LD + lane;
                 const uint32_t y = r0 ? e[0] : 0u;
                 uint32_t z = r0 + a.rc < rows ? e[KT * LD] : 0u;
                 if (open && y) {
@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(LD * KT) k_merge(CellArgs a, LineBufs lb, int 
 
 template <bool VERT>
 static cudaError_t launch_lines_v(const CellArgs &a, const LineBufs &lb, int K, int grid, int embed,
-                                  bool chunks, uint32_t *edges, cudaStream_t st)
+                                  bool chunks, uint16_t *edges, cudaStream_t st)
 {
     if ((!VERT && !lines_tile_ok(embed, a.line_tile)) || (VERT && a.line_tile != LINE_TILE_DEFAULT))
         return cudaErrorInvalidValue;
@@ -132,7 +132,7 @@ static cudaError_t launch_lines_v(const CellArgs &a, const LineBufs &lb, int K, 
 }
 
 cudaError_t launch_lines(const CellArgs &a, const LineBufs &lb, int K, int grid, int embed, bool vert,
-                         bool chunks, uint32_t *edges, cudaStream_t st)
+                         bool chunks, uint16_t *edges, cudaStream_t st)
 {
     return vert ? launch_lines_v<true>(a, lb, K, grid, embed, chunks, edges, st)
                 : launch_lines_v<false>(a, lb, K, grid, embed, chunks, edges, st);

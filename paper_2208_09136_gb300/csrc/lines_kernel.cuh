@@ -212,7 +212,7 @@ __device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane)
 // FK: a full sweep, K = KT thresholds known at compile time (the per-threshold
 // code then runs without a test of k against K); the argument is ignored.
 template <int M, int TAU, int JC, bool VERT, bool STAGE = false, bool FK = false>
-__global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, int K_arg, uint32_t *edges)
+__global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, int K_arg, uint16_t *edges)
 {
     const int K = FK ? KT : K_arg;
     static_assert(LD % JC == 0 && JC % 4 == 0, "windows of whole plane-4 groups");
@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                 const bool last = un.r_hi >= rows;             // the band's last row chunk
                 const int r_end = last ? rows : un.r_hi;
                 // lengths of the lines at the chunk's first and last row, [k][lane]
-                uint32_t *const edge = edges + (u * a.nb + (b - ub_lo)) * (2 * KT * LD) + lane;
+                uint16_t *const edge = edges + (u * a.nb + (b - ub_lo)) * (2 * KT * LD) + lane;
                 // thresholds whose line from the chunk's first row has not ended: k >= mr
                 int mr = un.r_lo > 0 ? 0 : K;
                 bool at_top = un.r_lo > 0;  // some lane has one
@@ -672,7 +672,7 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                             for (int p = 0; p < 5; ++p) km[p] = (((k + 1) >> p) & 1) ? FULL : 0u;
                             const uint32_t w = rank_le_word_lane(B[0], B[1], B[2], B[3], B[4], km);
                             if (k >= mr) {
-                                if (w != FULL) edge[k * LD] = (uint32_t)(i0 - un.r_lo) + (uint32_t)__ffs(~w) - 1u;
+                                if (w != FULL) edge[k * LD] = (uint16_t)(i0 - un.r_lo + __ffs(~w) - 1);
                                 else still = min(still, k);
                             }
                         }
@@ -745,8 +745,8 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                             lq[k * LD] = make_uint2(1u, c);
                             bmask |= 1u << k;
                         }
-                        if (!last) edge[(KT + k) * LD] = c;
-                        if (k >= mr) edge[k * LD] = c;  // from the chunk's first row to its last
+                        if (!last) edge[(KT + k) * LD] = (uint16_t)c;
+                        if (k >= mr) edge[k * LD] = (uint16_t)c;  // from the chunk's first row to its last
                     }
                 }
                 long_lines(bmask);
@@ -767,7 +767,7 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
 }  // namespace rqa
 
 namespace rqa {
-using LinesKernel = void (*)(CellArgs, LineBufs, int, uint32_t *);
+using LinesKernel = void (*)(CellArgs, LineBufs, int, uint16_t *);
 // Instantiations, one group per translation unit (they compile in parallel).
 // full: the diagonal pass's variant for a sweep of exactly LINE_KMAX thresholds
 LinesKernel lines_kernel_m3t3(int tile, bool vert, bool full);

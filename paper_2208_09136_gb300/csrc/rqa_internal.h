@@ -96,8 +96,9 @@ Split split_cells(uint64_t cells, int nb, int sm_count);
 // diagonals, one warp each: runs of whole bands, about eight units per resident
 // warp (16 per SM), so the tail stays short while each unit's histogram flush is
 // spread over many cells; below that, single bands cut into row chunks for
-// about four units per warp, of at least 256 rows (a chunk's first window and
-// its edges cost under a twentieth of that).  A unit covers at most 2^33 cells,
+// about two units per warp (four: 876 us instead of 805 for lorenz-n1e4, 391
+// instead of 346 for three series of 7001), of at least 256 rows (a chunk's edges
+// and its first window cost about three blocks).  A unit covers at most 2^33 cells,
 // so the warp's 32-bit counts of lines of length >= 4 (each line and the cell
 // after it: >= 5 cells) stay exact.
 Split split_lines(uint64_t cells, int64_t bands, int32_t ne_max, int unit_bands, int sm_count);
@@ -129,9 +130,10 @@ struct LineBufs {
 // boundaries; edges then holds LINE_EDGE_BYTES per unit and band of it: per
 // threshold and diagonal the length of the line that touches the chunk's first
 // and its last row.
-constexpr size_t LINE_EDGE_BYTES = 2 * LINE_KMAX * LINE_BAND * 4;
+constexpr size_t LINE_EDGE_BYTES = 2 * LINE_KMAX * LINE_BAND * 2;
+constexpr int LINE_CHUNK_MAX = 65504;  // rows of a chunk: its line lengths fit 16 bits
 cudaError_t launch_lines(const CellArgs &a, const LineBufs &lb, int K, int grid, int embed, bool vert,
-                         bool chunks, uint32_t *edges, cudaStream_t st);
+                         bool chunks, uint16_t *edges, cudaStream_t st);
 bool lines_tile_ok(int embed, int tile);
 // The diagonal pass of this embedding and window has a staged variant.
 bool lines_stage_ok(int embed, int tile);
