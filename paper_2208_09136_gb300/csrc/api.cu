@@ -107,7 +107,7 @@ struct rqa_ctx {
     DevBuf prefix, level, rank, below, tab_sub, tab_mid, tab_hash, ngroups, hist, krange,
         redo;
     DevBuf queue, status;
-    DevBuf eps_tmp, le_tmp, lt_tmp, count, lmax, hshort, edges;
+    DevBuf eps_tmp, le_tmp, lt_tmp, line_acc, edges;
     DevBuf meas;  // per-target L / ENTR when only their averages are asked for
     DevBuf grid_thr, grid_hist, grid_rr;  // the approximate grid search
 
@@ -158,7 +158,8 @@ struct Plan {
     std::vector<Split> lsplit1;              // ... and of each series alone
     std::vector<int64_t> uprefix;            // S+1 unit-count prefix along order
     int32_t line_tile = LINE_TILE_DEFAULT;   // diagonals per register window of the line pass
-    int32_t ne_max = 0;                      // largest Ne of the batch
+    int32_t ne_max = 0, n_max = 0;           // largest Ne and N of the batch
+    bool small = false;                      // short series: selected by one CTA each
     std::vector<int32_t> ident;              // 0..S-1
     std::vector<int64_t> uprefix1;           // [2s], [2s+1] = 0, units of s alone
     std::vector<uint8_t> dom;                // 1: the series may be bracketed
@@ -295,7 +296,11 @@ int make_plan(rqa_ctx *c, const rqa_batch *b, const int32_t *rr_num, int32_t rr_
     pl.split1.resize(S);
     pl.cprefix.assign(S + 1, 0);
     pl.cprefix1.assign(2 * (size_t)S, 0);
-    for (int s = 0; s < S; ++s) pl.ne_max = std::max(pl.ne_max, pl.sd[s].ne);
+    for (int s = 0; s < S; ++s) {
+        pl.ne_max = std::max(pl.ne_max, pl.sd[s].ne);
+        pl.n_max = std::max(pl.n_max, pl.sd[s].n);
+    }
+    pl.small = small_select_ok(K, pl.ne_max, pl.n_max, total_cells, c->sm_count);
     pl.line_tile = c->line_tile ? c->line_tile : LINE_TILE_DEFAULT;
     if (!lines_tile_ok(pl.mt, pl.line_tile)) pl.line_tile = LINE_TILE_DEFAULT;
     // warp work units of the line pass
@@ -560,6 +565,14 @@ int select_all(rqa_ctx *c, const rqa_batch *b, Plan &pl, float *eps, uint64_t *l
         if (int rc = check_cuda(cudaMemsetAsync(c->bstats.p, 0, 16, c->stream))) return rc;
     }
     mark(c, 0);
+    if (pl.small && !bracket && c->schedule != RQA_SCHED_PER_SERIES) {
+        mark(c, 1);
+        if (int rc = launched(c, launch_select_small(pl.y, pl.d_sd, pl.S, pl.n_max, pl.d_T, pl.K, eps, le, lt,
+                                                     P<int>(c->status), c->stream)))
+            return rc;
+        for (int i = 2; i <= 4; ++i) mark(c, i);
+        return RQA_OK;
+    }
     if (int rc = launched(c, launch_check_finite(b->y, pl.total, P<int>(c->status), c->stream)))
         return rc;
     mark(c, 1);
@@ -579,6 +592,10 @@ int select_all(rqa_ctx *c, const rqa_batch *b, Plan &pl, float *eps, uint64_t *l
     return run_select(c, pl, sb, cell_args(c, pl, -1), 0, pl.S, q, eps, le, lt, bracket);
 }
 
+// The line pass's accumulators in one block, cleared together: C_k, P_k(1..LSH)
+// and L_max of each (series, target).
+size_t line_acc_bytes(size_t sk) { return sk * (8 + LSH * 8 + 4); }
+
 int ensure_line_bufs(rqa_ctx *c, const Plan &pl)
 {
     const int K = pl.K;
@@ -594,9 +611,7 @@ int ensure_line_bufs(rqa_ctx *c, const Plan &pl)
                 slots = std::max(slots, pl.uprefix1[2 * (size_t)s + 1] * pl.lsplit1[s].nb);
     }
     if ((rc = ensure(c->edges, (size_t)slots * LINE_EDGE_BYTES))) return rc;
-    if ((rc = ensure(c->count, sk * 8))) return rc;
-    if ((rc = ensure(c->lmax, sk * 4))) return rc;
-    if ((rc = ensure(c->hshort, sk * LSH * 8))) return rc;
+    if ((rc = ensure(c->line_acc, line_acc_bytes(sk)))) return rc;
     return RQA_OK;
 }
 
@@ -607,16 +622,14 @@ int run_lines(rqa_ctx *c, const Plan &pl, const float *eps, uint64_t *hist, cons
     const int S = pl.S, K = pl.K;
     const size_t sk = (size_t)S * K;
     lb.eps = eps;
-    lb.count = P<uint64_t>(c->count);
-    lb.lmax = P<uint32_t>(c->lmax);
-    lb.hshort = P<uint64_t>(c->hshort);
+    lb.count = P<uint64_t>(c->line_acc);
+    lb.hshort = lb.count + sk;
+    lb.lmax = reinterpret_cast<uint32_t *>(lb.hshort + sk * LSH);
     lb.hist = hist;
     lb.hist_off = d_hoff;
     lb.kstride = K;
     lb.loi = vert && c->loi;  // only vertical lines run through the identity cells
-    if (int rc = check_cuda(cudaMemsetAsync(lb.count, 0, sk * 8, c->stream))) return rc;
-    if (int rc = check_cuda(cudaMemsetAsync(lb.lmax, 0, sk * 4, c->stream))) return rc;
-    if (int rc = check_cuda(cudaMemsetAsync(lb.hshort, 0, sk * LSH * 8, c->stream))) return rc;
+    if (int rc = check_cuda(cudaMemsetAsync(c->line_acc.p, 0, line_acc_bytes(sk), c->stream))) return rc;
     unsigned *q = nullptr;
     const int full_grid = persistent_grid(c, (size_t)1 << 30);
     auto grid_for = [&](int64_t units) {
@@ -820,8 +833,8 @@ void rqa_destroy(rqa_ctx *c)
                       &c->krange, &c->meas, &c->grid_thr, &c->grid_hist, &c->grid_rr,
                       &c->redo,
                       &c->queue,
-                      &c->status, &c->eps_tmp, &c->le_tmp, &c->lt_tmp, &c->count, &c->lmax,
-                      &c->hshort, &c->edges, &c->mlp, &c->feats, &c->centre, &c->ymlp, &c->acts,
+                      &c->status, &c->eps_tmp, &c->le_tmp, &c->lt_tmp, &c->line_acc,
+                      &c->edges, &c->mlp, &c->feats, &c->centre, &c->ymlp, &c->acts,
                       &c->bstats, &c->learn_scratch};
     for (DevBuf *b : bufs)
         if (b->p) cudaFree(b->p);

@@ -114,6 +114,16 @@ cudaError_t launch_count(int round, const CellArgs &a, const SelBufs &sb, int K,
 cudaError_t launch_select(int round, const SelBufs &sb, int s_begin, int n_series, int K, float *eps_out,
                           uint64_t *le_out, uint64_t *lt_out, int *status, cudaStream_t st);
 
+// The whole selection (and the finiteness check) of short series, one CTA
+// each.  Taken when every series has at most SMALL_NE vectors and the batch few
+// enough cells that its row-per-warp walk (25 instructions per 32 cells where
+// the counting rounds take 7 to 10) stays shorter than their dozen launches:
+// 2^17 cells per SM, one series of 512 vectors per SM.
+constexpr int SMALL_NE = 512;
+bool small_select_ok(int K, int32_t ne_max, int64_t n_max, uint64_t total_cells, int sm_count);
+cudaError_t launch_select_small(const float *y, const SeriesDev *series, int S, int n_max, const uint64_t *T, int K,
+                                float *eps_out, uint64_t *le_out, uint64_t *lt_out, int *status, cudaStream_t st);
+
 struct LineBufs {
     const float *eps;      // [s*kstride + k], ascending per series
     uint64_t *count;       // [s*kstride + k]

@@ -739,4 +739,193 @@ cudaError_t launch_select(int round, const SelBufs &sb, int s_begin, int n_serie
     return cudaGetLastError();
 }
 
+// ------------------------------------------------------------ short series
+// The whole selection of one short series by one CTA: the finiteness check and
+// the three radix rounds on bins in shared memory, the distances recomputed
+// in each round from the series' copy there.  A call on a few short series is
+// bound by its launches, not its cells: at N = 100 the general rounds are
+// twelve launches and memsets that take 71 us for 4950 cells.
+//
+// Groups as in the general rounds: the distinct coarse buckets of the
+// targets, then their distinct 21-bit prefixes; both ascend with the targets.
+constexpr int SM_T = 512;
+constexpr int SM_K = 24;  // targets: two sets of SM_K x NFINE bins fit in shared memory
+
+int small_select_smem(int n_max) { return (NCOARSE + 2 * SM_K * NFINE + n_max) * 4 + NCOARSE; }
+
+__global__ void __launch_bounds__(SM_T)
+k_select_small(const float *__restrict__ y, const SeriesDev *series, const uint64_t *T, int K, float *eps_out,
+               uint64_t *le_out, uint64_t *lt_out, int *status)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint32_t *h1 = reinterpret_cast<uint32_t *>(smem);    // coarse bins, then their cumulative counts
+    uint32_t *h2 = h1 + NCOARSE, *h3 = h2 + SM_K * NFINE;  // middle and low digits, per group
+    float *ys = reinterpret_cast<float *>(h3 + SM_K * NFINE);
+    __shared__ uint32_t pre[SM_K], rnk[SM_K], blw[SM_K], wsum[SM_T / 32];
+    __shared__ int grp[SM_K];
+    const int s = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const SeriesDev sd = series[s];
+    int8_t *t1 = reinterpret_cast<int8_t *>(ys + sd.n);  // coarse bucket -> group
+    const int64_t sk = (int64_t)s * K;
+    bool bad = false;
+    for (int i = t; i < sd.n; i += SM_T) {
+        const float v = y[sd.off + i];
+        ys[i] = v;
+        bad |= !isfinite(v);
+    }
+    if (__any_sync(FULL, bad) && lane == 0) set_status(status, 3 /*NONFINITE*/);
+    for (int i = t; i < NCOARSE + 2 * SM_K * NFINE; i += SM_T) h1[i] = 0;
+    for (int i = t; i < NCOARSE; i += SM_T) t1[i] = -1;
+    __syncthreads();
+
+    // f(key) for every pair: a warp per row, lanes along the columns
+    auto cells = [&](auto &&f) {
+        for (int i = warp; i < sd.ne - 1; i += SM_T / 32)
+            for (int j = i + 1 + lane; j < sd.ne; j += 32) {
+                float d = fabsf(ys[i] - ys[j]);
+                for (int q = 1; q < sd.m; ++q) d = fmaxf(d, fabsf(ys[i + q * sd.tau] - ys[j + q * sd.tau]));
+                f(__float_as_uint(d));
+            }
+        __syncthreads();
+    };
+    // targets 0 .. K-1: grp[k] = index of v[k] among the distinct ascending values
+    auto groups = [&](const uint32_t *v) {
+        if (warp == 0) {
+            const unsigned b = __ballot_sync(FULL, lane < K && (lane == 0 || v[lane] != v[lane - 1]));
+            if (lane < K) grp[lane] = __popc(b & (0xffffffffu >> (31 - lane))) - 1;
+        }
+        __syncthreads();
+    };
+    // a warp: the bin of the NFINE at src whose cumulative count first reaches R
+    auto search = [&](const uint32_t *src, uint32_t R, uint32_t &below, uint32_t &in) -> int {
+        uint32_t seg = 0;
+        for (int i = 0; i < 32; ++i) seg += src[32 * lane + ((i + lane) & 31)];
+        uint32_t cs = seg;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t u = __shfl_up_sync(FULL, cs, o);
+            if (lane >= o) cs += u;
+        }
+        const unsigned hit = __ballot_sync(FULL, cs >= R);
+        below = in = 0;
+        if (!hit) return NFINE;
+        const int sl = __ffs(hit) - 1;
+        const uint32_t base = __shfl_sync(FULL, cs - seg, sl);
+        const uint32_t v = src[32 * sl + lane];
+        uint32_t cv = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t u = __shfl_up_sync(FULL, cv, o);
+            if (lane >= o) cv += u;
+        }
+        cv += base;
+        const int bl = __ffs(__ballot_sync(FULL, cv >= R)) - 1;
+        below = __shfl_sync(FULL, cv - v, bl);
+        in = __shfl_sync(FULL, v, bl);
+        return 32 * sl + bl;
+    };
+
+    cells([&](uint32_t key) { atomicAdd(&h1[key >> COARSE_SHIFT], 1u); });
+    {   // cumulative coarse counts in place (four bins per thread)
+        uint32_t v[NCOARSE / SM_T], sum = 0;
+#pragma unroll
+        for (int i = 0; i < NCOARSE / SM_T; ++i) v[i] = sum += h1[t * (NCOARSE / SM_T) + i];
+        uint32_t incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t u = __shfl_up_sync(FULL, incl, o);
+            if (lane >= o) incl += u;
+        }
+        if (lane == 31) wsum[warp] = incl;
+        __syncthreads();
+        uint32_t excl = incl - sum;
+        for (int w = 0; w < warp; ++w) excl += wsum[w];
+#pragma unroll
+        for (int i = 0; i < NCOARSE / SM_T; ++i) h1[t * (NCOARSE / SM_T) + i] = excl + v[i];
+        __syncthreads();
+    }
+    if (t < K) {
+        const uint32_t R = (uint32_t)T[sk + t];
+        int lo = 0, hi = NCOARSE;  // first bucket whose cumulative count reaches R
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (h1[mid] < R) lo = mid + 1;
+            else hi = mid;
+        }
+        if (lo >= NCOARSE || R == 0) {
+            set_status(status, 10 /*INTERNAL*/);
+            lo = NCOARSE - 1;
+        }
+        blw[t] = lo ? h1[lo - 1] : 0u;
+        pre[t] = (uint32_t)lo;
+        rnk[t] = R - blw[t];
+    }
+    __syncthreads();
+    groups(pre);
+    if (t < K) t1[pre[t]] = (int8_t)grp[t];
+    __syncthreads();
+    cells([&](uint32_t key) {
+        const int g = t1[key >> COARSE_SHIFT];
+        if (g >= 0) atomicAdd(&h2[g * NFINE + ((key >> 10) & (NFINE - 1))], 1u);
+    });
+    for (int k = warp; k < K; k += SM_T / 32) {
+        uint32_t below, in;
+        const int x = search(h2 + grp[k] * NFINE, rnk[k], below, in);
+        __syncwarp();
+        if (lane == 0) {
+            if (x >= NFINE) set_status(status, 10);
+            pre[k] = pre[k] << 10 | (uint32_t)min(x, NFINE - 1);
+            rnk[k] -= below;
+            blw[k] += below;
+        }
+    }
+    __syncthreads();
+    // the middle bins become the table (coarse group, middle digit) -> prefix
+    // group + 1, zero for the others
+    for (int i = t; i < SM_K * NFINE; i += SM_T) h2[i] = 0;
+    __syncthreads();
+    uint32_t slot = 0;
+    if (t < K) slot = (uint32_t)grp[t] * NFINE + (pre[t] & (NFINE - 1));
+    groups(pre);
+    if (t < K) h2[slot] = (uint32_t)grp[t] + 1u;
+    __syncthreads();
+    cells([&](uint32_t key) {
+        const int g1 = t1[key >> COARSE_SHIFT];
+        if (g1 < 0) return;
+        const uint32_t g = h2[g1 * NFINE + ((key >> 10) & (NFINE - 1))];
+        if (g) atomicAdd(&h3[(g - 1u) * NFINE + (key & (NFINE - 1))], 1u);
+    });
+    for (int k = warp; k < K; k += SM_T / 32) {
+        uint32_t below, in;
+        const int x = search(h3 + grp[k] * NFINE, rnk[k], below, in);
+        if (lane == 0) {
+            if (x >= NFINE) {
+                set_status(status, 10);
+            } else {
+                eps_out[sk + k] = __uint_as_float(pre[k] << 10 | (uint32_t)x);
+                if (le_out) le_out[sk + k] = (uint64_t)blw[k] + below + in;
+                if (lt_out) lt_out[sk + k] = (uint64_t)blw[k] + below;
+            }
+        }
+    }
+}
+
+bool small_select_ok(int K, int32_t ne_max, int64_t n_max, uint64_t total_cells, int sm_count)
+{
+    return K <= SM_K && ne_max <= SMALL_NE && n_max <= 2 * SMALL_NE && total_cells <= (uint64_t)sm_count << 17;
+}
+
+cudaError_t launch_select_small(const float *y, const SeriesDev *series, int S, int n_max, const uint64_t *T, int K,
+                                float *eps_out, uint64_t *le_out, uint64_t *lt_out, int *status, cudaStream_t st)
+{
+    if (!y || !series || !T || !eps_out || !status || S < 1 || K < 1 || K > SM_K || n_max < 2 ||
+        n_max > 2 * SMALL_NE)
+        return cudaErrorInvalidValue;
+    const int smem = small_select_smem(n_max);
+    cudaError_t e = cudaFuncSetAttribute(k_select_small, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    k_select_small<<<S, SM_T, smem, st>>>(y, series, T, K, eps_out, le_out, lt_out, status);
+    return cudaGetLastError();
+}
+
 }  // namespace rqa
