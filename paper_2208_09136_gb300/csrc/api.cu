@@ -19,9 +19,10 @@ namespace rqa {
 
 Split split_cells(uint64_t cells, int nb, int sm_count)
 {
-    const uint64_t per_unit = cells / ((uint64_t)sm_count * 2 * 6);
-    const uint64_t blocks = per_unit / ((uint64_t)nb * DB * ROW_BLOCK);
-    return Split{nb, ROW_BLOCK * (int)std::min<uint64_t>(std::max<uint64_t>(blocks, 8), 585)};
+    const uint64_t block = (uint64_t)nb * DB * ROW_BLOCK, ctas = (uint64_t)sm_count * 2;
+    const uint64_t least = std::min<uint64_t>(std::max<uint64_t>(cells / (block * ctas), 2), 8);
+    const uint64_t blocks = std::max<uint64_t>(cells / (block * ctas * 6), least);
+    return Split{nb, ROW_BLOCK * (int)std::min<uint64_t>(blocks, 585)};
 }
 
 Split split_lines(uint64_t cells, int64_t bands, int32_t ne_max, int unit_bands, int sm_count)

@@ -90,7 +90,10 @@ constexpr int ROW_BLOCK = 28;  // rows per block of the cell walk (units start o
 constexpr int COUNT_NB = 8;  // bands per unit of the counting rounds: one per warp of a CTA
 // About six units per CTA (two CTAs per SM) over the whole launch, and rows
 // per unit between 8 and 585 blocks: shorter chunks pay their first window
-// loads over too few cells, longer ones leave a tail.
+// loads over too few cells (lorenz-n1e4: 771 us with at least 8 blocks, 848 with
+// 2), longer ones leave a tail.  A launch with fewer units than CTAs even so is
+// bound by one unit's latency and goes down to 2 blocks (two series of 2003
+// values: 135 us with 8, 87 with 2).
 Split split_cells(uint64_t cells, int nb, int sm_count);
 // Units of the line pass over series with these cells and bands of LINE_BAND
 // diagonals, one warp each: runs of whole bands, about eight units per resident
