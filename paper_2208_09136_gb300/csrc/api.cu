@@ -93,12 +93,11 @@ struct rqa_ctx {
     cudaStream_t stream = nullptr;
     int schedule = RQA_SCHED_BATCHED;
     int select = RQA_SELECT_AUTO;
-    int line_tile = 0;      // diagonals per register window of the line pass (0 = default)
+    int line_tile = 0;      // rqa_tuning.tile and .stage as set: kept for callers that read them back,
     int unit_bands = 0;     // bands per line-pass work unit (0 = planned)
     int line_ctas = 0;      // persistent line-pass CTAs per SM (0 = all that fit)
-    int line_stage = 0;     // line pass: series windows staged by bulk copies (1) or read per lane (0)
+    int line_stage = 0;     // no effect
     float tuned_ms = 0.f;   // line-pass time of the last rqa_autotune choice
-    bool tile_fixed = false;  // the caller chose the tile: rqa_autotune keeps it
     bool loi = false;         // RQA_FLAG_LOI: rates and DET over the whole matrix
     int bpsm = 0;
     int sm_count = 0;
@@ -158,7 +157,6 @@ struct Plan {
     Split lsplit{};                          // line-pass units of the batch ...
     std::vector<Split> lsplit1;              // ... and of each series alone
     std::vector<int64_t> uprefix;            // S+1 unit-count prefix along order
-    int32_t line_tile = LINE_TILE_DEFAULT;   // diagonals per register window of the line pass
     int32_t ne_max = 0, n_max = 0;           // largest Ne and N of the batch
     bool small = false;                      // short series: selected by one CTA each
     std::vector<int32_t> ident;              // 0..S-1
@@ -302,8 +300,6 @@ int make_plan(rqa_ctx *c, const rqa_batch *b, const int32_t *rr_num, int32_t rr_
         pl.n_max = std::max(pl.n_max, pl.sd[s].n);
     }
     pl.small = small_select_ok(K, pl.ne_max, pl.n_max, total_cells, c->sm_count);
-    pl.line_tile = c->line_tile ? c->line_tile : LINE_TILE_DEFAULT;
-    if (!lines_tile_ok(pl.mt, pl.line_tile)) pl.line_tile = LINE_TILE_DEFAULT;
     // warp work units of the line pass
     auto nbl = [&](int s) { return ((int64_t)pl.sd[s].ne - (vert ? 0 : 1) + LINE_BAND - 1) / LINE_BAND; };
     auto cells_of = [&](uint64_t P) { return vert ? 2 * P : P; };
@@ -477,10 +473,7 @@ CellArgs cell_args(rqa_ctx *c, const Plan &pl, int s, bool lines = false)
         a.uprefix = (lines ? pl.d_uprefix1 : pl.d_cprefix1) + 2 * (size_t)s;
         a.n_units = (lines ? pl.uprefix1 : pl.cprefix1)[2 * (size_t)s + 1];
     }
-    a.line_tile = pl.line_tile;
     a.line_ctas = c->line_ctas;
-    a.line_stage = c->line_stage;
-    a.y_len = pl.total;
     return a;
 }
 
@@ -803,7 +796,6 @@ int rqa_create(rqa_ctx **out, const rqa_config *cfg)
     c->schedule = cfg->schedule;
     c->select = cfg->select;
     c->line_tile = cfg->tile;
-    c->tile_fixed = cfg->tile != 0;
     c->graphs = !(cfg->flags & RQA_FLAG_NO_GRAPHS);
     c->loi = (cfg->flags & RQA_FLAG_LOI) != 0;
     c->bpsm = cfg->blocks_per_sm;
@@ -925,7 +917,7 @@ int rqa_det_avg(rqa_ctx *c, const rqa_batch *b, const int32_t *rr_num, int32_t r
         auto put = [&](uint64_t v) { sig.push_back(v); };
         auto ptr = [&](const void *p) { put((uint64_t)(uintptr_t)p); };
         put((uint64_t)pl.S); put((uint64_t)K); put((uint64_t)n_lmin); put((uint64_t)rr_den);
-        put(bracket); put((uint64_t)c->schedule); put((uint64_t)pl.line_tile); put((uint64_t)c->unit_bands); put((uint64_t)c->line_ctas); put((uint64_t)c->line_stage); put(c->timing);
+        put(bracket); put((uint64_t)c->schedule); put((uint64_t)c->unit_bands); put((uint64_t)c->line_ctas); put(c->timing);
         for (int s = 0; s < pl.S; ++s) put(pl.dom[s]);
         put(c->loi);
         uint32_t mb;
@@ -1064,13 +1056,8 @@ int rqa_vline_hist(rqa_ctx *c, const rqa_batch *b, const float *eps, int32_t K, 
     if (int rc = validate_batch(b)) return rc;
     if (int rc = validate_hist(b, K, vhist, vhist_offsets, c->loi ? 1 : 0)) return rc;
     cudaSetDevice(c->device);
-    // the vertical pass runs the default register window
-    const int saved = c->line_tile;
-    c->line_tile = LINE_TILE_DEFAULT;
     Plan pl;
-    const int rcp = make_plan(c, b, nullptr, 0, K, pl, true);
-    c->line_tile = saved;
-    if (rcp) return rcp;
+    if (int rc = make_plan(c, b, nullptr, 0, K, pl, true)) return rc;
     if (pl.ne_max > LINE_NE_MAX) return RQA_ERR_CAPACITY;
     if (int rc = ensure_line_bufs(c, pl)) return rc;
     if (int rc = upload_plan(c, pl, nullptr, 0, vhist ? vhist_offsets : nullptr)) return rc;
@@ -1228,15 +1215,13 @@ int rqa_autotune(rqa_ctx *c, const rqa_batch *b, const int32_t *rr_num, int32_t 
         cells += pc;
     }
     sb.n_series = j;
-    const int saved[4] = {c->line_tile, c->unit_bands, c->line_ctas, c->line_stage};
-    c->line_stage = 0;
+    const int saved[2] = {c->unit_bands, c->line_ctas};
     c->unit_bands = 0;  // the planned unit size, for the probe's plan
     c->line_ctas = 0;
     Plan probe;
     const int rcp = make_plan(c, &sb, nullptr, 0, K, probe);
-    c->unit_bands = saved[1];
-    c->line_ctas = saved[2];
-    c->line_stage = saved[3];
+    c->unit_bands = saved[0];
+    c->line_ctas = saved[1];
     if (rcp) return rcp;
     if (probe.ne_max > LINE_NE_MAX) return RQA_ERR_CAPACITY;
     if (int rc = ensure(c->eps_tmp, (size_t)sb.n_series * K * 4)) return rc;
@@ -1251,7 +1236,6 @@ int rqa_autotune(rqa_ctx *c, const rqa_batch *b, const int32_t *rr_num, int32_t 
         return check_cuda(cudaGetLastError());
     c->unit_bands = 0;
     c->line_ctas = 0;
-    c->line_stage = 0;
     // the line pass over the probe with the context's current knobs, best of two
     auto time_lines = [&](float *best) {
         float t_min = 3.4e38f;
@@ -1266,24 +1250,8 @@ int rqa_autotune(rqa_ctx *c, const rqa_batch *b, const int32_t *rr_num, int32_t 
         *best = t_min;
     };
     float best_ms = 3.4e38f;
-    // 1. register window (kept when the caller fixed it)
-    int best_tile = c->line_tile ? c->line_tile : LINE_TILE_DEFAULT;
-    if (!c->tile_fixed) {
-        const int cand[3] = {8, 16, 32};
-        for (int ci = 0; ci < 3 && rc == RQA_OK; ++ci) {
-            if (!lines_tile_ok(probe.mt, cand[ci])) continue;
-            c->line_tile = cand[ci];
-            float ms = 0.f;
-            time_lines(&ms);
-            if (ms < best_ms) {
-                best_ms = ms;
-                best_tile = cand[ci];
-            }
-        }
-    }
-    c->line_tile = best_tile;
-    if (best_ms == 3.4e38f && rc == RQA_OK) time_lines(&best_ms);
-    // 2. bands per work unit: half and twice the planned size
+    time_lines(&best_ms);  // the planned units, all CTAs that fit
+    // bands per work unit: half and twice the planned size
     int best_units = 0;
     const int planned = probe.lsplit.nb;
     const int ucand[2] = {std::max(1, planned / 2), std::min(64, planned * 2)};
@@ -1298,7 +1266,7 @@ int rqa_autotune(rqa_ctx *c, const rqa_batch *b, const int32_t *rr_num, int32_t 
         }
     }
     c->unit_bands = best_units;
-    // 3. CTAs per SM: all that fit, or six
+    // CTAs per SM: all that fit, or six
     int best_ctas = 0;
     if (rc == RQA_OK) {
         c->line_ctas = 6;
@@ -1310,25 +1278,11 @@ int rqa_autotune(rqa_ctx *c, const rqa_batch *b, const int32_t *rr_num, int32_t 
         }
     }
     c->line_ctas = best_ctas;
-    // 4. series windows staged by bulk copies, where the variant exists
-    int best_stage = 0;
-    if (rc == RQA_OK && lines_stage_ok(probe.mt, c->line_tile)) {
-        c->line_stage = 1;
-        float ms = 0.f;
-        time_lines(&ms);
-        if (ms < best_ms) {
-            best_ms = ms;
-            best_stage = 1;
-        }
-    }
-    c->line_stage = best_stage;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (rc != RQA_OK) {
-        c->line_tile = saved[0];
-        c->unit_bands = saved[1];
-        c->line_ctas = saved[2];
-        c->line_stage = saved[3];
+        c->unit_bands = saved[0];
+        c->line_ctas = saved[1];
         return rc;
     }
     c->tuned_ms = best_ms;

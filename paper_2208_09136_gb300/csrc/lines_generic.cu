@@ -8,14 +8,13 @@ namespace rqa {
 
 LinesKernel lines_kernel_generic(int m, bool vert)
 {
-    constexpr int T = LINE_TILE_DEFAULT;
-    if (vert) return k_lines<0, 0, T, true>;
+    if (vert) return k_lines<0, 0, true>;
     switch (m) {
-    case 1: return k_lines<1, 0, T, false>;
-    case 2: return k_lines<2, 0, T, false>;
-    case 3: return k_lines<3, 0, T, false>;
-    case 4: return k_lines<4, 0, T, false>;
-    default: return k_lines<0, 0, T, false>;
+    case 1: return k_lines<1, 0, false>;
+    case 2: return k_lines<2, 0, false>;
+    case 3: return k_lines<3, 0, false>;
+    case 4: return k_lines<4, 0, false>;
+    default: return k_lines<0, 0, false>;
     }
 }
 

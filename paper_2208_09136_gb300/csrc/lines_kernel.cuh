@@ -5,13 +5,15 @@
 // A warp owns a band of LD = 32 consecutive diagonals and walks down it 32
 // rows at a time.  Each 32 x 32 row block takes two phases:
 //
-//  cells  lane t holds row i0+t.  For every diagonal j of the band it computes
-//         the distance of cell (i0+t, i0+t+d_lo+j) and its rank
-//         r = #{k : eps_k < d} (one lookup in a bucket table of the
-//         thresholds, or a 5-step search over them) and stores r as a byte of
-//         row j of a 32 x 32 rank matrix in shared memory.
-//  runs   lane j holds diagonal j.  It reads row j of the matrix (the ranks of
-//         its 32 cells, two 16-byte loads) and gathers their five bit planes:
+//  cells  the rank r = #{k : eps_k < d} of every cell (one lookup in a bucket
+//         table of the thresholds, or a 5-step search over them).
+//         Compile-time embeddings: lane j walks down diagonal j and packs the
+//         ranks of its 32 cells into eight registers.  Others, and the vertical
+//         pass: lane t holds row i0+t and stores r as a byte of row j of a
+//         32 x 32 rank matrix in shared memory, which lane j then reads.
+//         (m = 3, cycles per SM quarter and 32 cells of the whole pass, mixed
+//         signals: 56.7 by diagonals, 65.1 by rows; tau = 1: 76 and 85.)
+//  runs   lane j holds diagonal j.  It gathers the five bit planes of its ranks:
 //         two words of four ranks are interleaved bit by bit, so one mask and
 //         one multiply bring bit p of eight ranks into the top byte of a
 //         product, and byte permutes put four such bytes together (the rows
@@ -86,54 +88,10 @@ static_assert(LSH > WSH, "lengths WSH+1..LSH go to the global short histogram");
 constexpr int O_LQ = 0, O_PL = O_LQ + KT * LD * 2, O_PL4 = O_PL + LD * 4, O_EPS = O_PL4 + LD,
               O_TAB = O_EPS + 32, O_HS = O_TAB + TMAX, WARP_WORDS = (O_HS + HROW * 32 + 3) & ~3;
 
-// Staged variant (diagonal pass, register windows): after hs, the series
-// values of one interior row block as the bulk-copy engine brings them in
-//   srow  [SR]  the rows' values y[i0 - 3 .. i0 + 32 + (m-1) tau + 3), 16-byte aligned
-//   scol  [SC]  the columns' values from y[i0 + d_lo - 3 ..], 16-byte aligned
-//   bar   one mbarrier (8 bytes) that counts the two copies' bytes
-constexpr int SR = 44, SC = 72;
-constexpr int O_STG = WARP_WORDS, O_BAR = O_STG + SR + SC, WARP_WORDS_ST = (O_BAR + 2 + 3) & ~3;
-static_assert(O_STG % 4 == 0 && (O_STG + SR) % 4 == 0 && O_BAR % 2 == 0, "copy and barrier alignment");
-constexpr uint32_t STAGE_SPIN = 1u << 20;  // polls of a staged block's barrier before giving up
-
 // CTAs of 2 warps: eight fit per SM (shared memory and registers), sixteen warps
 constexpr int LTHREADS = 64;
 constexpr int LWARPS = LTHREADS / 32;
-inline int lines_smem_bytes_impl(bool stage) { return LWARPS * (stage ? WARP_WORDS_ST : WARP_WORDS) * 4; }
-
-// mbarrier and 1-D bulk copy (global -> this CTA's shared memory) in inline PTX.
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(bar), "r"(count) : "memory");
-}
-// the barrier's initialisation made visible to the copy engine (async proxy),
-// and, before a copy overwrites a buffer, the generic-proxy reads of it ordered first
-__device__ __forceinline__ void fence_proxy_async_smem()
-{
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-// one arrival that also announces `bytes` of copies completing on the barrier
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(bar), "r"(bytes)
-                 : "memory");
-}
-// dst and src 16-byte aligned, bytes a multiple of 16
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar)
-{
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-        :: "r"(dst), "l"(__cvta_generic_to_global(src)), "r"(bytes), "r"(bar) : "memory");
-}
-// true once the barrier's phase of the given parity has completed
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-                 "selp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    return ok != 0;
-}
+inline int lines_smem_bytes() { return LWARPS * WARP_WORDS * 4; }
 
 // Recurrence word of threshold k over the 32 rows: bit t = [r_t <= k], i.e.
 // the borrow out of r_t - (k+1) rippled through the bit planes B[0..4] of the
@@ -188,8 +146,6 @@ __device__ __forceinline__ uint32_t rank_le_word_lane(uint32_t b0, uint32_t b1, 
 // Warp-centric: every warp pulls units from one global queue and keeps its
 // own histogram in shared memory, flushed after each unit.  No CTA-wide
 // barrier, so no warp waits for another.
-// JC: diagonals whose cells a lane computes from one register window of the
-// series (the cell phase walks the band's 32 diagonals in LD / JC windows).
 // Transpose a 32 x 32 bit matrix held one row per lane: on return lane k
 // holds column k (bit j of the result = bit k of lane j's word).  Five rounds
 // of exchanging off-diagonal blocks with the lane s apart.
@@ -206,22 +162,17 @@ __device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane)
     return x;
 }
 
-// STAGE: the interior row blocks' series values come into shared memory by
-// bulk copies (one per segment, issued by lane 0 for the next row block while
-// the current one computes) instead of per-lane loads through L1.
 // FK: a full sweep, K = KT thresholds known at compile time (the per-threshold
 // code then runs without a test of k against K); the argument is ignored.
-template <int M, int TAU, int JC, bool VERT, bool STAGE = false, bool FK = false>
+template <int M, int TAU, bool VERT, bool FK = false>
 __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, int K_arg, uint16_t *edges)
 {
     const int K = FK ? KT : K_arg;
-    static_assert(LD % JC == 0 && JC % 4 == 0, "windows of whole plane-4 groups");
-    static_assert(!STAGE || (TAU > 0 && !VERT && ((32 + (M - 1) * TAU + 6) & ~3) <= SR &&
-                             ((31 + LD + (M - 1) * TAU + 6) & ~3) <= SC),
-                  "staging: register windows of the diagonal pass that fit the buffers");
+    constexpr bool WALK = TAU > 0 && !VERT;  // cells by diagonals, else by rows
+    constexpr int JC = 16;  // by rows: diagonals per register window
     extern __shared__ __align__(16) unsigned char smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    uint32_t *ws = reinterpret_cast<uint32_t *>(smem) + warp * (STAGE ? WARP_WORDS_ST : WARP_WORDS);
+    uint32_t *ws = reinterpret_cast<uint32_t *>(smem) + warp * WARP_WORDS;
     uint32_t *pl = ws + O_PL, *pl4 = ws + O_PL4, *epsb = ws + O_EPS, *tab = ws + O_TAB;
     uint32_t *hs = ws + O_HS + lane;  // this lane's column: [l * 32], threshold kk (below)
     uint2 *lqa = reinterpret_cast<uint2 *>(ws + O_LQ);  // [k * LD + j]
@@ -248,17 +199,6 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
 
     for (int l = 0; l < HROW; ++l) hs[l * 32] = 0;
 
-    // staging state (warp-uniform): the buffers hold at most one row block
-    float *const srow = reinterpret_cast<float *>(ws + O_STG), *const scol = srow + SR;
-    const uint32_t sbar = static_cast<uint32_t>(__cvta_generic_to_shared(ws + O_BAR));
-    bool son = STAGE && (reinterpret_cast<uintptr_t>(a.y) & 15u) == 0;  // copies allowed
-    bool sinf = false;      // a copy issued and not yet waited for
-    uint32_t sph = 0;       // parity of the barrier phase that copy completes
-    int srs = 0, scs = 0;   // offsets of y[i0] in srow and of y[i0 + d_lo] in scol
-    if (STAGE && lane == 0) {
-        mbar_init(sbar, 1);
-        fence_proxy_async_smem();
-    }
     __syncwarp();
     uint64_t lmass = 0;  // cells on lines of threshold kk longer than WSH (this unit, this lane)
     uint32_t lmx = 0;    // the longest of them
@@ -434,46 +374,6 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
             lb.hist ? lb.hist + lb.hist_off[s] + (int64_t)lb.k0 * hrow : nullptr;
         uint64_t *const gshort = lb.hshort + ((int64_t)s * lb.kstride + lb.k0) * LSH;
 
-        // Staging of interior row block i0 of the band at d_lo: the values of
-        // its rows, y[i0 .. i0 + 32 + (m-1) tau), and of its columns,
-        // y[i0 + d_lo .. i0 + d_lo + 31 + LD + (m-1) tau), both widened to
-        // 16-byte boundaries; only when the widened segments stay inside the
-        // batch buffer (else the block reads global memory).  The caller has
-        // finished reading the buffers.
-        auto stage_issue = [&](int i0, int d_lo) -> bool {
-            const int64_t gr = sd.off + i0, gc = gr + d_lo;
-            const int64_t ar = gr & ~(int64_t)3, ac = gc & ~(int64_t)3;
-            const int64_t er = (gr + 32 + (M - 1) * TAU + 3) & ~(int64_t)3;
-            const int64_t ec = (gc + 31 + LD + (M - 1) * TAU + 3) & ~(int64_t)3;
-            if (er > a.y_len || ec > a.y_len) return false;
-            srs = (int)(gr - ar);
-            scs = (int)(gc - ac);
-            __syncwarp();  // every lane's reads of the buffers done
-            if (lane == 0) {
-                const uint32_t br = (uint32_t)(er - ar) * 4u, bc = (uint32_t)(ec - ac) * 4u;
-                fence_proxy_async_smem();
-                mbar_arrive_expect_tx(sbar, br + bc);
-                bulk_g2s(static_cast<uint32_t>(__cvta_generic_to_shared(srow)), a.y + ar, br, sbar);
-                bulk_g2s(static_cast<uint32_t>(__cvta_generic_to_shared(scol)), a.y + ac, bc, sbar);
-            }
-            sinf = true;
-            return true;
-        };
-        // wait (bounded) for the staged block; on a time-out the block reads
-        // global memory, staging stops and the status records RQA_ERR_TIMEOUT
-        auto stage_wait = [&]() -> bool {
-            bool ok = false;
-            for (uint32_t it = 0; it < STAGE_SPIN && !ok; ++it) ok = mbar_try_wait(sbar, sph);
-            if (__all_sync(FULL, ok)) {
-                sph ^= 1u;
-                sinf = false;
-                return true;
-            }
-            son = false;
-            if (lane == 0) set_status(a.status, 6 /*TIMEOUT*/);
-            return false;
-        };
-
         // a line of threshold kk longer than WSH (rare): its length into the
         // series' short histogram or the caller's full one
         auto emit_rare = [&](uint32_t len) {
@@ -569,30 +469,16 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                 uint32_t st[KT];
 #pragma unroll
                 for (int k = 0; k < KT; ++k) st[k] = 0;
-                bool staged = false;  // the next interior row block is in the buffers
-
-                // cell phase of the 32 rows i0..i0+31: bit planes of the ranks
-                // of every diagonal into pl / pl4.  INTERIOR: every cell of the
-                // block inside the triangle (no bounds checks).
-                // STAGE: `next` says that row block i0 + 32 is interior too;
-                // its copy is issued once this block's windows are in registers.
-                auto cell_phase = [&](int i0, auto interior, bool next) {
+                // cell phase of the 32 rows i0..i0+31, lane = row: the ranks of
+                // every diagonal into the rank matrix.  INTERIOR: every cell of
+                // the block inside the matrix (no bounds checks).
+                auto cell_phase = [&](int i0, auto interior) {
                     constexpr bool INTERIOR = decltype(interior)::value;
                     const int i = i0 + lane;
-                    bool from_smem = false;
-                    if (STAGE && INTERIOR && staged) {
-                        from_smem = stage_wait();
-                        staged = false;
-                    }
 #pragma unroll 1
                     for (int jc = 0; jc < LD; jc += JC) {
                         BandTile<M, TAU, JC> tile;
-                        if constexpr (STAGE) {
-                            if (INTERIOR && from_smem) tile.load_smem(srow + srs, scol + scs + jc, lane);
-                            else if (INTERIOR) tile.load_fast(ys, i, d_lo + jc, sd.tau);
-                            else tile.load(ys, sd.n, i, d_lo + jc, rows, sd.tau, sd.m);
-                            if (INTERIOR && next && son && jc + JC == LD) staged = stage_issue(i0 + 32, d_lo);
-                        } else if (VERT) {
+                        if (VERT) {
                             if (INTERIOR) tile.load_vert_fast(ys, i, c_lo + jc, sd.tau);
                             else tile.load_vert(ys, sd.n, sd.ne, i, c_lo + jc, sd.tau);
                         } else {
@@ -621,12 +507,83 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                     }
                 };
 
-                // run phase of the same 32 rows: lane j takes diagonal j
-                auto run_phase = [&](int i0) {
+                // The same by diagonals (WALK), lane = diagonal: the coordinate
+                // difference e(s) = y[s] - y[s + d] of row s serves the cells of
+                // rows s, s - tau, .., s - (m-1) tau, so a cell takes one
+                // subtraction and one maximum (by rows: m subtractions and 1.3
+                // window loads), and the ranks stay in the lane that needs them
+                // (by rows: a byte store, and two 16-byte loads per lane).  The
+                // windows of a block come through the slots' shared memory,
+                // requested one block ahead.
+                constexpr int H = WALK ? (M - 1) * TAU : 0;  // rows of differences kept
+                float eh[H + 8];
+                float pc0 = 0.f, pc1 = 0.f, pr = 0.f;
+                float *const rw = reinterpret_cast<float *>(ws + O_LQ), *const cw = rw + 32;
+                auto walk_fetch = [&](int i0) {
+                    const int c = i0 + H + d_lo + lane, r = i0 + H + lane;
+                    pc0 = c < sd.n ? __ldg(ys + c) : 0.f;
+                    pc1 = c + 32 < sd.n ? __ldg(ys + c + 32) : 0.f;
+                    pr = r < sd.n ? __ldg(ys + r) : 0.f;
+                };
+                auto walk_begin = [&](int i0) {
+#pragma unroll
+                    for (int x = 0; x < H; ++x) {
+                        const int c = i0 + x + d_lo + lane;
+                        eh[x] = c < sd.n ? __ldg(ys + i0 + x) - __ldg(ys + c) : 0.f;
+                    }
+                    walk_fetch(i0);
+                };
+                auto walk = [&](int i0, auto interior, uint32_t (&R)[8]) {
+                    constexpr bool INTERIOR = decltype(interior)::value;
                     __syncwarp();
-                    const uint4 ra = *reinterpret_cast<const uint4 *>(rkm + lane * 32);
-                    const uint4 rb = *reinterpret_cast<const uint4 *>(rkm + lane * 32 + 16);
-                    const uint32_t R[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
+                    rw[lane] = pr;
+                    cw[lane] = pc0;
+                    cw[lane + 32] = pc1;
+                    __syncwarp();
+                    walk_fetch(i0 + 32);
+                    const int lim = sd.ne - d_lo - lane - i0;  // rows of this block on the lane's diagonal
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        const float4 ra = *reinterpret_cast<const float4 *>(rw + 8 * h);
+                        const float4 rb = *reinterpret_cast<const float4 *>(rw + 8 * h + 4);
+                        const float rv[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
+                        uint32_t key[8], r[8];
+#pragma unroll
+                        for (int t = 0; t < 8; ++t) {
+                            eh[H + t] = rv[t] - cw[8 * h + t + lane];
+                            float x[M > 0 ? M : 1];
+#pragma unroll
+                            for (int q = 0; q < M; ++q) x[q] = eh[t + q * TAU];
+                            key[t] = __float_as_uint(maxnorm<(M > 0 ? M : 1)>(x));
+                        }
+                        if (TABLE) {  // eight lookups in flight before the first is used
+                            uint32_t lo[8], e[8];
+#pragma unroll
+                            for (int t = 0; t < 8; ++t) {
+                                const uint64_t pk = (uint64_t)key[t] * tmul;
+                                lo[t] = (uint32_t)pk;
+                                e[t] = tab[__viaddmin_s32_relu((int)(uint32_t)(pk >> 32), -tbm1, tnb + 1)];
+                            }
+#pragma unroll
+                            for (int t = 0; t < 8; ++t) r[t] = lo[t] > e[t] ? (e[t] >> 5) : e[t];
+                        } else {
+#pragma unroll
+                            for (int t = 0; t < 8; ++t) r[t] = rank_of(key[t]);
+                        }
+                        if (!INTERIOR) {
+#pragma unroll
+                            for (int t = 0; t < 8; ++t) r[t] = 8 * h + t < lim ? r[t] : 31u;
+                        }
+                        // the byte order of the rank matrix: even rows, odd rows
+                        R[2 * h] = __byte_perm(__byte_perm(r[0], r[2], 0x0040), __byte_perm(r[4], r[6], 0x0040), 0x5410);
+                        R[2 * h + 1] = __byte_perm(__byte_perm(r[1], r[3], 0x0040), __byte_perm(r[5], r[7], 0x0040), 0x5410);
+#pragma unroll
+                        for (int x = 0; x < H; ++x) eh[x] = eh[x + 8];
+                    }
+                };
+
+                // run phase of the same 32 rows: lane j takes diagonal j
+                auto run_phase = [&](int i0, const uint32_t (&R)[8]) {
                     // Words 2h and 2h + 1 hold rows 8h .. 8h + 7 (byte u of word
                     // 2h: row 8h + 2u, of word 2h + 1: row 8h + 2u + 1).  X[h]
                     // interleaves their even bits (bit p of byte u of word 2h
@@ -721,17 +678,24 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                 int i0 = un.r_lo;
                 // interior row blocks: every cell of the block inside the matrix
                 const int i_end = min(r_end, VERT ? (c_lo + LD <= sd.ne ? rows - 31 : 0) : rows - (LD - 1) - 31);
-                if (STAGE && son && i0 < i_end) staged = stage_issue(i0, d_lo);
-                for (; i0 < i_end; i0 += 32) {
-                    cell_phase(i0, std::true_type{}, i0 + 32 < i_end);
-                    run_phase(i0);
+                auto block = [&](auto interior) {
+                    uint32_t R[8];
+                    if constexpr (WALK) {
+                        walk(i0, interior, R);
+                    } else {
+                        cell_phase(i0, interior);
+                        __syncwarp();
+                        const uint4 ra = *reinterpret_cast<const uint4 *>(rkm + lane * 32);
+                        const uint4 rb = *reinterpret_cast<const uint4 *>(rkm + lane * 32 + 16);
+                        R[0] = ra.x; R[1] = ra.y; R[2] = ra.z; R[3] = ra.w;
+                        R[4] = rb.x; R[5] = rb.y; R[6] = rb.z; R[7] = rb.w;
+                    }
+                    run_phase(i0, R);
                     if (++nrb == SETTLE) settle();
-                }
-                for (; i0 < r_end; i0 += 32) {
-                    cell_phase(i0, std::false_type{}, false);
-                    run_phase(i0);
-                    if (++nrb == SETTLE) settle();
-                }
+                };
+                if constexpr (WALK) walk_begin(i0);
+                for (; i0 < i_end; i0 += 32) block(std::true_type{});
+                for (; i0 < r_end; i0 += 32) block(std::false_type{});
                 // lines that reach the end of a diagonal, or of the chunk, exactly at
                 // a block's last row: a line of length c ending just above a word
                 // (end bit 0)
@@ -756,12 +720,6 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
         else bands(std::false_type{});
     }
     flush();
-    // a copy left in flight by a time-out: wait for it (bounded) before the
-    // CTA's shared memory is released
-    if (STAGE && sinf) {
-        bool ok = false;
-        for (uint32_t it = 0; it < STAGE_SPIN && !ok; ++it) ok = mbar_try_wait(sbar, sph);
-    }
 }
 
 }  // namespace rqa
@@ -770,9 +728,9 @@ namespace rqa {
 using LinesKernel = void (*)(CellArgs, LineBufs, int, uint16_t *);
 // Instantiations, one group per translation unit (they compile in parallel).
 // full: the diagonal pass's variant for a sweep of exactly LINE_KMAX thresholds
-LinesKernel lines_kernel_m3t3(int tile, bool vert, bool full);
-LinesKernel lines_kernel_m3t1(int tile, bool vert, bool full);
-LinesKernel lines_kernel_m1t1(int tile, bool vert, bool full);
+// full: the diagonal pass's variant for a sweep of exactly LINE_KMAX thresholds
+LinesKernel lines_kernel_m3t3(bool vert, bool full);
+LinesKernel lines_kernel_m3t1(bool vert, bool full);
+LinesKernel lines_kernel_m1t1(bool vert, bool full);
 LinesKernel lines_kernel_generic(int m, bool vert);
-LinesKernel lines_kernel_staged(int embed, int tile);  // nullptr where there is none
 }  // namespace rqa

@@ -1,21 +1,14 @@
 // Instantiations of the line pass kernel (lines_kernel.cuh) for m = 3, tau = 3:
-// the diagonal pass with register windows of 8, 16 and 32 diagonals (each also
-// for a full sweep of LINE_KMAX thresholds), and the vertical pass.  One group
-// per translation unit, so they compile in parallel.
+// the diagonal pass (also for a full sweep of LINE_KMAX thresholds) and the
+// vertical pass.  One group per translation unit, so they compile in parallel.
 #include "lines_kernel.cuh"
 
 namespace rqa {
 
-LinesKernel lines_kernel_m3t3(int tile, bool vert, bool full)
+LinesKernel lines_kernel_m3t3(bool vert, bool full)
 {
-    if (vert) return k_lines<3, 3, LINE_TILE_DEFAULT, true>;
-    switch (tile) {
-    case 8: return full ? k_lines<3, 3, 8, false, false, true> : k_lines<3, 3, 8, false>;
-    case 32: return full ? k_lines<3, 3, 32, false, false, true> : k_lines<3, 3, 32, false>;
-    default:
-        return full ? k_lines<3, 3, LINE_TILE_DEFAULT, false, false, true>
-                    : k_lines<3, 3, LINE_TILE_DEFAULT, false>;
-    }
+    if (vert) return k_lines<3, 3, true>;
+    return full ? k_lines<3, 3, false, true> : k_lines<3, 3, false>;
 }
 
 }  // namespace rqa

@@ -23,7 +23,7 @@ constexpr int LSH = 64;            // line lengths 1..LSH counted in shared memo
 constexpr int LMIN_MAX = 8;        // entries of an lmin list
 constexpr int THREADS = 256;       // threads per CTA of the cell kernels
 constexpr int DB = 128;            // diagonals (columns) per warp band of the cell walk
-constexpr int LINE_TILE_DEFAULT = 16;  // diagonals per register window of the line pass's cell phase
+constexpr int LINE_TILE_DEFAULT = 16;  // rqa_tuning.tile when none was set (reported only)
 constexpr int LINE_NE_MAX = (1 << 26) - 1;  // vectors per series the line pass counts exactly
 constexpr int64_t COUNT_NE_MAX = (int64_t)3 << 25;  // vectors per series the counting rounds take
 constexpr int WARPS = THREADS / 32;
@@ -72,10 +72,7 @@ struct CellArgs {
     const int64_t *uprefix;  // n_pos + 1 prefix of unit counts along order
     int32_t n_pos;
     int32_t nb, rc;          // bands per unit and rows per unit (a multiple of the kernel's row block)
-    int32_t line_tile;       // diagonals per register window of the line pass (8, 16 or 32)
     int32_t line_ctas;       // persistent CTAs of the line pass per SM (0: as many as fit)
-    int32_t line_stage;      // line pass: stage the series windows by bulk copies (where supported)
-    int64_t y_len;           // values in the batch buffer y (bulk copies stay below it)
     int64_t n_units;
     unsigned int *queue;   // ticket counter (64-bit aligned), zeroed before launch
     int *status;
@@ -147,9 +144,6 @@ constexpr size_t LINE_EDGE_BYTES = 2 * LINE_KMAX * LINE_BAND * 2;
 constexpr int LINE_CHUNK_MAX = 65504;  // rows of a chunk: its line lengths fit 16 bits
 cudaError_t launch_lines(const CellArgs &a, const LineBufs &lb, int K, int grid, int embed, bool vert,
                          bool chunks, uint16_t *edges, cudaStream_t st);
-bool lines_tile_ok(int embed, int tile);
-// The diagonal pass of this embedding and window has a staged variant.
-bool lines_stage_ok(int embed, int tile);
 cudaError_t launch_finalize_det(const LineBufs &lb, const SeriesDev *series, int S, int K,
                                 const int32_t *lmin_dev, int n_lmin, double *det,
                                 double *det_avg, bool loi, cudaStream_t st);
