@@ -16,7 +16,7 @@ static LinesKernel lines_kernel(int embed, bool vert, bool full)
     case E_M3T3: return lines_kernel_m3t3(vert, full);
     case E_M3T1: return lines_kernel_m3t1(vert, full);
     case E_M1T1: return lines_kernel_m1t1(vert, full);
-    case E_M1: case E_M2: case E_M3: case E_M4: return lines_kernel_generic(embed, vert);
+    case E_M2: case E_M3: case E_M4: return lines_kernel_generic(embed, vert);
     default: return lines_kernel_generic(0, vert);
     }
 }

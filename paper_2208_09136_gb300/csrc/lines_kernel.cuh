@@ -168,8 +168,8 @@ template <int M, int TAU, bool VERT, bool FK = false>
 __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, int K_arg, uint16_t *edges)
 {
     const int K = FK ? KT : K_arg;
-    constexpr bool WALK = TAU > 0 && !VERT;  // cells by diagonals, else by rows
-    constexpr int JC = 16;  // by rows: diagonals per register window
+    constexpr bool WALK = M > 0;            // cells by diagonals (columns), else by rows
+    constexpr bool RING = TAU > 0 && !VERT;  // differences kept from row to row
     extern __shared__ __align__(16) unsigned char smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint32_t *ws = reinterpret_cast<uint32_t *>(smem) + warp * WARP_WORDS;
@@ -475,55 +475,49 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                 auto cell_phase = [&](int i0, auto interior) {
                     constexpr bool INTERIOR = decltype(interior)::value;
                     const int i = i0 + lane;
-#pragma unroll 1
-                    for (int jc = 0; jc < LD; jc += JC) {
-                        BandTile<M, TAU, JC> tile;
-                        if (VERT) {
-                            if (INTERIOR) tile.load_vert_fast(ys, i, c_lo + jc, sd.tau);
-                            else tile.load_vert(ys, sd.n, sd.ne, i, c_lo + jc, sd.tau);
-                        } else {
-                            if (INTERIOR) tile.load_fast(ys, i, d_lo + jc, sd.tau);
-                            else tile.load(ys, sd.n, i, d_lo + jc, rows, sd.tau, sd.m);
-                        }
-#pragma unroll
-                        for (int j = 0; j < JC; ++j) {
-                            const int col = c_lo + jc + j;   // vertical pass: column
-                            // diagonal pass: cell (i, i + dl); vertical: (i, col)
-                            const int dl = VERT ? col - i : d_lo + jc + j;
-                            const bool valid =
-                                VERT ? (INTERIOR || (i < sd.ne && col < sd.ne)) && (lb.loi || dl != 0)
-                                     : INTERIOR || i < sd.ne - dl;
-                            uint32_t r = 31;  // outside the matrix: recurrent for no k
-                            // register windows read no memory per cell, so cells
-                            // outside the triangle are computed and discarded
-                            if (TAU > 0 || valid) {
-                                const uint32_t key =
-                                    __float_as_uint(tile.dist(ys, j, i, dl, sd.tau, sd.m));
-                                const uint32_t rk = rank_of(key);
-                                r = valid ? rk : 31u;
-                            }
-                            rkm[(jc + j) * 32 + rcol] = (unsigned char)r;
-                        }
+#pragma unroll 4
+                    for (int j = 0; j < LD; ++j) {
+                        const int col = c_lo + j;   // vertical pass: column
+                        // diagonal pass: cell (i, i + dl); vertical: (i, col)
+                        const int dl = VERT ? col - i : d_lo + j;
+                        const bool valid = INTERIOR || (VERT ? i < sd.ne && col < sd.ne && (lb.loi || dl != 0)
+                                                             : i < sd.ne - dl);
+                        uint32_t r = 31;  // outside the matrix: recurrent for no k
+                        if (valid) r = rank_of(__float_as_uint(cell_dist(ys, i, dl, sd.tau, sd.m)));
+                        rkm[j * 32 + rcol] = (unsigned char)r;
                     }
                 };
 
-                // The same by diagonals (WALK), lane = diagonal: the coordinate
-                // difference e(s) = y[s] - y[s + d] of row s serves the cells of
-                // rows s, s - tau, .., s - (m-1) tau, so a cell takes one
-                // subtraction and one maximum (by rows: m subtractions and 1.3
-                // window loads), and the ranks stay in the lane that needs them
-                // (by rows: a byte store, and two 16-byte loads per lane).  The
-                // windows of a block come through the slots' shared memory,
+                // The same by diagonals (WALK), lane = diagonal, the ranks staying
+                // in the lane that needs them (by rows: a byte store per cell and
+                // two 16-byte loads per lane).
+                //  RING  compile-time embedding: the coordinate difference
+                //        e(s) = y[s] - y[s + d] of row s serves the cells of rows
+                //        s, s - tau, .., s - (m-1) tau, so a cell takes one
+                //        subtraction and one maximum (by rows: m subtractions and
+                //        1.3 window loads).
+                //  delay known at run time: a window per coordinate, m
+                //        subtractions of conflict-free shared loads.
+                //  VERT  the lane's column vector in registers, the rows of each
+                //        coordinate as a broadcast window.
+                // The windows of a block come through the slots' shared memory,
                 // requested one block ahead.
-                constexpr int H = WALK ? (M - 1) * TAU : 0;  // rows of differences kept
-                float eh[H + 8];
-                float pc0 = 0.f, pc1 = 0.f, pr = 0.f;
-                float *const rw = reinterpret_cast<float *>(ws + O_LQ), *const cw = rw + 32;
+                constexpr int NW = RING || M == 0 ? 1 : M;   // windows
+                constexpr int H = RING ? (M - 1) * TAU : 0;  // rows of differences kept
+                const int tau = TAU > 0 ? TAU : sd.tau;
+                float eh[RING ? H + 8 : 1], av[VERT && M > 0 ? M : 1];
+                float pc[NW][2], pr[NW];
+                float *const rw = reinterpret_cast<float *>(ws + O_LQ), *const cw = rw + 32 * NW;
                 auto walk_fetch = [&](int i0) {
-                    const int c = i0 + H + d_lo + lane, r = i0 + H + lane;
-                    pc0 = c < sd.n ? __ldg(ys + c) : 0.f;
-                    pc1 = c + 32 < sd.n ? __ldg(ys + c + 32) : 0.f;
-                    pr = r < sd.n ? __ldg(ys + r) : 0.f;
+#pragma unroll
+                    for (int q = 0; q < NW; ++q) {
+                        const int r = i0 + H + q * tau + lane, c = r + d_lo;
+                        pr[q] = r < sd.n ? __ldg(ys + r) : 0.f;
+                        if (!VERT) {
+                            pc[q][0] = c < sd.n ? __ldg(ys + c) : 0.f;
+                            pc[q][1] = c + 32 < sd.n ? __ldg(ys + c + 32) : 0.f;
+                        }
+                    }
                 };
                 auto walk_begin = [&](int i0) {
 #pragma unroll
@@ -531,30 +525,55 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                         const int c = i0 + x + d_lo + lane;
                         eh[x] = c < sd.n ? __ldg(ys + i0 + x) - __ldg(ys + c) : 0.f;
                     }
+                    if (VERT) {
+#pragma unroll
+                        for (int q = 0; q < M; ++q) av[q] = __ldg(ys + min(c_lo + lane + q * tau, sd.n - 1));
+                    }
                     walk_fetch(i0);
                 };
                 auto walk = [&](int i0, auto interior, uint32_t (&R)[8]) {
                     constexpr bool INTERIOR = decltype(interior)::value;
                     __syncwarp();
-                    rw[lane] = pr;
-                    cw[lane] = pc0;
-                    cw[lane + 32] = pc1;
+#pragma unroll
+                    for (int q = 0; q < NW; ++q) {
+                        rw[32 * q + lane] = pr[q];
+                        if (!VERT) {
+                            cw[64 * q + lane] = pc[q][0];
+                            cw[64 * q + lane + 32] = pc[q][1];
+                        }
+                    }
                     __syncwarp();
                     walk_fetch(i0 + 32);
-                    const int lim = sd.ne - d_lo - lane - i0;  // rows of this block on the lane's diagonal
+                    // rows of this block on the lane's diagonal (column); the
+                    // identity cell of a column, unless it counts
+                    const int col = c_lo + lane;
+                    const int lim = VERT ? (col < sd.ne ? sd.ne - i0 : 0) : sd.ne - d_lo - lane - i0;
+                    const int same = VERT && !lb.loi ? col - i0 : -1;
 #pragma unroll
                     for (int h = 0; h < 4; ++h) {
-                        const float4 ra = *reinterpret_cast<const float4 *>(rw + 8 * h);
-                        const float4 rb = *reinterpret_cast<const float4 *>(rw + 8 * h + 4);
-                        const float rv[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
                         uint32_t key[8], r[8];
 #pragma unroll
-                        for (int t = 0; t < 8; ++t) {
-                            eh[H + t] = rv[t] - cw[8 * h + t + lane];
-                            float x[M > 0 ? M : 1];
+                        for (int g = 0; g < 8; g += 4) {
+                            float rv[NW][4];
 #pragma unroll
-                            for (int q = 0; q < M; ++q) x[q] = eh[t + q * TAU];
-                            key[t] = __float_as_uint(maxnorm<(M > 0 ? M : 1)>(x));
+                            for (int q = 0; q < NW; ++q) {
+                                const float4 v = *reinterpret_cast<const float4 *>(rw + 32 * q + 8 * h + g);
+                                rv[q][0] = v.x;
+                                rv[q][1] = v.y;
+                                rv[q][2] = v.z;
+                                rv[q][3] = v.w;
+                            }
+#pragma unroll
+                            for (int t = 0; t < 4; ++t) {
+                                float x[M > 0 ? M : 1];
+                                if (RING) eh[RING ? H + g + t : 0] = rv[0][t] - cw[8 * h + g + t + lane];
+#pragma unroll
+                                for (int q = 0; q < M; ++q)
+                                    x[q] = RING   ? eh[RING ? g + t + q * TAU : 0]
+                                           : VERT ? rv[RING ? 0 : q][t] - av[VERT ? q : 0]
+                                                  : rv[RING ? 0 : q][t] - cw[64 * q + 8 * h + g + t + lane];
+                                key[g + t] = __float_as_uint(maxnorm<(M > 0 ? M : 1)>(x));
+                            }
                         }
                         if (TABLE) {  // eight lookups in flight before the first is used
                             uint32_t lo[8], e[8];
@@ -572,13 +591,14 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                         }
                         if (!INTERIOR) {
 #pragma unroll
-                            for (int t = 0; t < 8; ++t) r[t] = 8 * h + t < lim ? r[t] : 31u;
+                            for (int t = 0; t < 8; ++t)
+                                r[t] = 8 * h + t < lim && (!VERT || 8 * h + t != same) ? r[t] : 31u;
                         }
                         // the byte order of the rank matrix: even rows, odd rows
                         R[2 * h] = __byte_perm(__byte_perm(r[0], r[2], 0x0040), __byte_perm(r[4], r[6], 0x0040), 0x5410);
                         R[2 * h + 1] = __byte_perm(__byte_perm(r[1], r[3], 0x0040), __byte_perm(r[5], r[7], 0x0040), 0x5410);
 #pragma unroll
-                        for (int x = 0; x < H; ++x) eh[x] = eh[x + 8];
+                        for (int x = 0; x < H; ++x) eh[x] = eh[RING ? x + 8 : 0];
                     }
                 };
 
@@ -676,8 +696,6 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
 
                 // the packed tallies take SETTLE row blocks before a field could overflow
                 int i0 = un.r_lo;
-                // interior row blocks: every cell of the block inside the matrix
-                const int i_end = min(r_end, VERT ? (c_lo + LD <= sd.ne ? rows - 31 : 0) : rows - (LD - 1) - 31);
                 auto block = [&](auto interior) {
                     uint32_t R[8];
                     if constexpr (WALK) {
@@ -694,8 +712,15 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                     if (++nrb == SETTLE) settle();
                 };
                 if constexpr (WALK) walk_begin(i0);
-                for (; i0 < i_end; i0 += 32) block(std::true_type{});
-                for (; i0 < r_end; i0 += 32) block(std::false_type{});
+                for (; i0 < r_end; i0 += 32) {
+                    // interior row blocks: every cell inside the matrix (and off the
+                    // identity line)
+                    const bool inside = VERT ? c_lo + LD <= sd.ne && i0 + 32 <= rows &&
+                                                   (lb.loi || i0 + 32 <= c_lo || i0 >= c_lo + LD)
+                                             : i0 + 32 <= rows - (LD - 1);
+                    if (inside) block(std::true_type{});
+                    else block(std::false_type{});
+                }
                 // lines that reach the end of a diagonal, or of the chunk, exactly at
                 // a block's last row: a line of length c ending just above a word
                 // (end bit 0)

@@ -56,138 +56,18 @@ __device__ __forceinline__ float maxnorm(const float (&diff)[M])
     return d;
 }
 
-// Distances of one lane's cells in a band: row i (lane), diagonals
-// d_lo .. d_lo+D-1.  Maximum-norm distance (Sect. 2) with FP32 subtract, abs
-// and max only, so every value is exact and equal to a CPU evaluation.
-//
-// Compile-time embedding (M >= 1, TAU >= 1): the row vector
-// x_i = (y[i], y[i+TAU], ...) and the column window y[i+d_lo .. i+d_lo+D-1+
-// (M-1)TAU] are loaded into registers once per 32-row block, so the D cells of
-// the lane need no further memory traffic.
-template <int M, int TAU, int D>
-struct BandTile {
-    float a[M];
-    float w[D + (M - 1) * TAU];
-    __device__ __forceinline__ void load(const float *__restrict__ ys, int n, int i, int d_lo,
-                                         int rows, int, int)
-    {
-        if (i < rows) {
-#pragma unroll
-            for (int q = 0; q < M; ++q) a[q] = __ldg(ys + i + q * TAU);
-        }
-#pragma unroll
-        for (int x = 0; x < D + (M - 1) * TAU; ++x) {
-            const int idx = i + d_lo + x;
-            w[x] = (i < rows && idx < n) ? __ldg(ys + idx) : 0.f;
-        }
-    }
-    // every lane's row and window inside the series (an interior row block)
-    __device__ __forceinline__ void load_fast(const float *__restrict__ ys, int i, int d_lo, int)
-    {
-#pragma unroll
-        for (int q = 0; q < M; ++q) a[q] = __ldg(ys + i + q * TAU);
-#pragma unroll
-        for (int x = 0; x < D + (M - 1) * TAU; ++x) w[x] = __ldg(ys + i + d_lo + x);
-    }
-    // the same window from shared memory: rb holds y[i0..], cb y[i0 + d_lo + jc..]
-    // (row i = i0 + lane)
-    __device__ __forceinline__ void load_smem(const float *rb, const float *cb, int lane)
-    {
-#pragma unroll
-        for (int q = 0; q < M; ++q) a[q] = rb[lane + q * TAU];
-#pragma unroll
-        for (int x = 0; x < D + (M - 1) * TAU; ++x) w[x] = cb[lane + x];
-    }
-    // vertical pass: row i, columns c_lo .. c_lo+D-1 (the same window for
-    // every lane); zeros outside the series
-    __device__ __forceinline__ void load_vert(const float *__restrict__ ys, int n, int ne, int i,
-                                              int c_lo, int)
-    {
-#pragma unroll
-        for (int q = 0; q < M; ++q) a[q] = i < ne ? __ldg(ys + i + q * TAU) : 0.f;
-#pragma unroll
-        for (int x = 0; x < D + (M - 1) * TAU; ++x)
-            w[x] = c_lo + x < n ? __ldg(ys + c_lo + x) : 0.f;
-    }
-    __device__ __forceinline__ void load_vert_fast(const float *__restrict__ ys, int i, int c_lo, int)
-    {
-#pragma unroll
-        for (int q = 0; q < M; ++q) a[q] = __ldg(ys + i + q * TAU);
-#pragma unroll
-        for (int x = 0; x < D + (M - 1) * TAU; ++x) w[x] = __ldg(ys + c_lo + x);
-    }
-    // cell (i, i + d_lo + j), or (i, c_lo + j) after load_vert; only called
-    // for cells inside the matrix
-    __device__ __forceinline__ float dist(const float *__restrict__, int j, int, int, int,
-                                          int) const
-    {
-        float diff[M];
-#pragma unroll
-        for (int q = 0; q < M; ++q) diff[q] = a[q] - w[j + q * TAU];
-        return maxnorm<M>(diff);
-    }
-};
-
-// Compile-time M, run-time tau: the row vector in registers, columns read per cell.
-template <int M, int D>
-struct BandTile<M, 0, D> {
-    float a[M];
-    __device__ __forceinline__ void load(const float *__restrict__ ys, int, int i, int,
-                                         int rows, int tau, int)
-    {
-        if (i < rows) {
-#pragma unroll
-            for (int q = 0; q < M; ++q) a[q] = __ldg(ys + i + q * tau);
-        }
-    }
-    __device__ __forceinline__ void load_fast(const float *__restrict__ ys, int i, int, int tau)
-    {
-#pragma unroll
-        for (int q = 0; q < M; ++q) a[q] = __ldg(ys + i + q * tau);
-    }
-    __device__ __forceinline__ void load_vert(const float *__restrict__ ys, int, int ne, int i, int,
-                                              int tau)
-    {
-        if (i < ne) {
-#pragma unroll
-            for (int q = 0; q < M; ++q) a[q] = __ldg(ys + i + q * tau);
-        }
-    }
-    __device__ __forceinline__ void load_vert_fast(const float *__restrict__ ys, int i, int, int tau)
-    {
-        load_fast(ys, i, 0, tau);
-    }
-    __device__ __forceinline__ float dist(const float *__restrict__ ys, int, int i, int dl,
-                                          int tau, int) const
-    {
-        const int j = i + dl;
-        float diff[M];
-#pragma unroll
-        for (int q = 0; q < M; ++q) diff[q] = a[q] - __ldg(ys + j + q * tau);
-        return maxnorm<M>(diff);
-    }
-};
-
-// Generic embedding: everything read per cell.
-template <int D>
-struct BandTile<0, 0, D> {
-    __device__ __forceinline__ void load(const float *, int, int, int, int, int, int) {}
-    __device__ __forceinline__ void load_fast(const float *, int, int, int) {}
-    __device__ __forceinline__ void load_vert(const float *, int, int, int, int, int) {}
-    __device__ __forceinline__ void load_vert_fast(const float *, int, int, int) {}
-    __device__ __forceinline__ float dist(const float *__restrict__ ys, int, int i, int dl,
-                                          int tau, int m) const
-    {
-        const int j = i + dl;
-        float d = fabsf(__ldg(ys + i) - __ldg(ys + j));
-        for (int q = 1; q < m; ++q)
-            d = fmaxf(d, fabsf(__ldg(ys + i + q * tau) - __ldg(ys + j + q * tau)));
-        return d;
-    }
-};
+// Distance of cell (i, i + dl), any embedding, read through L1.
+__device__ __forceinline__ float cell_dist(const float *__restrict__ ys, int i, int dl, int tau, int m)
+{
+    const int j = i + dl;
+    float d = fabsf(__ldg(ys + i) - __ldg(ys + j));
+    for (int q = 1; q < m; ++q)
+        d = fmaxf(d, fabsf(__ldg(ys + i + q * tau) - __ldg(ys + j + q * tau)));
+    return d;
+}
 
 // Embedding variants with their own kernel instantiation.
-enum Embed : int { E_GENERIC = 0, E_M1 = 1, E_M2 = 2, E_M3 = 3, E_M4 = 4,
+enum Embed : int { E_GENERIC = 0, E_M2 = 2, E_M3 = 3, E_M4 = 4,
                    E_M1T1 = 11, E_M3T1 = 31, E_M3T3 = 33 };
 
 // Host: CTAs of `kern` (THREADS threads, `smem` dynamic bytes) resident per
