@@ -157,7 +157,7 @@ struct Plan {
     Split lsplit{};                          // line-pass units of the batch ...
     std::vector<Split> lsplit1;              // ... and of each series alone
     std::vector<int64_t> uprefix;            // S+1 unit-count prefix along order
-    int32_t ne_max = 0, n_max = 0;           // largest Ne and N of the batch
+    int32_t ne_max = 0, n_max = 0, m_max = 0;  // largest Ne, N and m of the batch
     bool small = false;                      // short series: selected by one CTA each
     std::vector<int32_t> ident;              // 0..S-1
     std::vector<int64_t> uprefix1;           // [2s], [2s+1] = 0, units of s alone
@@ -298,6 +298,7 @@ int make_plan(rqa_ctx *c, const rqa_batch *b, const int32_t *rr_num, int32_t rr_
     for (int s = 0; s < S; ++s) {
         pl.ne_max = std::max(pl.ne_max, pl.sd[s].ne);
         pl.n_max = std::max(pl.n_max, pl.sd[s].n);
+        pl.m_max = std::max(pl.m_max, pl.sd[s].m);
     }
     pl.small = small_select_ok(K, pl.ne_max, pl.n_max, total_cells, c->sm_count);
     // warp work units of the line pass
@@ -461,6 +462,7 @@ CellArgs cell_args(rqa_ctx *c, const Plan &pl, int s, bool lines = false)
     a.y = pl.y;
     a.series = pl.d_sd;
     a.status = P<int>(c->status);
+    a.m_max = pl.m_max;
     const Split sp = lines ? (s < 0 ? pl.lsplit : pl.lsplit1[s]) : (s < 0 ? pl.split : pl.split1[s]);
     a.nb = sp.nb;
     a.rc = sp.rc;

@@ -68,8 +68,8 @@ k_count_grid(CellArgs a, const float *__restrict__ thr, int n_thr, uint64_t *his
     __shared__ int next_band;
     __shared__ uint32_t sink[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t *win = reinterpret_cast<uint32_t *>(smem) + warp * WIN_WORDS;
-    uint32_t *h = reinterpret_cast<uint32_t *>(smem) + (GT / 32) * WIN_WORDS;  // bin r + 1; bin 0 belongs to r = 0
+    uint32_t *win = reinterpret_cast<uint32_t *>(smem) + warp * Src::WORDS;
+    uint32_t *h = reinterpret_cast<uint32_t *>(smem) + (GT / 32) * Src::WORDS;  // bin r + 1; bin 0 belongs to r = 0
     uint32_t *tk = h + n_thr + 2;  // keys of thr_0 = 0, thr_1, .., thr_n
     for (int x = threadIdx.x; x < n_thr + 2; x += GT) h[x] = 0;
     int cur = -1;
@@ -231,20 +231,23 @@ cudaError_t launch_grid_select(const CellArgs &a, int S, int n_thr, float *thr, 
                                cudaStream_t st)
 {
     if (!a.y || !a.series || !a.order || !a.uprefix || !a.queue || a.n_units < 1 || a.n_pos < 1 ||
-        a.nb < 1 || a.rc < RB || a.rc % RB || S < 1 || n_thr < 1 || n_thr > 1024 || !thr || !hist || !rr_num_dev || K < 1 || K > KMAX || !eps_out ||
+        a.m_max < 1 || a.nb < 1 || a.rc < RB || a.rc % RB || S < 1 || n_thr < 1 || n_thr > 1024 || !thr || !hist || !rr_num_dev || K < 1 || K > KMAX || !eps_out ||
         grid < 1)
         return cudaErrorInvalidValue;
     k_grid_thr<<<S, GT, 0, st>>>(a.y, a.series, n_thr, thr);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int smem = ((GT / 32) * WIN_WORDS + 2 * n_thr + 3) * 4;
     void (*kern)(CellArgs, const float *, int, uint64_t *);
+    int words = WIN_WORDS;
     switch (embed) {
     case E_M1T1: kern = k_count_grid<DiagSrc<1, 1>>; break;
     case E_M3T1: kern = k_count_grid<DiagSrc<3, 1>>; break;
     case E_M3T3: kern = k_count_grid<DiagSrc<3, 3>>; break;
-    default: kern = k_count_grid<GenSrc>; break;
+    default:
+        kern = a.m_max <= WinSrc::MAXM ? k_count_grid<WinSrc> : k_count_grid<GenSrc>;
+        words = a.m_max <= WinSrc::MAXM ? WinSrc::WORDS : GenSrc::WORDS;
     }
+    const int smem = ((GT / 32) * words + 2 * n_thr + 3) * 4;
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
         return e;
     grid = persistent_cap(reinterpret_cast<const void *>(kern), smem, grid, GT);

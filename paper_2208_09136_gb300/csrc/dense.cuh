@@ -72,6 +72,7 @@ template <int M, int TAU>
 struct DiagSrc {
     static constexpr int H = (M - 1) * TAU, RS = 8;
     static_assert(H < RS, "history rows");
+    static constexpr int WORDS = WIN_WORDS;  // shared memory per warp
     float e[RS][DPL];
     float pc[COLW / 32], pr;  // the next block's windows on their way from memory
     float4 c0;
@@ -160,6 +161,7 @@ struct DiagSrc {
 // one three-input maximum serves both.  CHECK: indexes past the series are
 // pulled back to its last value (the caller discards those cells).
 struct GenSrc {
+    static constexpr int WORDS = 0;
     const float *ys;
     int n, d0, lane, m, tau;
 
@@ -228,6 +230,87 @@ struct GenSrc {
 // compile-time true inside the triangle and a run-time mask (bit 4 r + j) in
 // blocks that reach over its edge.  f sees sixteen cells at once so that it
 // can issue their lookups together before it uses any.
+// Any embedding with at most MAXM coordinates: a window of rows and one of
+// columns per coordinate in shared memory, so that four rows of a lane's
+// sixteen cells take three 16-byte loads per coordinate, nine wavefronts.
+// Through L1 (GenSrc) the column reads of one coordinate are seven loads that
+// stride over four lines each, 28 wavefronts, and bind the rounds: four series
+// of 2e4 samples, all rounds, m = 2, 4, 5, 6: 1.62, 2.61, 3.14, 3.65 ms through
+// L1 and 1.28, 1.87, 2.16, 2.47 ms here.  Six windows are the most that leave
+// two CTAs on an SM; larger m keeps GenSrc.
+struct WinSrc {
+    static constexpr int MAXM = 6, WORDS = MAXM * WIN_WORDS;
+    const float *ys;
+    int n, d0, lane, m, tau;
+    float *win;  // [q]: COLW columns, ROWW rows
+
+    __device__ __forceinline__ void init(const float *y, const SeriesDev &sd, int lane_, uint32_t *w)
+    {
+        ys = y;
+        n = sd.n;
+        m = sd.m;
+        tau = sd.tau;
+        lane = lane_;
+        win = reinterpret_cast<float *>(w);
+    }
+    __device__ __forceinline__ void begin(int d, int) { d0 = d; }
+    __device__ __forceinline__ void enter(int i0)
+    {
+        __syncwarp();
+        for (int q = 0; q < m; ++q) {
+            float *w = win + q * WIN_WORDS + lane;
+            const int r = i0 + q * tau + lane, c = r + d0;
+            float v[COLW / 32 + 1];
+#pragma unroll
+            for (int x = 0; x < COLW / 32; ++x) v[x] = __ldg(ys + min(c + 32 * x, n - 1));
+            v[COLW / 32] = __ldg(ys + min(r, n - 1));
+#pragma unroll
+            for (int x = 0; x <= COLW / 32; ++x) w[32 * x] = v[x];
+        }
+        __syncwarp();
+    }
+    __device__ __forceinline__ void diff(const float *w, int u, float (&x)[4][DPL]) const
+    {
+        const float4 c0 = *reinterpret_cast<const float4 *>(w + 4 * u + DPL * lane);
+        const float4 c1 = *reinterpret_cast<const float4 *>(w + 4 * u + 4 + DPL * lane);
+        const float4 r4 = *reinterpret_cast<const float4 *>(w + COLW + 4 * u);
+        const float rv[4] = {r4.x, r4.y, r4.z, r4.w};
+        const float cv[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int j = 0; j < DPL; ++j) x[r][j] = rv[r] - cv[r + j];
+    }
+    template <bool CHECK, int PH>
+    __device__ __forceinline__ void quad(int u, int, float (&d)[4][DPL])
+    {
+        diff(win, u, d);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int j = 0; j < DPL; ++j) d[r][j] = fabsf(d[r][j]);
+        int q = 1;
+        for (; q + 1 < m; q += 2) {
+            float a[4][DPL], b[4][DPL];
+            diff(win + q * WIN_WORDS, u, a);
+            diff(win + (q + 1) * WIN_WORDS, u, b);
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int j = 0; j < DPL; ++j) d[r][j] = fmax3(d[r][j], fabsf(a[r][j]), fabsf(b[r][j]));
+        }
+        if (q < m) {
+            float a[4][DPL];
+            diff(win + q * WIN_WORDS, u, a);
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int j = 0; j < DPL; ++j) d[r][j] = fmaxf(d[r][j], fabsf(a[r][j]));
+        }
+    }
+    __device__ __forceinline__ void leave() {}
+};
+
 // A block's steps of four rows: q(phase, u) for u = 0 .. 6.
 template <class Q>
 __device__ __forceinline__ void each_quad(Q &&q)

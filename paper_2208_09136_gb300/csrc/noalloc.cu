@@ -233,6 +233,7 @@ extern "C" int rqa_eps_for_rr_noalloc(const rqa_batch *b, const int32_t *rr_num,
     a.order = reinterpret_cast<const int32_t *>(scr + O_ORDER);
     a.uprefix = reinterpret_cast<const int64_t *>(scr + O_UPREFIX);
     a.n_pos = pl.S;
+    for (int s = 0; s < pl.S; ++s) a.m_max = std::max(a.m_max, pl.sd[s].m);
     a.nb = split.nb;
     a.rc = split.rc;
     a.n_units = pl.uprefix[pl.S];

@@ -71,6 +71,7 @@ struct CellArgs {
     const int32_t *order;    // series, largest first
     const int64_t *uprefix;  // n_pos + 1 prefix of unit counts along order
     int32_t n_pos;
+    int32_t m_max;           // largest embedding dimension of the batch
     int32_t nb, rc;          // bands per unit and rows per unit (a multiple of the kernel's row block)
     int32_t line_ctas;       // persistent CTAs of the line pass per SM (0: as many as fit)
     int64_t n_units;
@@ -160,8 +161,5 @@ cudaError_t launch_lam_tt(const uint64_t *hist, const int64_t *hoff_dev, int S, 
                           double *lam_avg, double *tt_avg, cudaStream_t st);
 cudaError_t launch_finalize_hist(const LineBufs &lb, const SeriesDev *series, int S, int K,
                                  uint64_t *stencil, cudaStream_t st);
-
-// Largest dynamic shared memory a count round needs for K thresholds.
-int count_smem_bytes(int round, int K);
 
 }  // namespace rqa

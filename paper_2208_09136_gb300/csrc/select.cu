@@ -59,9 +59,9 @@ static int count_bins(int round, int K)
     }
 }
 
-int count_smem_bytes(int round, int K)
+static int count_smem_bytes(int round, int K, int win_words)
 {
-    const int win = CW * WIN_WORDS * 4;
+    const int win = CW * win_words * 4;
     switch (round) {
     case R_COARSE: return win + NCOARSE * 4;
     case R_COARSE_SUB: case R_MID: return win + count_bins(round, K) * 4 + NCOARSE;
@@ -107,8 +107,8 @@ __global__ void __launch_bounds__(CT, 2) k_count(CellArgs a, SelBufs sb, int K, 
     __shared__ int n_pfx;
     __shared__ unsigned fbits[4];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t *win = reinterpret_cast<uint32_t *>(smem) + warp * WIN_WORDS;
-    uint32_t *h = reinterpret_cast<uint32_t *>(smem) + CW * WIN_WORDS;
+    uint32_t *win = reinterpret_cast<uint32_t *>(smem) + warp * Src::WORDS;
+    uint32_t *h = reinterpret_cast<uint32_t *>(smem) + CW * Src::WORDS;
     int8_t *t1 = reinterpret_cast<int8_t *>(h + nbins);                   // sparse ranges
     unsigned char *t8 = reinterpret_cast<unsigned char *>(h);             // final round, byte table
     uint32_t *th = h;                                                     // final round, hashed table
@@ -367,14 +367,24 @@ template <int ROUND>
 static cudaError_t launch_count_m(const CellArgs &a, const SelBufs &sb, int K, int grid,
                                   int embed, cudaStream_t st)
 {
-    const int smem = count_smem_bytes(ROUND, K);
     void (*kern)(CellArgs, SelBufs, int, int);
+    int words = WIN_WORDS;
     switch (embed) {
     case E_M1T1: kern = k_count<ROUND, DiagSrc<1, 1>>; break;
     case E_M3T1: kern = k_count<ROUND, DiagSrc<3, 1>>; break;
     case E_M3T3: kern = k_count<ROUND, DiagSrc<3, 3>>; break;
-    default: kern = k_count<ROUND, GenSrc>; break;
+    default:
+        // the bracket and middle rounds' bins leave no room for windows per
+        // coordinate beside a second CTA on the SM
+        if ((ROUND == R_COARSE || ROUND == R_FINAL) && a.m_max <= WinSrc::MAXM) {
+            kern = k_count<ROUND, WinSrc>;
+            words = WinSrc::WORDS;
+        } else {
+            kern = k_count<ROUND, GenSrc>;
+            words = GenSrc::WORDS;
+        }
     }
+    const int smem = count_smem_bytes(ROUND, K, words);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     grid = persistent_cap(reinterpret_cast<const void *>(kern), smem, grid, CT);
@@ -386,7 +396,7 @@ cudaError_t launch_count(int round, const CellArgs &a, const SelBufs &sb, int K,
                          int embed, cudaStream_t st)
 {
     if (!a.y || !a.series || !a.order || !a.uprefix || !a.queue || !a.status || !sb.hist || K < 1 ||
-        K > KMAX || grid < 1 || a.n_units < 1 || a.n_units > 0x7fffffff || a.n_pos < 1 || a.nb < 1 ||
+        K > KMAX || grid < 1 || a.n_units < 1 || a.n_units > 0x7fffffff || a.n_pos < 1 || a.m_max < 1 || a.nb < 1 ||
         a.rc < RB || a.rc % RB)
         return cudaErrorInvalidValue;
     if (round == R_MID && (a.g0 < 0 || a.gn < 1 || a.gn > MID_GROUPS)) return cudaErrorInvalidValue;
