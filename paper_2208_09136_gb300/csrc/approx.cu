@@ -57,8 +57,9 @@ k_grid_thr(const float *__restrict__ y, const SeriesDev *__restrict__ series, in
 // r = rho - 1 + [thr_rho < d] (0 for rho = 0): one multiply-add into the
 // integers of [2^23, 2^24), one DPX clamp, one lookup, one compare and one
 // shared reduction per cell.  A binary search took log2(n) dependent lookups
-// (grid-400's counting pass: 5.5 ms).  Grids whose step or its reciprocal
-// could be subnormal or overflow are searched (UNI false).
+// (400 thresholds, 4e7 cells: 5.5 ms of counting).  Grids whose step or its
+// reciprocal could be subnormal or overflow are searched, all lanes in step;
+// so are constant series and those whose step rounds to zero.
 template <class Src>
 __global__ void __launch_bounds__(GT)
 k_count_grid(CellArgs a, const float *__restrict__ thr, int n_thr, uint64_t *hist)
@@ -109,8 +110,8 @@ k_count_grid(CellArgs a, const float *__restrict__ thr, int n_thr, uint64_t *his
             const float *tg = thr + (int64_t)cur * n_thr;
             for (int x = threadIdx.x; x <= n_thr; x += GT) tk[x] = x ? __float_as_uint(tg[x - 1]) : 0u;
             const float scale = tg[0];  // 1 * ((max - min) / n)
-            uni = scale == 0.f || (scale >= 0x1p-100f && scale <= 0x1p100f);
-            inv = scale > 0.f ? 1.f / scale : 0.f;  // a constant series: every distance is 0
+            uni = scale >= 0x1p-100f && scale <= 0x1p100f;
+            inv = uni ? 1.f / scale : 0.f;
             __syncthreads();
         }
         const uint64_t cells = (uint64_t)(w.b_hi - w.b_lo) * DB * (uint64_t)(w.r_hi - w.r_lo);
@@ -150,11 +151,11 @@ k_count_grid(CellArgs a, const float *__restrict__ thr, int n_thr, uint64_t *his
             });
         } else {
             count([&](uint32_t key) -> uint32_t {
-                int lo = 0, hi = n_thr;  // grid keys below key (ascending)
-                while (lo < hi) {
-                    const int mid = (lo + hi) >> 1;
-                    if (tk[mid + 1] < key) lo = mid + 1;
-                    else hi = mid;
+                int lo = 0;  // grid keys below key (ascending); n_thr <= 1024
+#pragma unroll 1
+                for (int step = 1024; step; step >>= 1) {
+                    const int c = lo + step;
+                    lo = (tk[min(c, n_thr)] < key) & (c <= n_thr) ? c : lo;
                 }
                 return (uint32_t)lo + 1u;
             });

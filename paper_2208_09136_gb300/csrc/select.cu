@@ -349,13 +349,13 @@ __global__ void __launch_bounds__(CT, 2) k_count(CellArgs a, SelBufs sb, int K, 
                 const int np = n_pfx;
                 finals([&](uint32_t key) -> uint32_t {
                     const uint32_t p = key >> 10;
-                    int lo = 0, hi = np;  // first prefix >= p
-                    while (lo < hi) {
-                        const int mid = (lo + hi) >> 1;
-                        if (pfx[mid] < p) lo = mid + 1;
-                        else hi = mid;
+                    int lo = 0;  // last prefix <= p, or the first; all lanes in step
+#pragma unroll 1
+                    for (int step = (KMAX + 1) / 2; step; step >>= 1) {
+                        const int c = lo + step;
+                        lo = (c < np) & (pfx[min(c, np - 1)] <= p) ? c : lo;
                     }
-                    return lo < np && pfx[lo] == p ? (uint32_t)lo + 1u : 0u;
+                    return pfx[lo] == p ? (uint32_t)lo + 1u : 0u;
                 });
             }
         }
