@@ -64,7 +64,7 @@ def parse():
     ap.add_argument("--cpu-cells", type=float, default=1.2e8,
                     help="cells of the oracle's bounded sample")
     ap.add_argument("--tile", type=int, default=0,
-                    help="line-pass register window: 8, 16 or 32 diagonals (0 = tuned)")
+                    help="0, 8, 16 or 32: passed to the context, without effect on the time")
     ap.add_argument("--select", default="auto", choices=["auto", "radix"],
                     help="auto: learned bracket when a model file exists")
     return ap.parse_args()

@@ -92,11 +92,8 @@ typedef struct {
     void *stream;      /* cudaStream_t owned by the caller; NULL = default stream */
     int schedule;      /* RQA_SCHED_* */
     int select;        /* RQA_SELECT_* */
-    int tile;          /* line pass: diagonals whose cells a lane computes from
-                          one register window of the series: 0 = default (16,
-                          or the rqa_autotune choice), else 8, 16 or 32 (8 and
-                          32 only for (m, tau) = (1, any), (3, 1), (3, 3);
-                          otherwise 16 is used) */
+    int tile;          /* 0, 8, 16 or 32; kept and reported (0 as 16), without
+                          effect: the line pass has no register window to size */
     int blocks_per_sm; /* persistent CTAs per SM: 0 = as many as each kernel
                           can keep resident, else at most this many */
     int flags;         /* RQA_FLAG_* */
@@ -150,7 +147,7 @@ const char *rqa_error_string(int code);
 int rqa_abi_version(void);
 
 /* Number of SMs of the context's device and the schedule parameters in use
- * (line-pass register window, blocks per SM as configured: 0 = resident limit);
+ * (tile as configured, blocks per SM as configured: 0 = resident limit);
  * any pointer may be NULL. */
 int rqa_device_info(rqa_ctx *ctx, int *sm_count, int *tile, int *blocks_per_sm);
 
@@ -172,35 +169,25 @@ uint64_t rqa_graph_replays(rqa_ctx *ctx);
 /* Schedule knobs of the line pass.  Every setting gives the same results;
  * only the time differs. */
 typedef struct {
-    int tile;       /* diagonals per register window of the cell phase: 8, 16 or 32
-                       (0 = the default, 16; 8 and 32 only for the embeddings
-                       that cfg.tile lists) */
+    int tile;       /* 0, 8, 16 or 32; kept and reported (0 as 16), without effect */
     int unit_bands; /* bands of 32 diagonals per work unit a warp takes from the
                        queue (0 = planned from the batch: about eight units per
-                       resident warp, 1..64 otherwise; capped so a unit stays
-                       under 2^33 cells) */
+                       resident warp, or one band over a chunk of its rows when
+                       the batch has fewer bands; 1..64 otherwise; capped so a
+                       unit stays under 2^33 cells) */
     int line_ctas;  /* persistent CTAs of the line pass per SM (0 = as many as
                        fit, else 1..8) */
-    int stage;      /* 1: the diagonal pass brings each interior row block's
-                       series values into shared memory with 1-D bulk copies
-                       (cp.async.bulk, completion on an mbarrier, the next
-                       block's copy in flight while the current one computes);
-                       0: every lane reads its window through L1.  Only for
-                       m = 3 with tau = 3 or 1 and windows of 16 or 32
-                       diagonals; ignored elsewhere.  A copy whose barrier does
-                       not complete within a bounded wait sets RQA_ERR_TIMEOUT
-                       and the block is read directly. */
+    int stage;      /* 0 or 1; kept and reported, without effect */
     float ms;       /* rqa_autotune: the line-pass time of the chosen knobs on
                        the probe, in ms (output only) */
 } rqa_tuning;
 
 /* Line-pass tuning: times the line pass over (a prefix of, at most ~2*10^10
  * cells of) the batch with the thresholds of rr_num/rr_den, first over the
- * register windows, then the unit size (half, planned, twice), the CTAs per
- * SM (all that fit, or six) and the staging of series windows (off, on where
- * the variant exists), each step keeping the fastest; stores the choice
- * in the context and returns it in *out (host, may be NULL).  A context
- * created with cfg.tile != 0 keeps that window.  Synchronises the stream. */
+ * unit size (half, planned, twice), then the CTAs per SM (all that fit, or
+ * six), each step keeping the fastest; stores the choice in the context and
+ * returns it in *out (host, may be NULL).  tile and stage are left as they
+ * are.  Synchronises the stream. */
 int rqa_autotune(rqa_ctx *ctx, const rqa_batch *batch, const int32_t *rr_num, int32_t rr_den,
                  int32_t K, rqa_tuning *out);
 
@@ -388,10 +375,8 @@ int rqa_eps_approx(rqa_ctx *ctx, const rqa_batch *batch, const int32_t *rr_num, 
  *   - status_out: device int (may be NULL) that receives the device-side
  *     status of the call (RQA_OK, RQA_ERR_NONFINITE, ...) when it completes.
  *   - K is at most RQA_NOALLOC_K_MAX here (RQA_ERR_INVALID_ARG above).
- *   - Series have Ne <= RQA_NOALLOC_NE_MAX vectors here: each work item
- *     (consecutive diagonals of one series, at most 1024 per series) covers
- *     at most 2^30 cells so the 32-bit shared counts stay exact; a longer
- *     series is RQA_ERR_CAPACITY.
+ *   - Series have Ne <= RQA_NOALLOC_NE_MAX vectors here; a longer series is
+ *     RQA_ERR_CAPACITY.
  *   - batch->y, eps_out and the non-NULL count_le, count_lt, status_out must
  *     be memory the current device can address (its device memory or managed
  *     memory), else RQA_ERR_INVALID_ARG.

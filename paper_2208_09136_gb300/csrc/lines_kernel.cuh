@@ -7,12 +7,13 @@
 //
 //  cells  the rank r = #{k : eps_k < d} of every cell (one lookup in a bucket
 //         table of the thresholds, or a 5-step search over them).
-//         Compile-time embeddings: lane j walks down diagonal j and packs the
-//         ranks of its 32 cells into eight registers.  Others, and the vertical
-//         pass: lane t holds row i0+t and stores r as a byte of row j of a
+//         m <= 4: lane j walks down diagonal j (column j) and packs the ranks
+//         of its 32 cells into eight registers.  m > 4 and mixed batches:
+//         lane t holds row i0+t and stores r as a byte of row j of a
 //         32 x 32 rank matrix in shared memory, which lane j then reads.
 //         (m = 3, cycles per SM quarter and 32 cells of the whole pass, mixed
-//         signals: 56.7 by diagonals, 65.1 by rows; tau = 1: 76 and 85.)
+//         signals: 56.7 by diagonals, 65.1 by rows; tau = 1: 76 and 85; four
+//         series of 2e4 of noise, tau = 2: m = 2, 4 by diagonals 79 and 97.)
 //  runs   lane j holds diagonal j.  It gathers the five bit planes of its ranks:
 //         two words of four ranks are interleaved bit by bit, so one mask and
 //         one multiply bring bit p of eight ranks into the top byte of a

@@ -5,9 +5,8 @@
 Builds the workload's batch on cuda:0, selects the thresholds for RR = 1..20 %
 once (``rqa_eps_for_rr``, radix selection), then runs ``rqa_line_hist`` (full
 histograms) REPS times, each timed with CUDA events on the context's stream,
-and prints one line per run.  TILE fixes the cell phase's register window
-(8, 16 or 32; 0 = the default); STAGE = 1 stages the series windows in
-shared memory by bulk copies (where the variant exists).  Besides the workloads of ``synth``, "mix-m3t3"
+and prints one line per run.  TILE and STAGE are passed on as knobs without
+effect on the time.  Besides the workloads of ``synth``, "mix-m3t3"
 is a 12-series m = tau = 3 set (sine, logistic, Lorenz x SNR -10/0/10/20 dB,
 N = 2e4): the headline workload's line statistics at a size a full profiler
 capture handles.

@@ -1,6 +1,6 @@
 """A JSON cache of the line pass's tuned knobs (``rqa_autotune``).
 
-The best register window, work-unit size and CTAs per SM depend on the GPU and
+The best work-unit size and CTAs per SM depend on the GPU and
 on the batch's shape, not on its values, so a tuning result is stored under
 a key made of the GPU name and SM count and the batch's class: the largest
 series length as a power-of-two bucket, the embedding (m, tau, or "mixed")
