@@ -27,7 +27,12 @@ constexpr uint64_t SERIES_MULT = 0xD1B54A32D192ED03ull;
 // ------------------------------------------------------------ sketch
 // One CTA per series: 4096 random pairs, their distances sorted in shared
 // memory (bitonic network on the bit patterns), 128 quantiles, their logs.
-__global__ void __launch_bounds__(THREADS)
+// Bound by the latency of the network's 78 steps: 1024 threads take two
+// exchanges each per step, and steps of stride <= 32 stay inside a warp's 64
+// keys, so 28 of them end in a barrier of the CTA instead of all.
+constexpr int SKETCH_T = 1024;
+static_assert(SKETCH_PAIRS % (2 * SKETCH_T) == 0, "whole warps exchange in every step");
+__global__ void __launch_bounds__(SKETCH_T)
 k_sketch(const float *__restrict__ y, const SeriesDev *series, int s_base, uint64_t seed,
          float *feats, float *centre, float *qdist)
 {
@@ -37,7 +42,7 @@ k_sketch(const float *__restrict__ y, const SeriesDev *series, int s_base, uint6
     const SeriesDev sd = series[s];
     const float *ys = y + sd.off;
     const uint64_t ks = sm64_mix(seed ^ ((uint64_t)(s + 1) * SERIES_MULT));
-    for (int p = threadIdx.x; p < SKETCH_PAIRS; p += THREADS) {
+    for (int p = threadIdx.x; p < SKETCH_PAIRS; p += SKETCH_T) {
         const uint64_t a = sm64_mix(ks + (uint64_t)(2 * p + 1) * SM64_GAMMA);
         const uint64_t b = sm64_mix(ks + (uint64_t)(2 * p + 2) * SM64_GAMMA);
         const int i = (int)(a % (uint64_t)sd.ne);
@@ -52,7 +57,8 @@ k_sketch(const float *__restrict__ y, const SeriesDev *series, int s_base, uint6
     // bitonic sort, ascending
     for (int size = 2; size <= SKETCH_PAIRS; size <<= 1) {
         for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int t = threadIdx.x; t < SKETCH_PAIRS / 2; t += THREADS) {
+#pragma unroll
+            for (int t = threadIdx.x; t < SKETCH_PAIRS / 2; t += SKETCH_T) {
                 const int lo = 2 * t - (t & (stride - 1));
                 const int hi = lo + stride;
                 const bool up = (lo & size) == 0;
@@ -62,7 +68,9 @@ k_sketch(const float *__restrict__ y, const SeriesDev *series, int s_base, uint6
                     keys[hi] = x;
                 }
             }
-            __syncthreads();
+            // the next step's stride: half of this one, or the next size's first
+            if (stride > 32 || (stride > 1 ? stride >> 1 : size) > 32) __syncthreads();
+            else __syncwarp();
         }
     }
     const int t = threadIdx.x;
@@ -87,7 +95,7 @@ cudaError_t launch_sketch(const float *y, const SeriesDev *series, int s_base, i
                           uint64_t seed, float *feats, float *centre, float *qdist, cudaStream_t st)
 {
     if (!y || !series || !feats || S < 1) return cudaErrorInvalidValue;
-    k_sketch<<<S, THREADS, 0, st>>>(y, series, s_base, seed, feats, centre, qdist);
+    k_sketch<<<S, SKETCH_T, 0, st>>>(y, series, s_base, seed, feats, centre, qdist);
     return cudaGetLastError();
 }
 
@@ -401,13 +409,20 @@ cudaError_t launch_gather_rows(const float *src, const int64_t *idx, int n, int 
 // from the lowest to the highest end is split (and up to two below); else the
 // buckets nearest each target's middle bucket first, then the narrowest gaps
 // between split buckets.  Keys between the first and the last split bucket
-// are counted either way (unsplit buckets at coarse resolution).
-__global__ void k_bracket(const float *__restrict__ Yb, const float *__restrict__ centre,
+// are counted either way (unsplit buckets at coarse resolution).  One thread
+// marks them (a few dozen steps); all 256 number the marks, eight buckets each,
+// instead of one thread over the table's 2048 entries (with the sketch above:
+// bracket phase of four series of 1e4 225 -> 191 us).
+constexpr int BRACKET_T = 256;
+static_assert(NCOARSE == 8 * BRACKET_T, "eight buckets per thread");
+__global__ void __launch_bounds__(BRACKET_T)
+k_bracket(const float *__restrict__ Yb, const float *__restrict__ centre,
                           float margin, int K, const uint8_t *__restrict__ dom, int8_t *tab_sub,
                           int32_t *n_sub, uint32_t *range)
 {
     __shared__ uint16_t lo_b[KMAX], hi_b[KMAX], mid_b[KMAX];
-    __shared__ int8_t tb[NCOARSE];
+    __shared__ __align__(8) int8_t tb[NCOARSE];
+    __shared__ int wsum[BRACKET_T / 32];
     const int s = blockIdx.x;
     if (!dom[s]) {  // outside the network's domain: the full selection takes it
         int8_t *tab = tab_sub + (int64_t)s * NCOARSE;
@@ -455,7 +470,7 @@ __global__ void k_bracket(const float *__restrict__ Yb, const float *__restrict_
         } else {
             // rings around each target's most likely bucket, inside its
             // interval, all targets alike, until the split budget is spent
-            int used = 0;
+            int used = 0, first = NCOARSE - 1, last = 0;  // marked buckets
             for (int r = 0; used < NSUB_MAX; ++r) {
                 bool any = false;
                 for (int k = 0; k < K; ++k) {
@@ -467,15 +482,14 @@ __global__ void k_bracket(const float *__restrict__ Yb, const float *__restrict_
                         if (tb[b] != 0 && used < NSUB_MAX) {
                             tb[b] = 0;
                             ++used;
+                            first = min(first, b);
+                            last = max(last, b);
                         }
                     }
                 }
                 if (!any) break;
             }
             // the rest of the budget closes the narrowest gaps between them
-            int first = 0, last = NCOARSE - 1;
-            while (first < NCOARSE && tb[first] != 0) ++first;
-            while (last > first && tb[last] != 0) --last;
             for (;;) {
                 int best_a = -1, best_n = NCOARSE;
                 for (int b = first; b <= last; ++b) {
@@ -493,26 +507,50 @@ __global__ void k_bracket(const float *__restrict__ Yb, const float *__restrict_
                 used += best_n;
             }
         }
-        int g = 0;  // marked buckets numbered in ascending order
-        int first = -1, last = -1;
-        for (int b = 0; b < NCOARSE; ++b) {
-            if (tb[b] != 0) continue;
-            if (g < NSUB_MAX) {
-                tb[b] = (int8_t)(g++);
-                if (first < 0) first = b;
-                last = b;
-            } else {
-                tb[b] = -1;
-            }
-        }
-        n_sub[s] = g;
-        // keys the bracket round counts: from its first to its last split bucket
-        range[2 * s] = first < 0 ? 0xffffffffu : (uint32_t)first << COARSE_SHIFT;
-        range[2 * s + 1] = first < 0 ? 0u : (((uint32_t)last + 1u) << COARSE_SHIFT) - 1u;
     }
     __syncthreads();
+    // marked buckets numbered in ascending order; keys the bracket round counts:
+    // from its first to its last split bucket
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const uint2 eight = *reinterpret_cast<const uint2 *>(tb + 8 * t);
+    bool mark[8];
+    int own = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        mark[i] = (((i < 4 ? eight.x : eight.y) >> (8 * (i & 3))) & 0xffu) == 0u;
+        own += mark[i] ? 1 : 0;
+    }
+    int incl = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += u;
+    }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    int g = incl - own, total = 0;
+    for (int w = 0; w < BRACKET_T / 32; ++w) {
+        if (w < warp) g += wsum[w];
+        total += wsum[w];
+    }
+    total = min(total, NSUB_MAX);
     int8_t *tab = tab_sub + (int64_t)s * NCOARSE;
-    for (int x = threadIdx.x; x < NCOARSE; x += blockDim.x) tab[x] = tb[x];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const bool in = mark[i] && g < total;
+        const uint32_t b = (uint32_t)(8 * t + i);
+        tab[b] = in ? (int8_t)g : (int8_t)-1;
+        if (in && g == 0) range[2 * s] = b << COARSE_SHIFT;
+        if (in && g == total - 1) range[2 * s + 1] = ((b + 1u) << COARSE_SHIFT) - 1u;
+        g += mark[i] ? 1 : 0;
+    }
+    if (t == 0) {
+        n_sub[s] = total;
+        if (total == 0) {
+            range[2 * s] = 0xffffffffu;
+            range[2 * s + 1] = 0u;
+        }
+    }
 }
 
 cudaError_t launch_bracket(const float *Y, const float *centre, float margin, int S, int K,
@@ -520,7 +558,7 @@ cudaError_t launch_bracket(const float *Y, const float *centre, float margin, in
                            cudaStream_t st)
 {
     if (!dom) return cudaErrorInvalidValue;
-    k_bracket<<<S, 256, 0, st>>>(Y, centre, margin, K, dom, tab_sub, n_sub, range);
+    k_bracket<<<S, BRACKET_T, 0, st>>>(Y, centre, margin, K, dom, tab_sub, n_sub, range);
     return cudaGetLastError();
 }
 
