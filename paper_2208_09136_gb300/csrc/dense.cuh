@@ -235,11 +235,11 @@ struct GenSrc {
 // sixteen cells take three 16-byte loads per coordinate, nine wavefronts.
 // Through L1 (GenSrc) the column reads of one coordinate are seven loads that
 // stride over four lines each, 28 wavefronts, and bind the rounds: four series
-// of 2e4 samples, all rounds, m = 2, 4, 5, 6: 1.62, 2.61, 3.14, 3.65 ms through
-// L1 and 1.28, 1.87, 2.16, 2.47 ms here.  Six windows are the most that leave
-// two CTAs on an SM; larger m keeps GenSrc.
+// of 2e4 samples, all rounds, m = 2, 4, 6, 8: 1.62, 2.61, 3.65, 4.72 ms through
+// L1 and 1.28, 1.87, 2.47, 3.13 ms here.  Eight windows leave two CTAs on an
+// SM in the rounds that use them; larger m keeps GenSrc.
 struct WinSrc {
-    static constexpr int MAXM = 6, WORDS = MAXM * WIN_WORDS;
+    static constexpr int MAXM = 8, WORDS = MAXM * WIN_WORDS;
     const float *ys;
     int n, d0, lane, m, tau;
     float *win;  // [q]: COLW columns, ROWW rows

@@ -86,9 +86,9 @@ def test_counted_ranges(rqa_lib, m, tau, rr):
     _compare(ys, m, tau, rr)
 
 
-# windows per coordinate for m <= 6, samples through L1 above it; Ne around the
+# windows per coordinate for m <= 8, samples through L1 above it; Ne around the
 # 28-row blocks and 128-diagonal bands
-@pytest.mark.parametrize("m_max", [6, 7])
+@pytest.mark.parametrize("m_max", [6, 7, 8, 9])
 def test_mixed_embeddings(rqa_lib, m_max):
     rng = np.random.default_rng(m_max)
     ys, ms, taus = [], [], []
@@ -104,7 +104,7 @@ def test_mixed_embeddings(rqa_lib, m_max):
 # grids that one multiplication locates, and grids whose steps are lost in the
 # type's smallest values or overflow, which are searched
 @pytest.mark.parametrize("scale", [1e-42, 1e-38, 1e-20, 1.0, 1e30])
-@pytest.mark.parametrize("m,tau,n_thr", [(1, 1, 1024), (3, 3, 400), (2, 2, 1), (6, 1, 33), (7, 2, 100)])
+@pytest.mark.parametrize("m,tau,n_thr", [(1, 1, 1024), (3, 3, 400), (2, 2, 1), (6, 1, 33), (7, 2, 100), (8, 2, 100), (9, 1, 50)])
 def test_grid_of_any_scale(rqa_lib, scale, m, tau, n_thr):
     rqa = rqa_lib
     rng = np.random.default_rng(n_thr)
