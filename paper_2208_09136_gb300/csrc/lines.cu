@@ -26,7 +26,9 @@ static LinesKernel lines_kernel(int embed, bool vert, bool full)
 // one chunk and the first row of the next are both recurrent, the two counted
 // pieces x and y are one line of length x + y; a piece as long as its chunk
 // goes on to the next boundary.  The cells of the lines stay the same, so C_k
-// does.  One CTA per band, so that the loads of all bands are in flight.
+// does.  One CTA per band, so that the loads of all bands are in flight.  Only
+// edge lengths that k_lines wrote in this launch are read: it writes none for a
+// series that it skips.
 template <bool VERT>
 __global__ void __launch_bounds__(LD * KT) k_merge(CellArgs a, LineBufs lb, int K, const uint16_t *edges)
 {
@@ -35,51 +37,59 @@ __global__ void __launch_bounds__(LD * KT) k_merge(CellArgs a, LineBufs lb, int 
     const int t = threadIdx.x, lane = t % LD, k = t / LD;
     for (int i = t; i < LSH * KT; i += LD * KT) (&net[0][0])[i] = 0;
     if (t < KT) lmx[t] = 0;
-    for (int pos = blockIdx.y; pos < a.n_pos; pos += gridDim.y)
-    for (int b = blockIdx.x;; b += gridDim.x) {
+    for (int pos = blockIdx.y; pos < a.n_pos; pos += gridDim.y) {
         const int s = a.order[pos], ne = a.series[s].ne;
-        const int rows = VERT ? ne : ne - 1 - b * LD;
-        if ((VERT ? b * LD >= ne : rows <= 0) || a.rc >= rows) break;  // bands of one chunk have no boundary
         const int64_t o = (int64_t)s * lb.kstride + lb.k0;
-        const int64_t hrow = ne - 1 + (VERT && lb.loi ? 1 : 0);
-        uint64_t *hb = lb.hist && k < K ? lb.hist + lb.hist_off[s] + (int64_t)(lb.k0 + k) * hrow : nullptr;
-        __syncthreads();
-        auto add = [&](uint32_t len, bool more) {
-            if (len <= (uint32_t)LSH) atomicAdd(&net[len - 1][k], more ? 1u : ~0u);
-            else if (hb) atomicAdd(reinterpret_cast<unsigned long long *>(hb + (len - 1)), more ? 1ull : ~0ull);
-        };
-        if (k < K) {
-            int64_t base = a.uprefix[pos];       // first unit of the chunk
-            uint32_t open = 0;                   // length up to the boundary of the line that touches it
-            for (int r0 = 0; r0 < rows; r0 += a.rc) {
-                const uint16_t *e = edges + ((base + b / a.nb) * a.nb + b % a.nb) * (2 * KT * LD) + k * LD + lane;
-                const uint32_t y = r0 ? e[0] : 0u;
-                uint32_t z = r0 + a.rc < rows ? e[KT * LD] : 0u;
-                if (open && y) {
-                    add(open, false);
-                    add(y, false);
-                    add(open + y, true);
-                    atomicMax(&lmx[k], open + y);
-                    if (z == (uint32_t)a.rc) z += open;  // the whole chunk
+        bool ok = true;
+        if (t < K) {
+            const uint32_t v = threshold_key(lb.eps[o + t]);
+            ok = threshold_ok(v) && (t == 0 || threshold_key(lb.eps[o + t - 1]) <= v);
+        }
+        if (__syncthreads_or(!ok)) continue;  // skipped by k_lines
+        for (int b = blockIdx.x;; b += gridDim.x) {
+            const int rows = VERT ? ne : ne - 1 - b * LD;
+            if ((VERT ? b * LD >= ne : rows <= 0) || a.rc >= rows) break;  // bands of one chunk have no boundary
+            const int64_t hrow = ne - 1 + (VERT && lb.loi ? 1 : 0);
+            uint64_t *hb = lb.hist && k < K ? lb.hist + lb.hist_off[s] + (int64_t)(lb.k0 + k) * hrow : nullptr;
+            __syncthreads();
+            auto add = [&](uint32_t len, bool more) {
+                if ((int64_t)len > hrow) set_status(a.status, 10 /*INTERNAL*/);
+                else if (len <= (uint32_t)LSH) atomicAdd(&net[len - 1][k], more ? 1u : ~0u);
+                else if (hb) atomicAdd(reinterpret_cast<unsigned long long *>(hb + (len - 1)), more ? 1ull : ~0ull);
+            };
+            if (k < K) {
+                int64_t base = a.uprefix[pos];       // first unit of the chunk
+                uint32_t open = 0;                   // length up to the boundary of the line that touches it
+                for (int r0 = 0; r0 < rows; r0 += a.rc) {
+                    const uint16_t *e = edges + ((base + b / a.nb) * a.nb + b % a.nb) * (2 * KT * LD) + k * LD + lane;
+                    const uint32_t y = r0 ? e[0] : 0u;
+                    uint32_t z = r0 + a.rc < rows ? e[KT * LD] : 0u;
+                    if (open && y) {
+                        add(open, false);
+                        add(y, false);
+                        add(open + y, true);
+                        atomicMax(&lmx[k], open + y);
+                        if (z == (uint32_t)a.rc) z += open;  // the whole chunk
+                    }
+                    open = z;
+                    const int bands = VERT ? (ne + LD - 1) / LD : (ne - 1 - r0 + LD - 1) / LD;
+                    base += (bands + a.nb - 1) / a.nb;
                 }
-                open = z;
-                const int bands = VERT ? (ne + LD - 1) / LD : (ne - 1 - r0 + LD - 1) / LD;
-                base += (bands + a.nb - 1) / a.nb;
             }
-        }
-        __syncthreads();
-        for (int i = t; i < LSH * KT; i += LD * KT) {
-            const int l = i / KT, q = i - l * KT;
-            const int32_t v = (int32_t)net[l][q];
-            if (v) {
-                atomicAdd(reinterpret_cast<unsigned long long *>(lb.hshort + (o + q) * LSH + l),
-                          (unsigned long long)(long long)v);
-                net[l][q] = 0;
+            __syncthreads();
+            for (int i = t; i < LSH * KT; i += LD * KT) {
+                const int l = i / KT, q = i - l * KT;
+                const int32_t v = (int32_t)net[l][q];
+                if (v) {
+                    atomicAdd(reinterpret_cast<unsigned long long *>(lb.hshort + (o + q) * LSH + l),
+                              (unsigned long long)(long long)v);
+                    net[l][q] = 0;
+                }
             }
-        }
-        if (t < KT && lmx[t]) {
-            atomicMax(lb.lmax + o + t, lmx[t]);
-            lmx[t] = 0;
+            if (t < KT && lmx[t]) {
+                atomicMax(lb.lmax + o + t, lmx[t]);
+                lmx[t] = 0;
+            }
         }
     }
 }

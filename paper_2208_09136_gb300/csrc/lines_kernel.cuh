@@ -163,6 +163,16 @@ __device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane)
     return x;
 }
 
+// The key of a caller's threshold (-0 as +0), and whether it is one: neither
+// negative nor NaN.  The line pass skips a series with a threshold that is not,
+// or with thresholds that do not ascend (RQA_ERR_UNSORTED).
+__device__ __forceinline__ uint32_t threshold_key(float eps)
+{
+    const uint32_t v = __float_as_uint(eps);
+    return v == 0x80000000u ? 0u : v;
+}
+__device__ __forceinline__ bool threshold_ok(uint32_t v) { return !(v & 0x80000000u) && v <= 0x7f800000u; }
+
 // FK: a full sweep, K = KT thresholds known at compile time (the per-threshold
 // code then runs without a test of k against K); the argument is ignored.
 template <int M, int TAU, bool VERT, bool FK = false>
@@ -318,9 +328,8 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
             uint32_t v = 0xffffffffu;   // padding: above every key
             bool ok = true;
             if (klane) {
-                v = __float_as_uint(lb.eps[(int64_t)s * lb.kstride + lb.k0 + lane]);
-                if (v == 0x80000000u) v = 0u;                           // -0 == +0
-                if ((v & 0x80000000u) || v > 0x7f800000u) ok = false;  // negative or NaN
+                v = threshold_key(lb.eps[(int64_t)s * lb.kstride + lb.k0 + lane]);
+                ok = threshold_ok(v);
             }
             const uint32_t prev = __shfl_up_sync(FULL, v, 1);
             if (klane && lane > 0 && prev > v) ok = false;              // not ascending

@@ -1,0 +1,53 @@
+"""Calls at the limits of what the entry points accept: thresholds that the line
+pass rejects, several host threads, the longest series and the largest
+minibatches."""
+import numpy as np
+import pytest
+
+from oracle import c_oracle as CO
+from oracle import rqa_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+def _sine(n, period=628.0):
+    return np.sin(2 * np.pi * np.arange(n) / period).astype(np.float32)
+
+
+# Rows are cut into chunks from Ne = 257 on, and a second kernel joins the lines
+# at the cuts.  A series with rejected thresholds has none; its neighbours keep
+# theirs, whatever an earlier call left in the scratch.
+@pytest.mark.parametrize("bad", [[0.5, 0.2], [-0.5, 0.2], [0.2, np.nan]])
+@pytest.mark.parametrize("vertical,schedule", [(False, 0), (False, 1), (True, 0)])
+def test_rejected_thresholds_beside_valid_ones(rqa_lib, vertical, schedule, bad):
+    import torch
+    rqa = rqa_lib
+    ctx = rqa.Context(select=rqa.RQA_SELECT_RADIX, schedule=schedule)
+
+    def lines(ys, eps):
+        batch = rqa.Batch.from_numpy(ys, 1, 1)
+        e = torch.tensor(eps, dtype=torch.float32, device="cuda")
+        if vertical:
+            out = rqa.vline_hist(ctx, batch, e, 2)
+            out = {"hist": out["vhist"], "hist_offsets": out["vhist_offsets"], "lmax": out["vmax"], "count": out["vmass"]}
+        else:
+            out = rqa.line_hist(ctx, batch, e, 2)
+        code = rqa.rqa_status(ctx)
+        hist = rqa.unpack_hist(out["hist"].cpu().numpy(), out["hist_offsets"], batch, 2)
+        return code, hist, out["lmax"].cpu().numpy(), out["count"].cpu().numpy()
+
+    assert lines([_sine(3000)], [[0.1, 3.0]])[0] == 0  # long lines over every cut
+    good = [0.2, 0.5]
+    ys = [_sine(300), _sine(310), _sine(800)]
+    code, hist, lmax, count = lines(ys, [bad, good, bad])
+    assert code == 8
+    if vertical:
+        ref = O.vline_hist(ys[1], 1, 1, good)
+        assert np.array_equal(hist[1], ref["vhist"]) and np.array_equal(lmax[1], ref["vmax"])
+    else:
+        ref = CO.lines(ys[1], 1, 1, good)
+        assert np.array_equal(hist[1], ref["hist"]) and np.array_equal(lmax[1], ref["lmax"])
+        assert np.array_equal(count[1], ref["count"])
+    for s in (0, 2):
+        assert not hist[s].any() and not lmax[s].any() and not count[s].any(), s
+    ctx.close()
