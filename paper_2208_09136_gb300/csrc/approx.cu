@@ -21,7 +21,7 @@ k_grid_thr(const float *__restrict__ y, const SeriesDev *__restrict__ series, in
     const int s = blockIdx.x;
     const SeriesDev sd = series[s];
     float lo = 3.4e38f, hi = -3.4e38f;
-    for (int i = threadIdx.x; i < sd.n; i += GT) {
+    for (uint32_t i = threadIdx.x; i < (uint32_t)sd.n; i += GT) {  // n + GT may pass 2^31
         const float v = y[sd.off + i];
         lo = fminf(lo, v);
         hi = fmaxf(hi, v);

@@ -24,6 +24,8 @@ constexpr int RB = ROW_BLOCK;      // 28 rows per block: a multiple of 4 and of 
 constexpr int COLW = DB + RB + 4;  // column window of a block, in values
 constexpr int ROWW = 32;           // row window
 constexpr int WIN_WORDS = COLW + ROWW;  // 32-bit words of a warp's windows (16-byte multiples)
+// The windows reach up to 158 values past the end of a series, whose length
+// goes up to 2^31 - 65: an index that may pass the end is unsigned.
 static_assert(DB == 32 * DPL && RB % 4 == 0 && COLW % 32 == 0 && WIN_WORDS % 4 == 0, "band shape");
 
 // Work unit u of a launch: bands [b_lo, b_hi) of series s over rows
@@ -176,14 +178,14 @@ struct GenSrc {
     __device__ __forceinline__ void begin(int d, int) { d0 = d; }
     __device__ __forceinline__ void enter(int) {}
     template <bool CHECK>
-    __device__ __forceinline__ float at(int i) const
+    __device__ __forceinline__ float at(uint32_t i) const
     {
-        return __ldg(ys + (CHECK ? min(i, n - 1) : i));
+        return __ldg(ys + (CHECK ? min(i, (uint32_t)n - 1u) : i));
     }
     template <bool CHECK>
-    __device__ __forceinline__ void diff(int ri, float (&x)[4][DPL]) const
+    __device__ __forceinline__ void diff(uint32_t ri, float (&x)[4][DPL]) const
     {
-        const int ci = ri + d0 + DPL * lane;
+        const uint32_t ci = ri + (uint32_t)(d0 + DPL * lane);
         float rv[4], cv[3 + DPL];
 #pragma unroll
         for (int r = 0; r < 4; ++r) rv[r] = at<CHECK>(ri + r);
@@ -197,7 +199,7 @@ struct GenSrc {
     template <bool CHECK, int PH>
     __device__ __forceinline__ void quad(int u, int i0, float (&d)[4][DPL])
     {
-        const int i = i0 + 4 * u;
+        const uint32_t i = (uint32_t)(i0 + 4 * u);
         diff<CHECK>(i, d);
 #pragma unroll
         for (int r = 0; r < 4; ++r)
@@ -259,11 +261,12 @@ struct WinSrc {
         __syncwarp();
         for (int q = 0; q < m; ++q) {
             float *w = win + q * WIN_WORDS + lane;
-            const int r = i0 + q * tau + lane, c = r + d0;
+            const uint32_t r = (uint32_t)(q * tau) + (uint32_t)(i0 + lane);
+            const uint32_t c = r + (uint32_t)d0, end = (uint32_t)n - 1u;
             float v[COLW / 32 + 1];
 #pragma unroll
-            for (int x = 0; x < COLW / 32; ++x) v[x] = __ldg(ys + min(c + 32 * x, n - 1));
-            v[COLW / 32] = __ldg(ys + min(r, n - 1));
+            for (uint32_t x = 0; x < COLW / 32; ++x) v[x] = __ldg(ys + min(c + 32u * x, end));
+            v[COLW / 32] = __ldg(ys + min(r, end));
 #pragma unroll
             for (int x = 0; x <= COLW / 32; ++x) w[32 * x] = v[x];
         }

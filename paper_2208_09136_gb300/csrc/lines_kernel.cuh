@@ -521,11 +521,13 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                 auto walk_fetch = [&](int i0) {
 #pragma unroll
                     for (int q = 0; q < NW; ++q) {
-                        const int r = i0 + H + q * tau + lane, c = r + d_lo;
-                        pr[q] = r < sd.n ? __ldg(ys + r) : 0.f;
+                        // up to 94 values past the end: unsigned (dense.cuh)
+                        const uint32_t r = (uint32_t)(q * tau) + (uint32_t)(i0 + H + lane);
+                        const uint32_t c = r + (uint32_t)d_lo, n = (uint32_t)sd.n;
+                        pr[q] = r < n ? __ldg(ys + r) : 0.f;
                         if (!VERT) {
-                            pc[q][0] = c < sd.n ? __ldg(ys + c) : 0.f;
-                            pc[q][1] = c + 32 < sd.n ? __ldg(ys + c + 32) : 0.f;
+                            pc[q][0] = c < n ? __ldg(ys + c) : 0.f;
+                            pc[q][1] = c + 32u < n ? __ldg(ys + c + 32u) : 0.f;
                         }
                     }
                 };

@@ -51,3 +51,40 @@ def test_rejected_thresholds_beside_valid_ones(rqa_lib, vertical, schedule, bad)
     for s in (0, 2):
         assert not hist[s].any() and not lmax[s].any() and not count[s].any(), s
     ctx.close()
+
+
+# The longest series that are accepted: the walks look up to 158 values past the
+# end, so their indexes pass 2^31.  The same vectors stored without gaps are the
+# reference (m windows of Ne values, one after the other).  m: a window per
+# coordinate, rows of the line pass, values through L1.
+@pytest.mark.parametrize("m", [2, 5, 9])
+def test_longest_series(rqa_lib, m):
+    import torch
+    rqa = rqa_lib
+    n = (1 << 31) - 65
+    tau = (n - 300) // (m - 1)
+    ne = n - (m - 1) * tau
+    rng = np.random.default_rng(m)
+    z = rng.standard_normal(m * ne).astype(np.float32)
+    y = torch.zeros(n, dtype=torch.float32, device="cuda")
+    for q in range(m):
+        y[q * tau:q * tau + ne] = torch.from_numpy(z[q * ne:(q + 1) * ne]).cuda()
+    batch = rqa.Batch(y, np.array([0, n]), m, tau)
+    rr = [5, 30, 70]
+    ctx = rqa.Context(select=rqa.RQA_SELECT_RADIX)
+    sel = rqa.eps_for_rr(ctx, batch, rr, 100)
+    lines = rqa.line_hist(ctx, batch, sel["eps"], 3)
+    vert = rqa.vline_hist(ctx, batch, sel["eps"], 3)
+    grid = rqa.eps_approx(ctx, batch, rr, 100, 40)
+    assert rqa.rqa_status(ctx) == 0
+    ref = O.eps_for_rr(z, m, ne, rr, 100)
+    assert np.array_equal(sel["eps"].cpu().numpy()[0], ref["eps"])
+    assert np.array_equal(sel["count_le"].cpu().numpy()[0], ref["count_le"])
+    hist = CO.lines(z, m, ne, ref["eps"])["hist"]
+    assert np.array_equal(lines["hist"].cpu().numpy().reshape(3, -1), hist)
+    vhist = O.vline_hist(z, m, ne, ref["eps"])["vhist"]
+    assert np.array_equal(vert["vhist"].cpu().numpy().reshape(3, -1), vhist)
+    approx = O.eps_approx(z, m, ne, rr, 100, 40)
+    assert np.array_equal(grid["eps"].cpu().numpy()[0], approx["eps"])
+    assert np.array_equal(grid["count"].cpu().numpy()[0], approx["count"])
+    ctx.close()
