@@ -248,9 +248,9 @@ cudaError_t launch_grid_select(const CellArgs &a, int S, int n_thr, float *thr, 
         kern = a.m_max <= WinSrc::MAXM ? k_count_grid<WinSrc> : k_count_grid<GenSrc>;
         words = a.m_max <= WinSrc::MAXM ? WinSrc::WORDS : GenSrc::WORDS;
     }
-    const int smem = ((GT / 32) * words + 2 * n_thr + 3) * 4;
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
-        return e;
+    auto smem_of = [&](int n) { return ((GT / 32) * words + 2 * n + 3) * 4; };
+    const int smem = smem_of(n_thr);
+    if ((e = allow_smem(kern, smem_of(1024))) != cudaSuccess) return e;
     grid = persistent_cap(reinterpret_cast<const void *>(kern), smem, grid, GT);
     kern<<<grid, GT, smem, st>>>(a, thr, n_thr, hist);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;

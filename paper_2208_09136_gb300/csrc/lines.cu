@@ -105,7 +105,7 @@ static cudaError_t launch_lines_v(const CellArgs &a, const LineBufs &lb, int K, 
         return cudaErrorInvalidValue;
     LinesKernel kern = lines_kernel(embed, VERT, K == LINE_KMAX);
     const int smem = lines_smem_bytes();
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     grid *= WARPS / LWARPS;  // the caller counts CTAs of WARPS warps
     grid = persistent_cap(reinterpret_cast<const void *>(kern), smem, grid, LTHREADS);

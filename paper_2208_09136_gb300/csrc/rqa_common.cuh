@@ -70,6 +70,16 @@ __device__ __forceinline__ float cell_dist(const float *__restrict__ ys, int i, 
 enum Embed : int { E_GENERIC = 0, E_M2 = 2, E_M3 = 3, E_M4 = 4,
                    E_M1T1 = 11, E_M3T1 = 31, E_M3T3 = 33 };
 
+// Host: allow `kern` its dynamic shared memory.  The limit belongs to the
+// kernel, not to the call, so every launch sets the largest size that any call
+// needs (`most`): host threads with calls of different sizes would otherwise
+// lower it between each other's set and launch.
+template <class Kern>
+inline cudaError_t allow_smem(Kern kern, int most)
+{
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 // Host: CTAs of `kern` (THREADS threads, `smem` dynamic bytes) resident per
 // SM, and the SM count of the current device; both cached per host thread.
 inline int resident_per_sm(const void *kern, int smem, int threads = THREADS)

@@ -385,7 +385,7 @@ static cudaError_t launch_count_m(const CellArgs &a, const SelBufs &sb, int K, i
         }
     }
     const int smem = count_smem_bytes(ROUND, K, words);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem(kern, count_smem_bytes(ROUND, KMAX, words));
     if (e != cudaSuccess) return e;
     grid = persistent_cap(reinterpret_cast<const void *>(kern), smem, grid, CT);
     kern<<<grid, CT, smem, st>>>(a, sb, K, count_bins(ROUND, K));
@@ -932,7 +932,7 @@ cudaError_t launch_select_small(const float *y, const SeriesDev *series, int S, 
         n_max > 2 * SMALL_NE)
         return cudaErrorInvalidValue;
     const int smem = small_select_smem(n_max);
-    cudaError_t e = cudaFuncSetAttribute(k_select_small, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem(k_select_small, small_select_smem(2 * SMALL_NE));
     if (e != cudaSuccess) return e;
     k_select_small<<<S, SM_T, smem, st>>>(y, series, T, K, eps_out, le_out, lt_out, status);
     return cudaGetLastError();

@@ -88,3 +88,48 @@ def test_longest_series(rqa_lib, m):
     assert np.array_equal(grid["eps"].cpu().numpy()[0], approx["eps"])
     assert np.array_equal(grid["count"].cpu().numpy()[0], approx["count"])
     ctx.close()
+
+
+# One context per host thread: calls of different sizes, whose kernels take
+# different amounts of shared memory, at the same time.  The kernels of these
+# pairs differ in nothing else: short-series selection by the longest series,
+# the middle counting round by the targets, the grid count by the thresholds.
+@pytest.mark.parametrize("call", ["short", "middle", "grid"])
+def test_threads_with_calls_of_different_sizes(rqa_lib, call):
+    import threading
+
+    import torch
+    rqa = rqa_lib
+    rng = np.random.default_rng(5)
+    small, large = {"short": (100, 512), "middle": (25, 48), "grid": (8, 1024)}[call]
+    errors = []
+
+    def work(size, passes):
+        try:
+            n = size if call == "short" else 600
+            y = rng.standard_normal(2 * n).astype(np.float32)
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                ctx = rqa.Context(stream=stream, select=rqa.RQA_SELECT_RADIX)
+                batch = rqa.Batch.from_numpy([y], 2, n)
+                rr = list(range(1, 1 + (size if call == "middle" else 20)))
+                outs = []
+                for i in range(passes):
+                    if call == "grid":
+                        out = rqa.eps_approx(ctx, batch, rr, 100, size)
+                    else:
+                        out = rqa.eps_for_rr(ctx, batch, rr, 100)
+                    if i in (0, passes - 1):
+                        outs.append(out["eps"].clone())
+                assert rqa.rqa_status(ctx) == 0
+                assert torch.equal(outs[0], outs[1])
+                ctx.close()
+        except Exception as e:  # noqa: BLE001 - handed to the test's thread
+            errors.append((size, repr(e)))
+
+    threads = [threading.Thread(target=work, args=(size, 3000)) for size in (small, large)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
