@@ -498,7 +498,7 @@ int run_select(rqa_ctx *c, const Plan &pl, const SelBufs &sb, const CellArgs &ce
         if (int rc = check_cuda(mlp_forward(P<float>(c->mlp), feats, ns, ym, P<float>(c->acts),
                                             c->stream)))
             return rc;
-        c->launches += 3;
+        c->launches += 3 * mlp_row_launches(ns);
         if (int rc = launched(c, launch_bracket(ym, centre, c->margin, ns, K, pl.d_dom + s0,
                                                 sb.tab_sub + (int64_t)s0 * NCOARSE, sb.n_sub + s0,
                                                 sb.range + 2 * (int64_t)s0, c->stream)))
@@ -1314,7 +1314,7 @@ int rqa_mlp_forward(rqa_ctx *c, const float *params, const float *X, int32_t B, 
         if (int rc = ensure(c->learn_scratch, (size_t)B * 2 * HIDDEN * 4)) return rc;
         acts = P<float>(c->learn_scratch);
     }
-    c->launches += 3;
+    c->launches += 3 * mlp_row_launches(B);
     return check_cuda(mlp_forward(params, X, B, Y, acts, c->stream));
 }
 
@@ -1326,7 +1326,7 @@ int rqa_mlp_backward(rqa_ctx *c, const float *params, const float *X, const floa
     if (!(tau_lo > 0.f && tau_lo < 1.f && tau_hi > 0.f && tau_hi < 1.f)) return RQA_ERR_INVALID_ARG;
     cudaSetDevice(c->device);
     if (int rc = ensure(c->learn_scratch, (size_t)B * (MLP_OUT + 2 * HIDDEN) * 4)) return rc;
-    c->launches += 6;
+    c->launches += 4 + 2 * mlp_row_launches(B);  // the loss, three weight and two input gradients
     return check_cuda(mlp_backward(params, X, acts, Y, T, B, tau_lo, tau_hi, grads, loss,
                                    P<float>(c->learn_scratch), c->stream));
 }

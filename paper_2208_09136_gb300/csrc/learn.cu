@@ -114,6 +114,7 @@ cudaError_t launch_sketch(const float *y, const SeriesDev *series, int s_base, i
 // 64 x 64 tiles with sixteen values of K per step took 12 to 48 us and the
 // bias gradients three more launches of 16 us.
 constexpr int GT = 32, GK = 128, GG = 4;  // tile, panel of K, groups of threads along K
+static_assert(MLP_ROWS == 65535 * GT, "row tiles of a launch");
 
 template <bool TA, bool TB>
 __global__ void __launch_bounds__(256)
@@ -208,11 +209,27 @@ k_gemm(const float *__restrict__ A, const float *__restrict__ B, float *__restri
 static cudaError_t gemm(bool ta, bool tb, const float *A, const float *B, float *C, int M, int N,
                         int K, const float *bias, bool relu, const float *mask, float *rowsum, cudaStream_t st)
 {
-    dim3 grid((N + GT - 1) / GT, (M + GT - 1) / GT);
-    if (!ta && !tb) k_gemm<false, false><<<grid, 256, 0, st>>>(A, B, C, M, N, K, bias, relu, mask, rowsum);
-    else if (!ta && tb) k_gemm<false, true><<<grid, 256, 0, st>>>(A, B, C, M, N, K, bias, relu, mask, rowsum);
-    else k_gemm<true, false><<<grid, 256, 0, st>>>(A, B, C, M, N, K, bias, relu, mask, rowsum);
-    return cudaGetLastError();
+    // A launch's row tiles lie along gridDim.y, so more rows take more launches
+    // (only the products over a minibatch's rows have that many, never op(A) = A^T).
+    // All tiles along gridDim.x would need no loop, but the tile's division
+    // changed the code for the worse: backward pass of 65536 rows 6.02 ms, 4.91 so.
+    if (ta && M > MLP_ROWS) return cudaErrorInvalidValue;
+    for (int64_t m0 = 0; m0 < M; m0 += MLP_ROWS) {
+        const int rows = (int)std::min<int64_t>(M - m0, MLP_ROWS);
+        const dim3 grid((N + GT - 1) / GT, (rows + GT - 1) / GT);
+        const int64_t o = m0 * N;
+        const float *a = A + m0 * K, *mk = mask ? mask + o : nullptr;
+        if (ta) {
+            k_gemm<true, false><<<grid, 256, 0, st>>>(A, B, C, M, N, K, bias, relu, mask, rowsum);
+        } else if (tb) {
+            k_gemm<false, true><<<grid, 256, 0, st>>>(a, B, C + o, rows, N, K, bias, relu, mk, rowsum);
+        } else {
+            k_gemm<false, false><<<grid, 256, 0, st>>>(a, B, C + o, rows, N, K, bias, relu, mk, rowsum);
+        }
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 // Mean pinball loss of Y [B x 2K] against T [B x K] and its gradient.

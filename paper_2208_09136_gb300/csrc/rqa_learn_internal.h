@@ -14,6 +14,8 @@ constexpr int MLP_OUT = 40;   // 2 x 20 interval ends
 constexpr int MLP_K = 20;     // targets RR = 1..20 % the network predicts
 constexpr int64_t MLP_PARAMS = (int64_t)HIDDEN * FEATURES + HIDDEN + (int64_t)HIDDEN * HIDDEN +
                                HIDDEN + (int64_t)MLP_OUT * HIDDEN + MLP_OUT;
+constexpr int MLP_ROWS = 65535 * 32;  // rows per GEMM launch
+inline int mlp_row_launches(int B) { return (int)(((int64_t)B + MLP_ROWS - 1) / MLP_ROWS); }
 
 // series s_base .. s_base+S-1 of the batch (their rows of feats/centre/qdist)
 cudaError_t launch_sketch(const float *y, const SeriesDev *series, int s_base, int S,

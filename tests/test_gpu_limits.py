@@ -133,3 +133,54 @@ def test_threads_with_calls_of_different_sizes(rqa_lib, call):
     for t in threads:
         t.join()
     assert not errors, errors
+
+
+def test_network_on_millions_of_rows(rqa_lib):
+    """More rows than 65535 tiles of 32: nine rows repeated.  A row's outputs do
+    not depend on the others, so they are the small batch's bit for bit; the
+    gradients are means over the rows, so the small batch's but for rounding."""
+    import torch
+    rqa = rqa_lib
+    rep = 233017
+    B = 9 * rep  # 2097153
+    g = torch.Generator(device="cuda").manual_seed(4)
+    p = 0.05 * torch.randn(rqa.RQA_MLP_PARAMS, device="cuda", generator=g)
+    x = torch.randn((9, 131), device="cuda", generator=g)
+    t = torch.randn((9, 20), device="cuda", generator=g)
+    ctx = rqa.Context()
+
+    def run(X, T):
+        n = X.shape[0]
+        Y = torch.empty((n, 40), device="cuda")
+        acts = torch.empty(n * 512, device="cuda")
+        grads = torch.empty_like(p)
+        rqa.rqa_mlp_forward(ctx, p, X, Y, acts.view(n, 512))
+        rqa.rqa_mlp_backward(ctx, p, X, acts.view(n, 512), Y, T, 0.05, 0.95, grads)
+        return Y, acts, grads
+
+    Y, acts, grads = run(x.repeat(rep, 1), t.repeat(rep, 1))
+    y, a, _ = run(x, t)
+    assert rqa.rqa_status(ctx) == 0
+    assert torch.equal(Y, y.repeat(rep, 1))
+    for i in (0, 1):
+        h = acts[i * B * 256:(i + 1) * B * 256].view(rep, 9, 256)
+        assert torch.equal(h, a[i * 9 * 256:(i + 1) * 9 * 256].view(1, 9, 256).expand(rep, 9, 256))
+    # the gradients in 64 bits and, with absolute values throughout, the scale of
+    # their rounding: a sum of B rows by four partial sums is within
+    # (B / 4 + 1000) 2^-24 < 0.04 of it
+    W1, b1, W2, b2, W3, b3 = torch.split(p.double(), [256 * 131, 256, 256 * 256, 256, 40 * 256, 40])
+    W1, W2, W3 = W1.view(256, 131), W2.view(256, 256), W3.view(40, 256)
+    h1, h2 = a[:9 * 256].view(9, 256).double(), a[9 * 256:].view(9, 256).double()
+    q = torch.tensor([0.05, 0.95], device="cuda").double().repeat(20)
+    dY = torch.where(t.repeat_interleave(2, 1) >= y, -q, 1 - q) / (9 * 40)
+
+    def chain(dY, W3, W2, x):
+        dZ2 = (dY @ W3) * (h2 > 0)
+        dZ1 = (dZ2 @ W2) * (h1 > 0)
+        parts = (dZ1.T @ x, dZ1.sum(0), dZ2.T @ h1, dZ2.sum(0), dY.T @ h2, dY.sum(0))
+        return torch.cat([v.reshape(-1) for v in parts])
+
+    want = chain(dY, W3, W2, x.double())
+    scale = chain(dY.abs(), W3.abs(), W2.abs(), x.double().abs())
+    assert ((grads.double() - want).abs() <= 0.04 * scale).all()
+    ctx.close()
