@@ -543,8 +543,7 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                     }
                     walk_fetch(i0);
                 };
-                auto walk = [&](int i0, auto interior, uint32_t (&R)[8]) {
-                    constexpr bool INTERIOR = decltype(interior)::value;
+                auto walk = [&](int i0, uint32_t (&R)[8]) {
                     __syncwarp();
 #pragma unroll
                     for (int q = 0; q < NW; ++q) {
@@ -556,11 +555,6 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                     }
                     __syncwarp();
                     walk_fetch(i0 + 32);
-                    // rows of this block on the lane's diagonal (column); the
-                    // identity cell of a column, unless it counts
-                    const int col = c_lo + lane;
-                    const int lim = VERT ? (col < sd.ne ? sd.ne - i0 : 0) : sd.ne - d_lo - lane - i0;
-                    const int same = VERT && !lb.loi ? col - i0 : -1;
 #pragma unroll
                     for (int h = 0; h < 4; ++h) {
                         uint32_t key[8], r[8];
@@ -601,11 +595,6 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
 #pragma unroll
                             for (int t = 0; t < 8; ++t) r[t] = rank_of(key[t]);
                         }
-                        if (!INTERIOR) {
-#pragma unroll
-                            for (int t = 0; t < 8; ++t)
-                                r[t] = 8 * h + t < lim && (!VERT || 8 * h + t != same) ? r[t] : 31u;
-                        }
                         // the byte order of the rank matrix: even rows, odd rows
                         R[2 * h] = __byte_perm(__byte_perm(r[0], r[2], 0x0040), __byte_perm(r[4], r[6], 0x0040), 0x5410);
                         R[2 * h + 1] = __byte_perm(__byte_perm(r[1], r[3], 0x0040), __byte_perm(r[5], r[7], 0x0040), 0x5410);
@@ -614,8 +603,9 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                     }
                 };
 
-                // run phase of the same 32 rows: lane j takes diagonal j
-                auto run_phase = [&](int i0, const uint32_t (&R)[8]) {
+                // run phase of the same 32 rows: lane j takes diagonal j.  edge_block:
+                // the ranks may hold cells outside the matrix, which become 31
+                auto run_phase = [&](int i0, const uint32_t (&R)[8], bool edge_block) {
                     // Words 2h and 2h + 1 hold rows 8h .. 8h + 7 (byte u of word
                     // 2h: row 8h + 2u, of word 2h + 1: row 8h + 2u + 1).  X[h]
                     // interleaves their even bits (bit p of byte u of word 2h
@@ -644,6 +634,16 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                         const uint32_t lo = __byte_perm(v[0], v[1], 0x0073);
                         const uint32_t hi = __byte_perm(v[2], v[3], 0x7300);
                         B[p] = __byte_perm(lo, hi, 0x7610);
+                    }
+                    if (edge_block) {
+                        // rows that the lane's diagonal (column) does not have, and
+                        // the identity cell of a column unless it counts
+                        const int col = c_lo + lane;
+                        const int lim = VERT ? (col < sd.ne ? sd.ne - i0 : 0) : sd.ne - d_lo - lane - i0;
+                        uint32_t out = lim >= 32 ? 0u : FULL << max(lim, 0);
+                        if (VERT && !lb.loi && (uint32_t)(col - i0) < 32u) out |= 1u << (col - i0);
+#pragma unroll
+                        for (int p = 0; p < 5; ++p) B[p] |= out;
                     }
                     // this diagonal's planes, for rebuilding words of long lines
                     *reinterpret_cast<uint4 *>(pl + lane * 4) = make_uint4(B[0], B[1], B[2], B[3]);
@@ -706,23 +706,15 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                     long_lines(lmask);
                 };
 
-                // the packed tallies take SETTLE row blocks before a field could overflow
+                // One copy of the block's code for interior blocks and edges: the
+                // edges' ranks are corrected in the planes.  With a copy for each
+                // (and a select per cell) warps of short series alternated between
+                // the two, and both did not stay in the instruction cache: line pass
+                // over 10^4 series of 200, K = 13, m = 1, 2, 3 (tau = m): 0.83, 1.07,
+                // 0.92 ms with two copies, 0.50, 0.57, 0.55 with one (25 series of
+                // 2e4, K = 20: 6.6, 8.9, 6.9 and 6.5, 8.1, 6.9).
+                // The packed tallies take SETTLE row blocks before a field could overflow.
                 int i0 = un.r_lo;
-                auto block = [&](auto interior) {
-                    uint32_t R[8];
-                    if constexpr (WALK) {
-                        walk(i0, interior, R);
-                    } else {
-                        cell_phase(i0, interior);
-                        __syncwarp();
-                        const uint4 ra = *reinterpret_cast<const uint4 *>(rkm + lane * 32);
-                        const uint4 rb = *reinterpret_cast<const uint4 *>(rkm + lane * 32 + 16);
-                        R[0] = ra.x; R[1] = ra.y; R[2] = ra.z; R[3] = ra.w;
-                        R[4] = rb.x; R[5] = rb.y; R[6] = rb.z; R[7] = rb.w;
-                    }
-                    run_phase(i0, R);
-                    if (++nrb == SETTLE) settle();
-                };
                 if constexpr (WALK) walk_begin(i0);
                 for (; i0 < r_end; i0 += 32) {
                     // interior row blocks: every cell inside the matrix (and off the
@@ -730,8 +722,20 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                     const bool inside = VERT ? c_lo + LD <= sd.ne && i0 + 32 <= rows &&
                                                    (lb.loi || i0 + 32 <= c_lo || i0 >= c_lo + LD)
                                              : i0 + 32 <= rows - (LD - 1);
-                    if (inside) block(std::true_type{});
-                    else block(std::false_type{});
+                    uint32_t R[8];
+                    if constexpr (WALK) {
+                        walk(i0, R);
+                    } else {
+                        if (inside) cell_phase(i0, std::true_type{});
+                        else cell_phase(i0, std::false_type{});
+                        __syncwarp();
+                        const uint4 ra = *reinterpret_cast<const uint4 *>(rkm + lane * 32);
+                        const uint4 rb = *reinterpret_cast<const uint4 *>(rkm + lane * 32 + 16);
+                        R[0] = ra.x; R[1] = ra.y; R[2] = ra.z; R[3] = ra.w;
+                        R[4] = rb.x; R[5] = rb.y; R[6] = rb.z; R[7] = rb.w;
+                    }
+                    run_phase(i0, R, WALK && !inside);
+                    if (++nrb == SETTLE) settle();
                 }
                 // lines that reach the end of a diagonal, or of the chunk, exactly at
                 // a block's last row: a line of length c ending just above a word
