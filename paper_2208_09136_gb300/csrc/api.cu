@@ -54,6 +54,13 @@ int64_t units_of_series(int64_t ne, const Split &sp, bool vert, int w)
     return n;
 }
 
+int64_t cut_bands(int64_t ne, const Split &sp, bool vert)
+{
+    const int64_t rows = vert ? ne : ne - 1;
+    if (rows <= sp.rc) return 0;
+    return ((vert ? ne : rows - sp.rc) + LINE_BAND - 1) / LINE_BAND;
+}
+
 }  // namespace rqa
 
 namespace {
@@ -157,6 +164,7 @@ struct Plan {
     Split lsplit{};                          // line-pass units of the batch ...
     std::vector<Split> lsplit1;              // ... and of each series alone
     std::vector<int64_t> uprefix;            // S+1 unit-count prefix along order
+    std::vector<int64_t> mprefix, mprefix1;  // prefixes of the bands cut into row chunks, as uprefix / uprefix1
     int32_t ne_max = 0, n_max = 0, m_max = 0;  // largest Ne, N and m of the batch
     bool small = false;                      // short series: selected by one CTA each
     std::vector<int32_t> ident;              // 0..S-1
@@ -167,7 +175,8 @@ struct Plan {
     SeriesDev *d_sd = nullptr;
     uint64_t *d_T = nullptr;
     int32_t *d_order = nullptr, *d_ident = nullptr;
-    int64_t *d_uprefix = nullptr, *d_uprefix1 = nullptr, *d_cprefix = nullptr, *d_cprefix1 = nullptr;
+    int64_t *d_uprefix = nullptr, *d_uprefix1 = nullptr, *d_cprefix = nullptr, *d_cprefix1 = nullptr,
+            *d_mprefix = nullptr, *d_mprefix1 = nullptr;
     int32_t *d_lmin = nullptr;
     int64_t *d_hoff = nullptr;
     uint8_t *d_dom = nullptr;
@@ -292,9 +301,7 @@ int make_plan(rqa_ctx *c, const rqa_batch *b, const int32_t *rr_num, int32_t rr_
     }
     // units of the cell walk (counting rounds, grid search)
     pl.split = split_cells(total_cells, COUNT_NB, c->sm_count);
-    pl.split1.resize(S);
     pl.cprefix.assign(S + 1, 0);
-    pl.cprefix1.assign(2 * (size_t)S, 0);
     for (int s = 0; s < S; ++s) {
         pl.ne_max = std::max(pl.ne_max, pl.sd[s].ne);
         pl.n_max = std::max(pl.n_max, pl.sd[s].n);
@@ -307,23 +314,27 @@ int make_plan(rqa_ctx *c, const rqa_batch *b, const int32_t *rr_num, int32_t rr_
     int64_t total_bands = 0;
     for (int s = 0; s < S; ++s) total_bands += nbl(s);
     pl.lsplit = split_lines(cells_of(total_cells), total_bands, pl.ne_max, c->unit_bands, c->sm_count);
-    pl.lsplit1.resize(S);
     pl.order.resize(S);
     for (int s = 0; s < S; ++s) pl.order[s] = s;
     std::stable_sort(pl.order.begin(), pl.order.end(),
                      [&](int x, int y) { return pl.sd[x].P > pl.sd[y].P; });
     pl.uprefix.assign(S + 1, 0);
+    pl.mprefix.assign(S + 1, 0);
     for (int i = 0; i < S; ++i) {
+        pl.mprefix[i + 1] = pl.mprefix[i] + cut_bands(pl.sd[pl.order[i]].ne, pl.lsplit, vert);
         pl.uprefix[i + 1] = pl.uprefix[i] + units_of_series(pl.sd[pl.order[i]].ne, pl.lsplit, vert, LINE_BAND);
         pl.cprefix[i + 1] = pl.cprefix[i] + units_of_series(pl.sd[pl.order[i]].ne, pl.split, false);
     }
+    if (c->schedule != RQA_SCHED_PER_SERIES) return RQA_OK;
+    pl.split1.resize(S);
+    pl.lsplit1.resize(S);
     pl.ident.resize(S);
-    pl.uprefix1.resize(2 * (size_t)S);
+    for (auto *v : {&pl.cprefix1, &pl.uprefix1, &pl.mprefix1}) v->assign(2 * (size_t)S, 0);
     for (int s = 0; s < S; ++s) {
         pl.ident[s] = s;
         pl.lsplit1[s] = split_lines(cells_of(pl.sd[s].P), nbl(s), pl.sd[s].ne, c->unit_bands, c->sm_count);
-        pl.uprefix1[2 * s] = 0;
         pl.uprefix1[2 * s + 1] = units_of_series(pl.sd[s].ne, pl.lsplit1[s], vert, LINE_BAND);
+        pl.mprefix1[2 * s + 1] = cut_bands(pl.sd[s].ne, pl.lsplit1[s], vert);
         pl.split1[s] = split_cells(pl.sd[s].P, COUNT_NB, c->sm_count);
         pl.cprefix1[2 * s + 1] = units_of_series(pl.sd[s].ne, pl.split1[s], false);
     }
@@ -341,7 +352,9 @@ int upload_plan(rqa_ctx *c, Plan &pl, const int32_t *lmin, int n_lmin, const int
     const size_t o_upre = align16(o_order + pl.order.size() * sizeof(int32_t));
     const size_t o_ident = align16(o_upre + pl.uprefix.size() * sizeof(int64_t));
     const size_t o_upre1 = align16(o_ident + pl.ident.size() * sizeof(int32_t));
-    const size_t o_lmin = align16(o_upre1 + pl.uprefix1.size() * sizeof(int64_t));
+    const size_t o_mpre = align16(o_upre1 + pl.uprefix1.size() * sizeof(int64_t));
+    const size_t o_mpre1 = align16(o_mpre + pl.mprefix.size() * sizeof(int64_t));
+    const size_t o_lmin = align16(o_mpre1 + pl.mprefix1.size() * sizeof(int64_t));
     const size_t o_hoff = align16(o_lmin + (size_t)n_lmin * sizeof(int32_t));
     const size_t o_dom = align16(o_hoff + (hoff ? (size_t)(pl.S + 1) * sizeof(int64_t) : 0));
     const size_t total = align16(o_dom + pl.dom.size());
@@ -363,17 +376,22 @@ int upload_plan(rqa_ctx *c, Plan &pl, const int32_t *lmin, int n_lmin, const int
     if (int rc = ensure(c->arena, total)) return rc;
     c->graph_valid = false;  // the arena is about to hold another plan
     char *h = static_cast<char *>(c->h_stage);
-    std::memcpy(h + o_sd, pl.sd.data(), pl.sd.size() * sizeof(SeriesDev));
-    if (!pl.T.empty()) std::memcpy(h + o_T, pl.T.data(), pl.T.size() * sizeof(uint64_t));
-    std::memcpy(h + o_cpre, pl.cprefix.data(), pl.cprefix.size() * sizeof(int64_t));
-    std::memcpy(h + o_cpre1, pl.cprefix1.data(), pl.cprefix1.size() * sizeof(int64_t));
-    std::memcpy(h + o_order, pl.order.data(), pl.order.size() * sizeof(int32_t));
-    std::memcpy(h + o_upre, pl.uprefix.data(), pl.uprefix.size() * sizeof(int64_t));
-    std::memcpy(h + o_ident, pl.ident.data(), pl.ident.size() * sizeof(int32_t));
-    std::memcpy(h + o_upre1, pl.uprefix1.data(), pl.uprefix1.size() * sizeof(int64_t));
+    auto put = [&](size_t o, const auto &v) {
+        if (!v.empty()) std::memcpy(h + o, v.data(), v.size() * sizeof(v[0]));
+    };
+    put(o_sd, pl.sd);
+    put(o_T, pl.T);
+    put(o_cpre, pl.cprefix);
+    put(o_cpre1, pl.cprefix1);
+    put(o_order, pl.order);
+    put(o_upre, pl.uprefix);
+    put(o_ident, pl.ident);
+    put(o_upre1, pl.uprefix1);
+    put(o_mpre, pl.mprefix);
+    put(o_mpre1, pl.mprefix1);
     if (n_lmin) std::memcpy(h + o_lmin, lmin, (size_t)n_lmin * sizeof(int32_t));
     if (hoff) std::memcpy(h + o_hoff, hoff, (size_t)(pl.S + 1) * sizeof(int64_t));
-    std::memcpy(h + o_dom, pl.dom.data(), pl.dom.size());
+    put(o_dom, pl.dom);
     char *d = static_cast<char *>(c->arena.p);
     if (int rc = check_cuda(cudaMemcpyAsync(d, h, total, cudaMemcpyHostToDevice, c->stream))) return rc;
     if (int rc = check_cuda(cudaEventRecord(c->stage_done, c->stream))) return rc;
@@ -386,6 +404,8 @@ int upload_plan(rqa_ctx *c, Plan &pl, const int32_t *lmin, int n_lmin, const int
     pl.d_uprefix = reinterpret_cast<int64_t *>(d + o_upre);
     pl.d_ident = reinterpret_cast<int32_t *>(d + o_ident);
     pl.d_uprefix1 = reinterpret_cast<int64_t *>(d + o_upre1);
+    pl.d_mprefix = reinterpret_cast<int64_t *>(d + o_mpre);
+    pl.d_mprefix1 = reinterpret_cast<int64_t *>(d + o_mpre1);
     pl.d_lmin = reinterpret_cast<int32_t *>(d + o_lmin);
     pl.d_hoff = reinterpret_cast<int64_t *>(d + o_hoff);
     pl.d_dom = reinterpret_cast<uint8_t *>(d + o_dom);
@@ -471,9 +491,13 @@ CellArgs cell_args(rqa_ctx *c, const Plan &pl, int s, bool lines = false)
     if (s < 0) {
         a.uprefix = lines ? pl.d_uprefix : pl.d_cprefix;
         a.n_units = (lines ? pl.uprefix : pl.cprefix)[pl.S];
+        a.mprefix = pl.d_mprefix;
+        a.n_merge = pl.mprefix[pl.S];
     } else {
         a.uprefix = (lines ? pl.d_uprefix1 : pl.d_cprefix1) + 2 * (size_t)s;
         a.n_units = (lines ? pl.uprefix1 : pl.cprefix1)[2 * (size_t)s + 1];
+        a.mprefix = pl.d_mprefix1 + 2 * (size_t)s;
+        a.n_merge = pl.mprefix1[2 * (size_t)s + 1];
     }
     a.line_ctas = c->line_ctas;
     return a;
@@ -600,10 +624,10 @@ int ensure_line_bufs(rqa_ctx *c, const Plan &pl)
     // lines at row-chunk boundaries: a slot per unit and band of one launch
     int64_t slots = 0;
     if (c->schedule != RQA_SCHED_PER_SERIES) {
-        if (pl.lsplit.rc < pl.ne_max) slots = pl.uprefix[pl.S] * pl.lsplit.nb;
+        if (pl.mprefix[pl.S] > 0) slots = pl.uprefix[pl.S] * pl.lsplit.nb;
     } else {
         for (int s = 0; s < pl.S; ++s)
-            if (pl.lsplit1[s].rc < pl.sd[s].ne)
+            if (pl.mprefix1[2 * (size_t)s + 1] > 0)
                 slots = std::max(slots, pl.uprefix1[2 * (size_t)s + 1] * pl.lsplit1[s].nb);
     }
     if ((rc = ensure(c->edges, (size_t)slots * LINE_EDGE_BYTES))) return rc;
@@ -651,10 +675,10 @@ int run_lines(rqa_ctx *c, const Plan &pl, const float *eps, uint64_t *hist, cons
     if (c->schedule == RQA_SCHED_PER_SERIES) {
         if ((rc = reset_queue(c, S * ng, &q))) return rc;
         for (int s = 0; s < S && rc == RQA_OK; ++s)
-            rc = launch_groups(cell_args(c, pl, s, true), pl.lsplit1[s].rc < pl.sd[s].ne);
+            rc = launch_groups(cell_args(c, pl, s, true), pl.mprefix1[2 * (size_t)s + 1] > 0);
     } else {
         if ((rc = reset_queue(c, ng, &q))) return rc;
-        rc = launch_groups(cell_args(c, pl, -1, true), pl.lsplit.rc < pl.ne_max);
+        rc = launch_groups(cell_args(c, pl, -1, true), pl.mprefix[S] > 0);
     }
     lb.k0 = 0;  // the finalisation kernels read all K targets
     return rc;

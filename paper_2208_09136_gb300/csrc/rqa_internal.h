@@ -73,6 +73,8 @@ struct CellArgs {
     int32_t n_pos;
     int32_t m_max;           // largest embedding dimension of the batch
     int32_t nb, rc;          // bands per unit and rows per unit (a multiple of the kernel's row block)
+    const int64_t *mprefix;  // line pass: n_pos + 1 prefix of the bands cut into several row chunks ...
+    int64_t n_merge;         // ... and their number
     int32_t line_ctas;       // persistent CTAs of the line pass per SM (0: as many as fit)
     int64_t n_units;
     unsigned int *queue;   // ticket counter (64-bit aligned), zeroed before launch
@@ -106,6 +108,9 @@ Split split_lines(uint64_t cells, int64_t bands, int32_t ne_max, int unit_bands,
 // Units of a series of ne vectors with bands of w diagonals (vert: the vertical
 // pass, every column over every row).
 int64_t units_of_series(int64_t ne, const Split &sp, bool vert, int w = DB);
+// Bands of LINE_BAND diagonals (columns) of a series that are longer than a row
+// chunk: the lower ones, and all or none in the vertical pass.
+int64_t cut_bands(int64_t ne, const Split &sp, bool vert);
 
 // Kernels (launch wrappers return cudaGetLastError()).
 cudaError_t launch_check_finite(const float *y, int64_t n, int *status, cudaStream_t st);
