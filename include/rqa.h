@@ -172,9 +172,9 @@ typedef struct {
     int tile;       /* 0, 8, 16 or 32; kept and reported (0 as 16), without effect */
     int unit_bands; /* bands of 32 diagonals per work unit a warp takes from the
                        queue (0 = planned from the batch: about eight units per
-                       resident warp, or one band over a chunk of its rows when
-                       the batch has fewer bands; 1..64 otherwise; capped so a
-                       unit stays under 2^33 cells) */
+                       resident warp, or one band, or one over a chunk of its
+                       rows, when the batch has fewer; 1..64 otherwise; capped
+                       so a unit stays under 2^33 cells) */
     int line_ctas;  /* persistent CTAs of the line pass per SM (0 = as many as
                        fit, else 1..8) */
     int stage;      /* 0 or 1; kept and reported, without effect */

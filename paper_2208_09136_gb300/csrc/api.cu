@@ -36,8 +36,9 @@ Split split_lines(uint64_t cells, int64_t bands, int32_t ne_max, int unit_bands,
         sp.rc = whole;
     } else {
         sp.nb = 1;
-        const uint64_t blocks = cells / ((uint64_t)LINE_BAND * 32 * (uint64_t)warps * 2);
-        sp.rc = (int)std::min<uint64_t>(32 * std::max<uint64_t>(blocks, 8), (uint64_t)std::min(whole, LINE_CHUNK_MAX));
+        const uint64_t blocks = cells / ((uint64_t)LINE_BAND * 32 * (uint64_t)warps * 2);  // half a warp's share
+        if (whole <= 32 * 32 && (uint64_t)whole <= 4 * 32 * blocks) sp.rc = whole;
+        else sp.rc = (int)std::min<uint64_t>(32 * std::max<uint64_t>(blocks, 8), (uint64_t)std::min(whole, LINE_CHUNK_MAX));
     }
     if (unit_bands > 0) sp.nb = unit_bands;  // a tuned size
     sp.nb = (int)std::min<int64_t>(sp.nb, cap);

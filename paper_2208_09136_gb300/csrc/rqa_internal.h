@@ -97,13 +97,17 @@ constexpr int COUNT_NB = 8;  // bands per unit of the counting rounds: one per w
 Split split_cells(uint64_t cells, int nb, int sm_count);
 // Units of the line pass over series with these cells and bands of LINE_BAND
 // diagonals, one warp each: runs of whole bands, about eight units per resident
-// warp (16 per SM), so the tail stays short while each unit's histogram flush is
-// spread over many cells; below that, single bands cut into row chunks for
-// about two units per warp (four: 876 us instead of 805 for lorenz-n1e4, 391
-// instead of 346 for three series of 7001), of at least 256 rows (a chunk's edges
-// and its first window cost about three blocks).  A unit covers at most 2^33 cells,
-// so the warp's 32-bit counts of lines of length >= 4 (each line and the cell
-// after it: >= 5 cells) stay exact.
+// warp (16 per SM), so the tail stays short; below that single bands.  These are
+// cut into row chunks for about two units per warp (four: 876 us instead of 805
+// for lorenz-n1e4, 391 instead of 346 for three series of 7001), of at least 256
+// rows (a chunk's edges and its first window cost about three blocks of 32 rows),
+// unless the longest band has at most 32 blocks and at most twice a warp's share of
+// all of them: short chunks then cost more than the tail (line pass of a call, whole
+// and in chunks: 300 series of 500, 135 and 167 us; 100 of 1000, 162 and 199).
+// Longer bands gain from chunks (vertical pass of 30 of 2000: 421 whole, 402), and
+// so do short ones that are few (30 of 1000: 137 and 103).  A unit covers at most
+// 2^33 cells, so the warp's 32-bit counts of lines of length >= 4 (each line and
+// the cell after it: >= 5 cells) stay exact.
 Split split_lines(uint64_t cells, int64_t bands, int32_t ne_max, int unit_bands, int sm_count);
 // Units of a series of ne vectors with bands of w diagonals (vert: the vertical
 // pass, every column over every row).

@@ -68,3 +68,11 @@ def test_batch_of_unlike_lengths_vertical(rqa_lib):
 def test_tuned_units_of_cut_bands(rqa_lib, unit_bands, schedule):
     ys = [_wave(n, n) for n in (1800, 290, 33, 700)]
     _check(rqa_lib, ys, 3, 1, RR20, tuning={"unit_bands": unit_bands, "line_ctas": 2}, schedule=schedule)
+
+
+# Batches whose longest band has at most 32 blocks of 32 rows and no more than
+# twice a warp's share stay whole: 130 series of 1024 (m = 1) do, of 1025 not
+@pytest.mark.parametrize("n,copies", [(1024, 65), (1025, 65), (600, 30), (600, 100)])
+def test_whole_and_cut_bands(rqa_lib, n, copies):
+    a, b = _wave(n, 1), _wave(n, 2)
+    _check(rqa_lib, [a, b] * copies, 1, 1, [4, 11, 35])
