@@ -639,7 +639,7 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                         // rows that the lane's diagonal (column) does not have, and
                         // the identity cell of a column unless it counts
                         const int col = c_lo + lane;
-                        const int lim = VERT ? (col < sd.ne ? sd.ne - i0 : 0) : sd.ne - d_lo - lane - i0;
+                        const int lim = VERT ? (col < rows ? rows - i0 : 0) : rows - lane - i0;
                         uint32_t out = lim >= 32 ? 0u : FULL << max(lim, 0);
                         if (VERT && !lb.loi && (uint32_t)(col - i0) < 32u) out |= 1u << (col - i0);
 #pragma unroll
@@ -719,14 +719,19 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                 for (; i0 < r_end; i0 += 32) {
                     // interior row blocks: every cell inside the matrix (and off the
                     // identity line)
-                    const bool inside = VERT ? c_lo + LD <= sd.ne && i0 + 32 <= rows &&
-                                                   (lb.loi || i0 + 32 <= c_lo || i0 >= c_lo + LD)
-                                             : i0 + 32 <= rows - (LD - 1);
+                    // (full sweeps decide before the walk, the others after it, by the
+                    // registers that ptxas finds: K = 13, m = tau = 3 6 % less so)
+                    auto inside = [&]() -> bool {
+                        return VERT ? c_lo + LD <= sd.ne && i0 + 32 <= rows &&
+                                          (lb.loi || i0 + 32 <= c_lo || i0 >= c_lo + LD)
+                                    : i0 + 32 <= rows - (LD - 1);
+                    };
                     uint32_t R[8];
+                    const bool early = FK && !inside();
                     if constexpr (WALK) {
                         walk(i0, R);
                     } else {
-                        if (inside) cell_phase(i0, std::true_type{});
+                        if (inside()) cell_phase(i0, std::true_type{});
                         else cell_phase(i0, std::false_type{});
                         __syncwarp();
                         const uint4 ra = *reinterpret_cast<const uint4 *>(rkm + lane * 32);
@@ -734,7 +739,7 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
                         R[0] = ra.x; R[1] = ra.y; R[2] = ra.z; R[3] = ra.w;
                         R[4] = rb.x; R[5] = rb.y; R[6] = rb.z; R[7] = rb.w;
                     }
-                    run_phase(i0, R, WALK && !inside);
+                    run_phase(i0, R, WALK && (FK ? early : !inside()));
                     if (++nrb == SETTLE) settle();
                 }
                 // lines that reach the end of a diagonal, or of the chunk, exactly at
