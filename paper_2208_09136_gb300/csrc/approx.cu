@@ -66,7 +66,7 @@ k_count_grid(CellArgs a, const float *__restrict__ thr, int n_thr, uint64_t *his
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ Unit unit;
-    __shared__ int next_band;
+    __shared__ int next_part, unit_rows;
     __shared__ uint32_t sink[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t *win = reinterpret_cast<uint32_t *>(smem) + warp * Src::WORDS;
@@ -95,7 +95,8 @@ k_count_grid(CellArgs a, const float *__restrict__ thr, int n_thr, uint64_t *his
             const unsigned t = atomicAdd(a.queue, 1u);
             if ((int64_t)t < a.n_units) {
                 unit = unit_of<false>(a, (int64_t)t);
-                next_band = unit.b_lo;
+                next_part = 0;
+                unit_rows = part_rows(unit, GT / 32);
             } else {
                 unit.s = -1;
             }
@@ -122,13 +123,8 @@ k_count_grid(CellArgs a, const float *__restrict__ thr, int n_thr, uint64_t *his
         Src src;
         src.init(a.y + sd.off, sd, lane, win);
         auto bands = [&](auto &&f) {
-            for (;;) {
-                int b = 0;
-                if (lane == 0) b = atomicAdd(&next_band, 1);
-                b = __shfl_sync(FULL, b, 0);
-                if (b >= w.b_hi) break;
-                walk_keys(src, sd.ne, 1 + b * DB, w.r_lo, w.r_hi, lane, f);
-            }
+            each_part(unit, unit_rows, &next_part, lane,
+                      [&](int d0, int r_lo, int r_hi) { walk_keys(src, sd.ne, d0, r_lo, r_hi, lane, f); });
         };
         auto count = [&](auto &&bin) {  // bin(key): r + 1
             bands([&](const float (&d)[4][DPL], auto valid) {

@@ -64,6 +64,33 @@ __device__ __forceinline__ Unit unit_of(const CellArgs &a, int64_t u)
     return w;
 }
 
+// How the warps of a CTA share a unit: one band at a time, so that no warp
+// idles while another still has several left; a unit of fewer bands than warps
+// is cut further, into parts of part_rows(w, warps) rows (a multiple of RB).
+// Short series have fewer bands: @@
+__device__ __forceinline__ int part_rows(const Unit &w, int warps)
+{
+    const int nb = w.b_hi - w.b_lo, blocks = (w.r_hi - w.r_lo + RB - 1) / RB;
+    if (nb >= warps) return blocks * RB;
+    const int parts = min((warps + nb - 1) / nb, blocks);
+    return (blocks + parts - 1) / parts * RB;
+}
+// f(first diagonal, first row, end row) for every part that this warp takes.
+// All arguments lie in shared memory and are read again for each part, which
+// costs less than their registers; next: the unit's counter, 0 at its start.
+template <class F>
+__device__ __forceinline__ void each_part(const Unit &w, const int &rows, int *next, int lane, F &&f)
+{
+    for (;;) {
+        int i = 0;
+        if (lane == 0) i = atomicAdd(next, 1);
+        i = __shfl_sync(FULL, i, 0);
+        const int nb = w.b_hi - w.b_lo, part = i < nb ? 0 : i / nb, r = w.r_lo + part * rows;
+        if (r >= w.r_hi) break;
+        f(1 + (w.b_lo + i - part * nb) * DB, r, min(r + rows, w.r_hi));
+    }
+}
+
 // Distances of the compile-time embedding (M, TAU): the ring e[] holds the
 // coordinate differences of the last (M-1) TAU rows of each diagonal.  Eight
 // rows long, so that two steps of four rows bring it back to the same

@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(CT, 2) k_count(CellArgs a, SelBufs sb, int K, 
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ Unit unit;
-    __shared__ int next_band;
+    __shared__ int next_part, unit_rows;
     __shared__ uint32_t sink[32];  // lane x's reductions of cells that count nowhere (never read)
     __shared__ uint32_t pfx[KMAX + 1];  // final round: the distinct target prefixes, ascending
     __shared__ int n_pfx;
@@ -169,7 +169,8 @@ __global__ void __launch_bounds__(CT, 2) k_count(CellArgs a, SelBufs sb, int K, 
             const unsigned t = atomicAdd(a.queue, 1u);
             if ((int64_t)t < a.n_units) {
                 unit = unit_of<false>(a, (int64_t)t);
-                next_band = unit.b_lo;
+                next_part = 0;
+                unit_rows = part_rows(unit, CW);
             } else {
                 unit.s = -1;
             }
@@ -247,15 +248,8 @@ __global__ void __launch_bounds__(CT, 2) k_count(CellArgs a, SelBufs sb, int K, 
         Src src;
         src.init(a.y + sd.off, sd, lane, win);
         auto bands = [&](auto &&f) {
-            for (;;) {
-                // bands are handed to warps one at a time, so no warp idles
-                // while another still has several bands of the unit left
-                int b = 0;
-                if (lane == 0) b = atomicAdd(&next_band, 1);
-                b = __shfl_sync(FULL, b, 0);
-                if (b >= w.b_hi) break;
-                walk_keys(src, sd.ne, 1 + b * DB, w.r_lo, w.r_hi, lane, f);
-            }
+            each_part(unit, unit_rows, &next_part, lane,
+                      [&](int d0, int r_lo, int r_hi) { walk_keys(src, sd.ne, d0, r_lo, r_hi, lane, f); });
         };
         // f(key, ok) for the sixteen cells of a step, one after the other
         auto each = [&](auto &&f) {
