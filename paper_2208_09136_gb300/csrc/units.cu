@@ -34,7 +34,7 @@ Split split_lines(uint64_t cells, int64_t bands, int32_t ne_max, int unit_bands,
         else sp.rc = (int)std::min<uint64_t>(32 * std::max<uint64_t>(blocks, 8), (uint64_t)std::min(whole, LINE_CHUNK_MAX));
     }
     if (unit_bands > 0) sp.nb = unit_bands;  // a tuned size
-    sp.nb = (int)std::min<int64_t>(sp.nb, cap);
+    sp.nb = (int)std::min({(int64_t)sp.nb, cap, (int64_t)whole / LINE_BAND});  // edge scratch is sized by nb
     return sp;
 }
 

@@ -55,3 +55,14 @@ def test_units_of_the_counting_rounds(split, series, ne):
     assert nb * 128 * rc < 2**32
     if series == 1 or ne < 1 << 20:
         assert rc <= 585 * 28  # as before for batches that fitted
+
+
+# row chunks keep 2560 bytes for every band a unit may have: no more bands than
+# the longest series has, whatever the tuned size
+@pytest.mark.parametrize("unit_bands", [0, 1, 64])
+def test_edge_scratch_of_the_line_pass(split, unit_bands):
+    nb, rc, units, edges = split("lines", 1, 300, 19000, 33, unit_bands)
+    assert rc < 300 and nb <= 10
+    assert edges < 1 << 29
+    nb, rc, units, edges = split("lines", 4, 10000, 0, 2, unit_bands)
+    assert nb == max(unit_bands, 1) and edges < 1 << 26
