@@ -81,21 +81,25 @@ inline cudaError_t allow_smem(Kern kern, int most)
 }
 
 // Host: CTAs of `kern` (THREADS threads, `smem` dynamic bytes) resident per
-// SM, and the SM count of the current device; both cached per host thread.
+// SM, and the SM count of the current device; both cached per host thread (the
+// last 64 sizes asked for, as a call's sizes vary with its targets and thresholds).
 inline int resident_per_sm(const void *kern, int smem, int threads = THREADS)
 {
-    struct Entry { const void *k; int s, v; };
+    struct Entry { const void *k; int dev, s, v; };
     static thread_local Entry cache[64];
-    static thread_local int n = 0;
-    for (int i = 0; i < n; ++i)
-        if (cache[i].k == kern && cache[i].s == smem) return cache[i].v;
+    static thread_local unsigned n = 0;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    for (unsigned i = 0; i < (n < 64 ? n : 64); ++i)
+        if (cache[i].k == kern && cache[i].s == smem && cache[i].dev == dev) return cache[i].v;
     int v = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, kern, threads, smem) != cudaSuccess) {
         cudaGetLastError();
         v = 1;
     }
     v = v < 1 ? 1 : v;
-    if (n < 64) cache[n++] = Entry{kern, smem, v};
+    cache[n % 64] = Entry{kern, dev, smem, v};
+    n = n + 1 < 128 ? n + 1 : 64;
     return v;
 }
 

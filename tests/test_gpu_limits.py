@@ -184,3 +184,19 @@ def test_network_on_millions_of_rows(rqa_lib):
     scale = chain(dY.abs(), W3.abs(), W2.abs(), x.double().abs())
     assert ((grads.double() - want).abs() <= 0.04 * scale).all()
     ctx.close()
+
+
+def test_many_sizes_in_one_thread(rqa_lib):
+    """More pairs of kernel and size than the launchers remember."""
+    rqa = rqa_lib
+    rng = np.random.default_rng(8)
+    y = rng.standard_normal(600).astype(np.float32)
+    ctx = rqa.Context(select=rqa.RQA_SELECT_RADIX)
+    batch = rqa.Batch.from_numpy([y], 3, 1)
+    for n_thr in list(range(1, 80)) + [40, 400]:
+        out = rqa.eps_approx(ctx, batch, [10, 50], 100, n_thr)
+        assert rqa.rqa_status(ctx) == 0
+        ref = O.eps_approx(y, 3, 1, [10, 50], 100, n_thr)
+        assert np.array_equal(out["eps"].cpu().numpy()[0], ref["eps"]), n_thr
+        assert np.array_equal(out["count"].cpu().numpy()[0], ref["count"]), n_thr
+    ctx.close()
