@@ -153,8 +153,12 @@ void mark(rqa_ctx *c, int i)
 {
     if (c->timing && c->schedule == RQA_SCHED_BATCHED) {
         // "external": inside a stream capture this becomes an event-record node
-        // of the graph, so replays record the phase boundaries too
-        cudaEventRecordWithFlags(c->ev[i], c->stream, cudaEventRecordExternal);
+        // of the graph, so replays record the phase boundaries too; the flag is
+        // an error outside one
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        cudaStreamIsCapturing(c->stream, &cs);
+        cudaEventRecordWithFlags(c->ev[i], c->stream,
+                                 cs == cudaStreamCaptureStatusActive ? cudaEventRecordExternal : cudaEventRecordDefault);
         if (i == 6) c->ev_recorded = true;
     }
 }

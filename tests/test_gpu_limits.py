@@ -200,3 +200,25 @@ def test_many_sizes_in_one_thread(rqa_lib):
         assert np.array_equal(out["eps"].cpu().numpy()[0], ref["eps"]), n_thr
         assert np.array_equal(out["count"].cpu().numpy()[0], ref["count"]), n_thr
     ctx.close()
+
+
+@pytest.mark.parametrize("own_stream", [False, True])
+def test_phase_times_without_a_graph(rqa_lib, own_stream):
+    """Timing of calls that are not recorded in a graph (thresholds or lines
+    alone, or any on the default stream)."""
+    import torch
+    rqa = rqa_lib
+    stream = torch.cuda.Stream() if own_stream else torch.cuda.default_stream()
+    with torch.cuda.stream(stream):
+        ctx = rqa.Context(select=rqa.RQA_SELECT_RADIX, stream=stream)
+        batch = rqa.Batch.from_numpy([_sine(3000)], 3, 1)
+        rqa.rqa_set_timing(ctx, True)
+        det = rqa.det_avg(ctx, batch, [5, 10], 100)
+        assert rqa.rqa_status(ctx) == 0
+        ms = rqa.rqa_phase_times(ctx)
+        assert (ms[1:5] > 0).all()
+        rqa.eps_for_rr(ctx, batch, [5, 10], 100)
+        rqa.line_hist(ctx, batch, det["eps"], 2)
+        assert rqa.rqa_status(ctx) == 0
+        assert rqa.rqa_phase_times(ctx)[4] > 0
+        ctx.close()
