@@ -69,7 +69,7 @@ enum {
     RQA_ERR_NONFINITE = 3,   /* device: a series holds NaN or +-Inf */
     RQA_ERR_CUDA = 4,        /* a CUDA runtime call failed (no device, launch) */
     RQA_ERR_OOM = 5,         /* scratch allocation failed */
-    RQA_ERR_TIMEOUT = 6,     /* device: a bounded wait gave up */
+    RQA_ERR_TIMEOUT = 6,     /* device: a bounded wait gave up (no kernel waits at present) */
     RQA_ERR_CAPACITY = 7,    /* output buffer too small / size limit exceeded */
     RQA_ERR_UNSORTED = 8,    /* device: thresholds of a series not ascending */
     RQA_ERR_NO_MODEL = 9,    /* bracket selection requested without a model */

@@ -52,10 +52,10 @@ struct rqa_ctx {
     cudaStream_t stream = nullptr;
     int schedule = RQA_SCHED_BATCHED;
     int select = RQA_SELECT_AUTO;
-    int line_tile = 0;      // rqa_tuning.tile and .stage as set: kept for callers that read them back,
+    int line_tile = 0;      // rqa_tuning.tile (and line_stage, its .stage) as set: only read back
     int unit_bands = 0;     // bands per line-pass work unit (0 = planned)
     int line_ctas = 0;      // persistent line-pass CTAs per SM (0 = all that fit)
-    int line_stage = 0;     // no effect
+    int line_stage = 0;
     float tuned_ms = 0.f;   // line-pass time of the last rqa_autotune choice
     bool loi = false;         // RQA_FLAG_LOI: rates and DET over the whole matrix
     int bpsm = 0;
@@ -414,14 +414,13 @@ SelBufs sel_bufs(rqa_ctx *c, const Plan &pl)
     return sb;
 }
 
-
-// Zero the queue tickets of n launches; returns the first ticket pointer.
 // Counting launches of one selection (per series in the per-series
 // schedule): bracket/coarse, middle rounds of MID_GROUPS groups, final.
 int select_launches(int K) { return 3 + (K + MID_GROUPS - 1) / MID_GROUPS; }
 // Line-pass launches: groups of at most LINE_KMAX targets.
 int line_groups(int K) { return (K + LINE_KMAX - 1) / LINE_KMAX; }
 
+// Zero the queue tickets of n launches; returns the first ticket pointer.
 int reset_queue(rqa_ctx *c, int n, unsigned **q)
 {
     if (int rc = ensure(c->queue, (size_t)n * 64)) return rc;

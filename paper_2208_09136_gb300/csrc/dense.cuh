@@ -254,11 +254,6 @@ struct GenSrc {
     __device__ __forceinline__ void leave() {}
 };
 
-// Walk rows [r_lo, r_hi) of the band at diagonal d0 and hand the distance keys
-// of every lane's four rows x four diagonals to f(key, valid): valid is a
-// compile-time true inside the triangle and a run-time mask (bit 4 r + j) in
-// blocks that reach over its edge.  f sees sixteen cells at once so that it
-// can issue their lookups together before it uses any.
 // Any embedding with at most MAXM coordinates: a window of rows and one of
 // columns per coordinate in shared memory, so that four rows of a lane's
 // sixteen cells take three 16-byte loads per coordinate, nine wavefronts.
@@ -361,6 +356,11 @@ struct MaskValid {
     uint32_t m;
     __device__ __forceinline__ bool operator()(int r, int j) const { return (m >> (4 * r + j)) & 1u; }
 };
+// Walk rows [r_lo, r_hi) of the band at diagonal d0 and hand the distances of
+// every lane's four rows x four diagonals to f(d[4][DPL], valid): valid(r, j) is
+// a compile-time true inside the triangle and a bit of a run-time mask in blocks
+// that reach over its edge.  f sees sixteen cells at once so that it can issue
+// their lookups together before it uses any.
 template <class Src, class F>
 __device__ __forceinline__ void walk_keys(Src &src, int ne, int d0, int r_lo, int r_hi, int lane, F &&f)
 {

@@ -12,8 +12,7 @@
 //         lane t holds row i0+t and stores r as a byte of row j of a
 //         32 x 32 rank matrix in shared memory, which lane j then reads.
 //         (m = 3, cycles per SM quarter and 32 cells of the whole pass, mixed
-//         signals: 56.7 by diagonals, 65.1 by rows; tau = 1: 76 and 85; four
-//         series of 2e4 of noise, tau = 2: m = 2, 4 by diagonals 79 and 97.)
+//         signals: 56.7 by diagonals, 65.1 by rows; tau = 1: 76 and 85.)
 //  runs   lane j holds diagonal j.  It gathers the five bit planes of its ranks:
 //         two words of four ranks are interleaved bit by bit, so one mask and
 //         one multiply bring bit p of eight ranks into the top byte of a
@@ -36,21 +35,21 @@
 //
 // Outputs per (series, threshold): P_k(l) (lengths 1..3 from packed register
 // tallies, less the lines measured one by one for length 3; 4..WSH in the
-// warp's shared histogram; both flushed once per work
-// unit; WSH+1..LSH in the series' global short histogram; longer lines to the
-// caller's full histogram), L_max, and C_k = sum of l P_k(l), the recurrent
-// cells.
+// warp's shared histogram; both flushed when the warp goes on to another series
+// or at 2^33 cells; WSH+1..LSH in the series' global short histogram; longer lines
+// to the caller's full histogram), L_max, and C_k = sum of l P_k(l), the
+// recurrent cells.
 //
 // A batch with too few bands to fill the chip is cut into row chunks
 // (CellArgs::rc).  A chunk counts its rows as if the matrix ended at them and
 // keeps, per diagonal and threshold, the lengths of the lines that touch its
-// first and its last row (Edges); k_merge (lines.cu) then joins the lines that
+// first and its last row (edges); k_merge (lines.cu) then joins the lines that
 // meet at a chunk boundary.  The four 10^4-value series of lorenz-n1e4 have
 // 1252 bands for 2432 resident warps, each 10^4 rows long.
 //
 // The vertical pass (VERT) is the same kernel over bands of 32 consecutive
-// columns walked over every row of the matrix: the word of column c is the
-// ballot over 32 consecutive rows, so its runs are vertical lines.
+// columns walked over every row of the matrix: lane c's words are 32 rows of its
+// column, so their runs are vertical lines.
 #pragma once
 #include <cstdint>
 #include <type_traits>
@@ -144,9 +143,6 @@ __device__ __forceinline__ uint32_t rank_le_word_lane(uint32_t b0, uint32_t b1, 
     return lop3<0x8E>(b4, kbm[4], w);
 }
 
-// Warp-centric: every warp pulls units from one global queue and keeps its
-// own histogram in shared memory, flushed after each unit.  No CTA-wide
-// barrier, so no warp waits for another.
 // Transpose a 32 x 32 bit matrix held one row per lane: on return lane k
 // holds column k (bit j of the result = bit k of lane j's word).  Five rounds
 // of exchanging off-diagonal blocks with the lane s apart.
@@ -173,6 +169,9 @@ __device__ __forceinline__ uint32_t threshold_key(float eps)
 }
 __device__ __forceinline__ bool threshold_ok(uint32_t v) { return !(v & 0x80000000u) && v <= 0x7f800000u; }
 
+// Warp-centric: every warp pulls units from one global queue and keeps its
+// own histogram in shared memory, flushed when the series changes.  No CTA-wide
+// barrier, so no warp waits for another.
 // FK: a full sweep, K = KT thresholds known at compile time (the per-threshold
 // code then runs without a test of k against K); the argument is ignored.
 template <int M, int TAU, bool VERT, bool FK = false>
@@ -211,7 +210,7 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
     for (int l = 0; l < HROW; ++l) hs[l * 32] = 0;
 
     __syncwarp();
-    uint64_t lmass = 0;  // cells on lines of threshold kk longer than WSH (this unit, this lane)
+    uint64_t lmass = 0;  // cells on lines of threshold kk longer than WSH (since the last flush, this lane)
     uint32_t lmx = 0;    // the longest of them
 
     int cur = -1;
@@ -773,7 +772,6 @@ __global__ void __launch_bounds__(LTHREADS, 8) k_lines(CellArgs a, LineBufs lb, 
 namespace rqa {
 using LinesKernel = void (*)(CellArgs, LineBufs, int, uint16_t *);
 // Instantiations, one group per translation unit (they compile in parallel).
-// full: the diagonal pass's variant for a sweep of exactly LINE_KMAX thresholds
 // full: the diagonal pass's variant for a sweep of exactly LINE_KMAX thresholds
 LinesKernel lines_kernel_m3t3(bool vert, bool full);
 LinesKernel lines_kernel_m3t1(bool vert, bool full);
